@@ -266,13 +266,12 @@ class Evictor:
 # Slots of the per-CTA time accounting of a JACAP_TRACE build (jacap_ws_offsets.trace_cta):
 # kernel index -> (name, {slot: meaning}); "tiles" counts tiles, every other slot sums ns.
 TRACE_CTA_SLOTS = {
-    2: ("k_pass", {0: "producer: wait for a free stage", 1: "producer: loop", 2: "logits MMA: wait for an image",
-                   3: "logits MMA: wait for a K tile and a free buffer", 5: "logits MMA: loop", 6: "tiles",
-                   7: "kappa warp: wait for a K tile", 8: "kappa warp: its quarter of kappa",
-                   9: "kappa warp: wait for the group's slot", 10: "kappa warp: partials into the slot",
-                   11: "kappa warp: loop", 12: "readout warp: wait for logits",
-                   13: "readout warp: readout of a tile", 14: "readout warp: loop",
-                   15: "readout warp: wait for the kappa partials"}),
+    2: ("k_pass", {0: "producer: wait for a free stage", 1: "producer: loop", 2: "MMA: wait for the images",
+                   3: "MMA: wait for a tile's operands and a free accumulator", 5: "MMA: loop", 6: "tiles",
+                   7: "convert warp: wait for a K tile", 8: "convert warp: wait for a free operand buffer",
+                   9: "convert warp: stores into tensor memory", 11: "convert warp: loop",
+                   12: "readout warp: wait for an accumulator", 13: "readout warp: readout of a tile",
+                   14: "readout warp: loop"}),
     0: ("gram", {0: "producer: wait for a free stage", 1: "producer: loop", 2: "MMA: wait for a scaled operand",
                  3: "MMA: wait for a free accumulator", 4: "MMA: loop", 5: "tiles", 6: "scaling warp: wait for V",
                  7: "scaling warp: wait for the weights", 8: "scaling warp: wait for a free operand buffer",

@@ -6,27 +6,35 @@
 // plus an online (max, sum exp(l - max)) per work item and head, which the
 // weight pass combines into the softmax normaliser.
 //
-// The logits are a 128 x 128 x N contraction per 128-token tile and run on the
-// tensor cores: A = the TMA-staged K tile (shared memory, K-major), B = mu' =
-// mu / (tau sqrt d) split exactly into three bf16 parts (hi + mid + lo carries
-// ~24 significant bits) for the G heads, fp32 accumulation in tensor memory.
-// kappa needs the elementwise squares of k, which would double the tensor
-// instructions (k^2 has 16 significant bits: two bf16 operands) at a fixed
-// cost per instruction, so it runs on the CUDA cores instead: k^2 is exact in
-// fp32 and is weighted by lambda (fp32, broadcast from shared memory) with
-// packed fp32x2 multiply-adds.
+// Both are 128 x 128 x N contractions per 128-token tile and run on the tensor
+// cores. The logits take the TMA-staged K tile as A and B = mu' = mu / (tau sqrt
+// d); kappa takes the tile's squares, k^2 = hi + lo with hi = RN_bf16(k^2) and lo
+// = k^2 - hi (exact: a bf16 square has 16 significant bits; one packed multiply
+// and one packed fused multiply-add give both), which the convert warps write
+// into tensor memory as two A operands (lane = token, two channels per column),
+// and B = lambda. mu' and lambda are split exactly into three bf16 parts (hi +
+// mid + lo carries ~24 significant bits) for the G heads, so the products are
+// those of float32 operands. The MMAs' fp32 sums truncate: kappa's channels go
+// into KG groups of columns (four of 32 channels, two of 64 for G > 5) that the
+// readout adds, which keeps the scores as close to float64 as the float32
+// multiply-adds did (rel. 6.6e-7 either way at G = 4, n = 32768; one group for
+// all channels: 7.7e-7).
 //
-// Warp roles: 0 TMA producer; 1 issues the logits MMAs; 14 builds the mu'
-// image and lambda of each unit a CTA reaches (double-buffered, one run of the
-// unit's consecutive items ahead); 2-9 kappa (two groups of four warps alternate
-// tiles; in a group each warp takes one quarter of the channels for all 128
-// tokens, four per lane, so every lambda value read from shared memory serves
-// four tokens, and writes its partial sums of all four token subsets into the
-// group's slot); 10-13 read the logits back from tensor memory (one lane
-// quarter each), add the four partial kappa of their 32 tokens from the slot,
-// keep the online softmax statistics and store each token's row (logits,
-// kappa) in one piece. Each group has two slots (one for G > 4), handed over
-// with mbarriers, so a group writes one while the readout warps read the other.
+// Why this way: issued under elect.sync, an M = 128, N = 16 MMA costs 9 cycles
+// with A in tensor memory and 39 with A in shared memory (45 either way under a
+// lane test), so a tile's 24 MMAs take ~460 of the ~1500 cycles in which its 32
+// KB arrive at the copy rate. On the CUDA cores kappa took 1.2 us per tile and
+// group of four warps at G = 4, and grew with G. Measured, both kinds, K pass
+// alone (events): 32 layers x 8 KV heads x 32768 tokens, G = 4: 0.403 -> 0.385
+// ms; 40 x 8 x 9001, G = 5: 0.202 -> 0.147 ms; 28 x 4 x 20011, G = 7: 0.209 ->
+// 0.136 ms. What bounds it now is HBM (6.3 TB/s of K and rows at G = 4).
+//
+// Warp roles: 0 TMA producer; 1 issues the MMAs; 2 builds the mu' and lambda
+// images of each unit a CTA reaches (double-buffered, one run of the unit's
+// consecutive items ahead); 3-10 convert (two warps per tensor-memory lane
+// quarter, each 32 tokens x 64 channels); 11-14 read the accumulators back (one
+// lane quarter each), keep the online softmax statistics and store each token's
+// row (logits, kappa) in one piece.
 #include "jacap_dev.cuh"
 #include "jacap_internal.h"
 
@@ -34,120 +42,73 @@ namespace jacap {
 
 constexpr int KB_BOX = 16384;    // {64 channels, 128 tokens} bf16
 constexpr int KB_TILE_BYTES = 2 * KB_BOX;
-constexpr int KB_NACC = 4;       // tensor-memory logits buffers
-constexpr uint32_t KB_TMEM_COLS = 128;
 constexpr int KB_THREADS = 480;
-constexpr int KB_KAPPA_WARP0 = 2, KB_READ_WARP0 = 10, KB_BUILD_WARP = 14;
+constexpr int KB_BUILD_WARP = 2, KB_CONV_WARP0 = 3, KB_CONV_WARPS = 8, KB_READ_WARP0 = 11;
+constexpr uint32_t KB_TMEM_COLS = 512;
+constexpr uint32_t KB_ACC_COLS = 256;  // columns [0, 256): accumulators
+constexpr uint32_t KB_A_COLS = 128;    // an A buffer: hi(k^2) [0, 64), lo(k^2) [64, 128)
+static_assert(KB_ACC_COLS + 2 * KB_A_COLS <= KB_TMEM_COLS, "tensor memory budget");
 
 template <int G>
 struct KbCfg {
-  static constexpr int NB = (3 * G <= 16) ? 16 : 32;  // MMA N = rows of the mu' image
+  static constexpr int NB = (3 * G <= 16) ? 16 : 32;  // MMA N = rows of an image
+  static constexpr int KG = NB == 16 ? 4 : 2;          // kappa's channel groups, each with columns of its own
+  static constexpr int ACC = (1 + KG) * NB;            // columns of an accumulator slot: logits, then the groups
+  static constexpr int NACC = KB_ACC_COLS / ACC;
   static constexpr int IMG_ATOM = NB * 128;            // bytes per 64-channel atom
-  static constexpr int IMG_BYTES = 2 * IMG_ATOM;
-  static constexpr int LAM_BYTES = G * D * 4;          // lambda, fp32 [G][128]
-  // partial-kappa slots per group: two (the group writes one while the readout
-  // warps read the other) when they fit beside five K stages, else one
-  static constexpr int SLOTS = G <= 4 ? 2 : 1;
-  static constexpr int SLOT_FLOATS = 4 * 4 * G * 32;                 // [token subset][writer][G][32]
-  static constexpr int KRED_FLOATS = 2 * SLOTS * SLOT_FLOATS;        // [group][slot]
+  static constexpr int IMG_BYTES = 2 * IMG_ATOM;       // one image; a run has two (mu', lambda)
   static constexpr uint32_t IDESC = idesc_bf16_f32(128, NB, 0, 0);
-  static_assert(KB_NACC * NB <= (int)KB_TMEM_COLS, "tensor memory budget");
   static constexpr size_t smem_for(int stages) {
-    return 1024 + (size_t)stages * KB_TILE_BYTES + 2 * IMG_BYTES + 2 * LAM_BYTES + KRED_FLOATS * 4 + 4 * 2 * G * 4 +
-           512;
+    return 1024 + (size_t)stages * KB_TILE_BYTES + 4 * IMG_BYTES + TILE * 2 * G * 4 + 4 * 2 * G * 4 + 256;
   }
-  static constexpr int STAGES = smem_for(6) <= 232448 ? 6 : (smem_for(5) <= 232448 ? 5 : 4);  // K tiles in flight
+  static constexpr int STAGES = smem_for(6) <= 232448 ? 6 : 5;  // K tiles in flight
   static constexpr size_t SMEM = smem_for(STAGES);
 };
 
-// The K tile `it` lands on barrier full[kb_full(it)], one per (tile parity,
-// stage). A kappa group takes every other tile, so with an odd number of
-// stages it sees only every other use of a stage; on a barrier per stage its
-// parity wait could not tell "my tile landed" from "the other group's tile in
-// this stage has not landed yet". Per (parity, stage) every waiter sees
-// consecutive phases: the tile's use of its barrier is it / kb_full_period.
-template <int STAGES>
-__device__ __forceinline__ int kb_full(uint32_t it) { return (int)(it & 1) * STAGES + (int)(it % STAGES); }
-template <int STAGES>
-__device__ __forceinline__ uint32_t kb_full_parity(uint32_t it) {
-  return (it / (STAGES % 2 == 0 ? STAGES : 2 * STAGES)) & 1;
-}
-
-// mu' image of one item: rows n = part * G + h hold part (0 hi, 1 mid, 2 lo) of
-// src[h][0..127], K-major with the 128-byte swizzle (two 64-channel atoms).
+// The images of one run: row n = part G + h of an image holds part (0 hi, 1 mid,
+// 2 lo) of mu'_h (image 0) or lambda_h (image 1), K-major with the 128-byte
+// swizzle (two 64-channel atoms). Each lane takes 8 channels of a head at a
+// time: one read of the values gives all three parts (rows 3 G .. NB - 1 stay
+// zero).
 template <int G>
-__device__ __forceinline__ void build_split_image(uint8_t* im, const float* src, int lane) {
+__device__ __forceinline__ void build_split_images(uint8_t* im, const float* mu, const float* lam, int lane) {
   using C = KbCfg<G>;
-  for (int e = lane; e < C::NB * 16; e += 32) {
-    const int n = e >> 4, cc = e & 15;
-    uint32_t wv[4] = {0u, 0u, 0u, 0u};
-    if (n < 3 * G) {
-      const int part = n / G, h = n % G;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float x[2];
-#pragma unroll
-        for (int z = 0; z < 2; ++z) {
-          const float v = src[h * D + cc * 8 + 2 * q + z];
-          const float hi = __bfloat162float(__float2bfloat16_rn(v));
-          const float r1 = v - hi;
-          const float mid = __bfloat162float(__float2bfloat16_rn(r1));
-          x[z] = part == 0 ? hi : (part == 1 ? mid : r1 - mid);
-        }
-        wv[q] = pack_bf16x2(x[0], x[1]);
-      }
-    }
-    *(uint4*)(im + (cc >> 3) * C::IMG_ATOM + sw128_off(n, cc & 7)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-  }
-}
-
-// Partial kappa over channel quarter `cq` (chunks 4 cq .. 4 cq + 3 of 8
-// channels) for the four token rows lane + 32 j of a staged tile:
-// part[j][h] = sum_c lambda_h,c k_c^2. Each lambda load feeds JB tokens: all
-// four for G = 1, 2, 4; for other groups two passes over the quarter take two
-// tokens each, which halves the accumulators held at once (and keeps them in
-// registers).
-template <int G>
-__device__ __forceinline__ void kappa_quarter(uint32_t kt, uint32_t lam, int lane, int cq, float (&part)[4][G]) {
-  constexpr int JB = (G <= 2 || G == 4) ? 4 : 2;
-#pragma unroll
-  for (int j0 = 0; j0 < 4; j0 += JB) {
-    float2 acc[JB][G];
-#pragma unroll
-    for (int j = 0; j < JB; ++j)
-#pragma unroll
-      for (int h = 0; h < G; ++h) acc[j][h] = make_float2(0.f, 0.f);
+  constexpr int NB2 = G <= 2 ? 1 : 2;  // values of this many turns are loaded together
 #pragma unroll 1
-    for (int cc = 4 * cq; cc < 4 * cq + 4; ++cc) {
-      float4 l0[G], l1[G];
+  for (int e0 = lane; e0 < G * 16; e0 += 32 * NB2) {
+    float4 v[NB2][4];
 #pragma unroll
-      for (int h = 0; h < G; ++h) {
-        l0[h] = lds_f128(lam + (h * D + 8 * cc) * 4);
-        l1[h] = lds_f128(lam + (h * D + 8 * cc + 4) * 4);
-      }
-#pragma unroll
-      for (int j = 0; j < JB; ++j) {
-        const uint4 r = lds_u128(kt + (cc >> 3) * KB_BOX + sw128_off(lane + 32 * (j0 + j), cc & 7));
-        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-        float2 sq[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float2 x = make_float2(bf16lo(w[q]), bf16hi(w[q]));
-          sq[q] = __fmul2_rn(x, x);  // exact: 8-bit significands
-        }
-#pragma unroll
-        for (int h = 0; h < G; ++h) {
-          acc[j][h] = __ffma2_rn(sq[0], make_float2(l0[h].x, l0[h].y), acc[j][h]);
-          acc[j][h] = __ffma2_rn(sq[1], make_float2(l0[h].z, l0[h].w), acc[j][h]);
-          acc[j][h] = __ffma2_rn(sq[2], make_float2(l1[h].x, l1[h].y), acc[j][h]);
-          acc[j][h] = __ffma2_rn(sq[3], make_float2(l1[h].z, l1[h].w), acc[j][h]);
-        }
+    for (int i = 0; i < NB2; ++i) {
+      const int e = e0 + 32 * i;
+      if (e < G * 16) {
+        v[i][0] = *(const float4*)(mu + e * 8);
+        v[i][1] = *(const float4*)(mu + e * 8 + 4);
+        v[i][2] = *(const float4*)(lam + e * 8);
+        v[i][3] = *(const float4*)(lam + e * 8 + 4);
       }
     }
 #pragma unroll
-    for (int j = 0; j < JB; ++j)
+    for (int i = 0; i < NB2; ++i) {
+      const int e = e0 + 32 * i, h = e >> 4, cc = e & 15;
+      if (e >= G * 16) break;
 #pragma unroll
-      for (int h = 0; h < G; ++h) part[j0 + j][h] = acc[j][h].x + acc[j][h].y;
+      for (int m = 0; m < 2; ++m) {
+        const float4 p = v[i][2 * m], q = v[i][2 * m + 1];
+        const float x[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+        uint32_t w[3][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          w[0][j] = pack_bf16x2(x[2 * j], x[2 * j + 1]);
+          const float r0 = x[2 * j] - bf16lo(w[0][j]), r1 = x[2 * j + 1] - bf16hi(w[0][j]);
+          w[1][j] = pack_bf16x2(r0, r1);
+          w[2][j] = pack_bf16x2(r0 - bf16lo(w[1][j]), r1 - bf16hi(w[1][j]));
+        }
+#pragma unroll
+        for (int part = 0; part < 3; ++part)
+          *(uint4*)(im + m * C::IMG_BYTES + (cc >> 3) * C::IMG_ATOM + sw128_off(part * G + h, cc & 7)) =
+              make_uint4(w[part][0], w[part][1], w[part][2], w[part][3]);
+      }
+    }
   }
 }
 
@@ -156,22 +117,22 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
     kpass_bf16_kernel(const __grid_constant__ CUtensorMap kmap, Dims dm, Ws ws, const int32_t* __restrict__ cu) {
   pdl_wait();
   using C = KbCfg<G>;
+  constexpr int KB_STAGES = C::STAGES, NACC = C::NACC, NB = C::NB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  constexpr int KB_STAGES = C::STAGES;
   uint8_t* tiles = smem;
-  uint8_t* img = tiles + KB_STAGES * KB_TILE_BYTES;    // [parity][IMG_BYTES] mu' images
-  float* lams = (float*)(img + 2 * C::IMG_BYTES);       // [parity][G][128] lambda
-  float* kred = lams + 2 * G * D;                        // partial kappa of the upper channel half
-  float* red = kred + C::KRED_FLOATS;                    // [4 readout warps][2G]
-  uint64_t* full = (uint64_t*)(red + 4 * 2 * G);  // [tile parity][stage], see kb_full
-  uint64_t* empty = full + 2 * KB_STAGES;
-  uint64_t* accfull = empty + KB_STAGES;
-  uint64_t* accempty = accfull + KB_NACC;
-  uint64_t* imgready = accempty + KB_NACC;
-  uint64_t* imgfree = imgready + 2;
-  uint64_t* kready = imgfree + 2;            // [group][slot] a tile's partial kappa are in the slot
-  uint64_t* kfree = kready + 2 * C::SLOTS;   // [group][slot] the readout warps have read them
+  uint8_t* img = tiles + KB_STAGES * KB_TILE_BYTES;  // [parity][mu', lambda][IMG_BYTES]
+  float* rows = (float*)(img + 4 * C::IMG_BYTES);     // [TILE][2G] the tile's rows on their way out
+  float* red = rows + TILE * 2 * G;                   // [4 readout warps][2G]
+  uint64_t* full = (uint64_t*)(red + 4 * 2 * G);
+  uint64_t* empty = full + KB_STAGES;
+  uint64_t* afull = empty + KB_STAGES;   // [2] the tile's A operands are in tensor memory
+  uint64_t* aempty = afull + 2;          // [2] the MMAs have read them
+  uint64_t* accfull = aempty + 2;        // [NACC]
+  uint64_t* accempty = accfull + NACC;   // [NACC]
+  uint64_t* imgready = accempty + NACC;  // [2]
+  uint64_t* imgfree = imgready + 2;      // [2]
+  static_assert((2 * KB_STAGES + 4 + 2 * NACC + 4) * 8 <= 256, "barriers");
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort, s_skip;
 
@@ -181,24 +142,22 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
     s_skip = status_failed(ws) ? 1 : 0;
     for (int i = 0; i < KB_STAGES; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
-      mbar_init(smem_u32(&full[KB_STAGES + i]), 1);
-      mbar_init(smem_u32(&empty[i]), 5);  // MMA commit + the four kappa warps of the tile
+      mbar_init(smem_u32(&empty[i]), KB_CONV_WARPS + 1);  // and the MMAs' commit
     }
-    for (int i = 0; i < KB_NACC; ++i) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&afull[i]), KB_CONV_WARPS);
+      mbar_init(smem_u32(&aempty[i]), 1);
+      mbar_init(smem_u32(&imgready[i]), 1);
+      mbar_init(smem_u32(&imgfree[i]), 1);
+    }
+    for (int i = 0; i < NACC; ++i) {
       mbar_init(smem_u32(&accfull[i]), 1);
       mbar_init(smem_u32(&accempty[i]), 4);
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(&imgready[i]), 1);
-      mbar_init(smem_u32(&imgfree[i]), 9);  // MMA commit + the eight kappa warps
-
-    }
-    for (int i = 0; i < 2 * C::SLOTS; ++i) {
-      mbar_init(smem_u32(&kready[i]), 4);  // the group's four kappa warps
-      mbar_init(smem_u32(&kfree[i]), 4);   // the four readout warps
-    }
     fence_mbar_init();
   }
+  for (int e = tid; e < 4 * C::IMG_BYTES / 16; e += KB_THREADS) ((uint4*)img)[e] = make_uint4(0, 0, 0, 0);
+  fence_proxy_async_smem();
   __syncthreads();
   if (s_skip) return;
   if (warp == 1) {
@@ -233,7 +192,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
           }
           TRC_ADD(0, tr_w);
           uint8_t* kt = tiles + st * KB_TILE_BYTES;
-          const uint32_t fb = smem_u32(&full[kb_full<KB_STAGES>(it)]);
+          const uint32_t fb = smem_u32(&full[st]);
           mbar_arrive_expect_tx(fb, KB_TILE_BYTES);
           tma_load_4d(smem_u32(kt), &kmap, 0, (int)t, g, l, fb);
           tma_load_4d(smem_u32(kt + KB_BOX), &kmap, 64, (int)t, g, l, fb);
@@ -243,17 +202,17 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
       TRC_ADD(1, tr_all);
       TRC_PUT(ws, TR_K_KPASS, 2);
       for (uint32_t k = (it > (uint32_t)KB_STAGES ? it - KB_STAGES : 0); k < it; ++k)
-        mbar_wait(smem_u32(&full[kb_full<KB_STAGES>(k)]), kb_full_parity<KB_STAGES>(k), ws, nullptr);
+        mbar_wait(smem_u32(&full[k % KB_STAGES]), (k / KB_STAGES) & 1, ws, nullptr);
     }
   } else if (warp == 1) {
-    // ------------------------------------------------ logits MMA issuer ---
-    if (lane == 0) {
+    // ------------------------------------------------ MMA issuer ----------
+    if (elect_one()) {
       uint32_t it = 0, nrun = 0;  // nrun: runs of consecutive items of one unit started
       bool ok = true, cont = false;
       int p = 0;
       Item item;
-      // time accounting (trace builds): 2 waits for an image, 3 for a K tile and a free
-      // logits buffer, 5 the whole loop, 6 tiles
+      // time accounting (trace builds): 2 waits for an image, 3 for a tile's operands and a
+      // free accumulator, 5 the whole loop, 6 tiles
       TRC_DECL(TR_CTA_SLOTS);
       TRC_T(tr_all);
       for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); ok && is.next(item);) {
@@ -264,14 +223,15 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
           TRC_ADD(2, tr_i);
           tc_fence_after();
         }
-        const uint64_t b0 = smem_desc_sw128(smem_u32(img + p * C::IMG_BYTES), 16, 1024);
+        const uint64_t bmu = smem_desc_sw128(smem_u32(img + (2 * p) * C::IMG_BYTES), 16, 1024);
+        const uint64_t blam = smem_desc_sw128(smem_u32(img + (2 * p + 1) * C::IMG_BYTES), 16, 1024);
         for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
-          const int st = it % KB_STAGES;
-          const int ab = it % KB_NACC;
+          const int ab = it & 1, ac = it % NACC;
           TRC_T(tr_f);
-          if (!mbar_wait(smem_u32(&full[kb_full<KB_STAGES>(it)]), kb_full_parity<KB_STAGES>(it), ws, abort) ||
-              (it >= (uint32_t)KB_NACC &&
-               !mbar_wait(smem_u32(&accempty[ab]), ((it / KB_NACC) & 1) ^ 1, ws, abort))) {
+          const int st = it % KB_STAGES;
+          if (!mbar_wait(smem_u32(&full[st]), (it / KB_STAGES) & 1, ws, abort) ||
+              !mbar_wait(smem_u32(&afull[ab]), (it >> 1) & 1, ws, abort) ||
+              (it >= (uint32_t)NACC && !mbar_wait(smem_u32(&accempty[ac]), ((it / NACC) & 1) ^ 1, ws, abort))) {
             ok = false;
             break;
           }
@@ -279,16 +239,27 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
           TRC_INC(6);
           tc_fence_after();
           // descriptors advance by (byte offset >> 4) in their address field
+          const uint32_t a = tmem + KB_ACC_COLS + ab * KB_A_COLS;
           const uint64_t a0 = smem_desc_sw128(smem_u32(tiles + st * KB_TILE_BYTES), 16, 1024);
-          const uint32_t dl = tmem + ab * C::NB;
+          const uint32_t dl = tmem + ac * C::ACC;
+          constexpr int KS = D / 16 / C::KG;  // K-steps (16 channels) per group
 #pragma unroll
-          for (int k = 0; k < D / 16; ++k) {  // 16 channels per MMA
-            const uint64_t ad = a0 + (uint64_t)((((k >> 2) * KB_BOX) + (k & 3) * 32) >> 4);
-            const uint64_t bm = b0 + (uint64_t)((((k >> 2) * C::IMG_ATOM) + (k & 3) * 32) >> 4);
-            umma_f16_ss(dl, ad, bm, C::IDESC, k > 0 ? 1u : 0u);
+          for (int g = 0; g < C::KG; ++g) {
+#pragma unroll
+            for (int part = 0; part < 2; ++part)  // lo first: the sums stay small until the last steps
+#pragma unroll
+              for (int k = g * KS; k < (g + 1) * KS; ++k)
+                umma_f16_ts(dl + (1 + g) * NB, a + (part == 0 ? 64 : 0) + 8 * k,
+                            blam + (uint64_t)((((k >> 2) * C::IMG_ATOM) + (k & 3) * 32) >> 4), C::IDESC,
+                            part == 0 && k == g * KS ? 0u : 1u);
           }
+#pragma unroll
+          for (int k = 0; k < D / 16; ++k)
+            umma_f16_ss(dl, a0 + (uint64_t)((((k >> 2) * KB_BOX) + (k & 3) * 32) >> 4),
+                        bmu + (uint64_t)((((k >> 2) * C::IMG_ATOM) + (k & 3) * 32) >> 4), C::IDESC, k > 0 ? 1u : 0u);
           umma_commit(smem_u32(&empty[st]));
-          umma_commit(smem_u32(&accfull[ab]));
+          umma_commit(smem_u32(&aempty[ab]));
+          umma_commit(smem_u32(&accfull[ac]));
         }
         if (!ok) break;
         cont = is.next_same_unit(item);
@@ -298,100 +269,85 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
         }
       }
       // every MMA issued here completes before the CTA tears down tensor memory
-      if (it > 0) mbar_wait(smem_u32(&accfull[(it - 1) % KB_NACC]), ((it - 1) / KB_NACC) & 1, ws, nullptr);
+      if (it > 0) mbar_wait(smem_u32(&accfull[(it - 1) % NACC]), ((it - 1) / NACC) & 1, ws, nullptr);
       TRC_ADD(5, tr_all);
       TRC_PUT(ws, TR_K_KPASS, 7);
     }
   } else if (warp == KB_BUILD_WARP) {
-    // ------------------ mu' image and lambda, once per run, one run ahead
+    // ------------------ mu' and lambda images, once per run, one run ahead
     uint32_t nrun = 0;
     bool cont = false;
     Item item;
     for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); is.next(item);) {
       const bool same = cont;
       cont = is.next_same_unit(item);
-      if (same) continue;  // the run's image is in place
+      if (same) continue;  // the run's images are in place
       const int l = item.plane / dm.Hkv, g = item.plane % dm.Hkv;
       const int p = nrun & 1;
       if (nrun >= 2 && !mbar_wait(smem_u32(&imgfree[p]), ((nrun >> 1) - 1) & 1, ws, abort)) break;
       const int64_t qb = (((int64_t)item.seq * dm.L + l) * dm.Hq + (int64_t)g * G) * D;
-      build_split_image<G>(img + p * C::IMG_BYTES, ws.mu + qb, lane);
-      float* lam_s = lams + p * G * D;
-      for (int e = lane; e < G * D / 4; e += 32) ((float4*)lam_s)[e] = ((const float4*)(ws.lam + qb))[e];
+      build_split_images<G>(img + 2 * p * C::IMG_BYTES, ws.mu + qb, ws.lam + qb, lane);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&imgready[p]));
       ++nrun;
     }
-  } else if (warp >= KB_KAPPA_WARP0 && warp < KB_READ_WARP0) {
-    // ------------------------------------------------------ kappa ---------
-    // A group's warp writes its partial kappa of all four token subsets into
-    // the group's slot and signals kready; the readout warp of each subset
-    // adds the four partials (in writer order) and stores the token's row.
-    const int kw = warp - KB_KAPPA_WARP0;
-    const int grp = kw >> 2;                  // tiles with it % 2 == grp
-    const int cq = kw & 3;                    // channel quarter
-    uint32_t it = 0, nrun = 0, ng = 0;        // ng: tiles of this group so far
-    bool cont = false;
-    int p = 0;
+  } else if (warp >= KB_CONV_WARP0 && warp < KB_CONV_WARP0 + KB_CONV_WARPS) {
+    // ------------------------------------------------ convert -------------
+    // Lane = token 32 quarter + lane of the tile, 64 channels of it: 128 bytes
+    // from the staged tile (eight 16-byte loads, free of bank conflicts under
+    // the swizzle), 32 columns of each of the three operands.
+    const int quarter = warp & 3, half = (warp - KB_CONV_WARP0) >> 2;
+    const int row = quarter * 32 + lane;
+    const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
+    uint32_t it = 0;
     Item item;
-    // time accounting (trace builds, warp 2): 7 waits for a K tile, 8 its quarter
-    // of kappa, 9 waits for the group's slot, 10 the partials into it, 11 the loop
+    // time accounting (trace builds, first convert warp): 7 waits for a K tile, 8 for a
+    // free operand buffer, 9 the conversion, 11 the loop
     TRC_DECL(TR_CTA_SLOTS);
     TRC_T(tr_all);
     // Every wait is bounded and the warps meet at no named barrier, so a warp
     // whose wait failed (the abort flag is set) leaves on its own.
     for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); is.next(item);) {
-      if (!cont) {
-        p = nrun & 1;
-        if (!mbar_wait(smem_u32(&imgready[p]), (nrun >> 1) & 1, ws, abort)) goto kappa_done;
-      }
-      {
-        const uint32_t lam_s = smem_u32(lams + p * G * D);
-        for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
-          if ((int)(it & 1) != grp) continue;
-          const int st = it % KB_STAGES;
-          float part[4][G];
-          TRC_T(tr_f);
-          if (!mbar_wait(smem_u32(&full[kb_full<KB_STAGES>(it)]), kb_full_parity<KB_STAGES>(it), ws, abort))
-            goto kappa_done;
-          TRC_ADD(7, tr_f);
-          TRC_T(tr_k);
-          kappa_quarter<G>(smem_u32(tiles + st * KB_TILE_BYTES), lam_s, lane, cq, part);
-          TRC_ADD(8, tr_k);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
-          TRC_T(tr_b);
-          // slot b of the group takes its tiles ng = b, b + SLOTS, ...; it is free
-          // once the readout warps have read its previous tile
-          const int b = ng % C::SLOTS, use = ng / C::SLOTS;
-          const int ks = grp * C::SLOTS + b;
-          if (use >= 1 && !mbar_wait(smem_u32(&kfree[ks]), (use - 1) & 1, ws, abort)) goto kappa_done;
-          TRC_ADD(9, tr_b);
-          TRC_T(tr_r);
-          float* slot = kred + ks * C::SLOT_FLOATS;
+      for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
+        const int st = it % KB_STAGES, ab = it & 1;
+        TRC_T(tr_f);
+        if (!mbar_wait(smem_u32(&full[st]), (it / KB_STAGES) & 1, ws, abort)) goto conv_done;
+        TRC_ADD(7, tr_f);
+        const uint32_t kt = smem_u32(tiles + st * KB_TILE_BYTES + half * KB_BOX);
+        uint32_t r[32];
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int h = 0; h < G; ++h) slot[((j * 4 + cq) * G + h) * 32 + lane] = part[j][h];
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&kready[ks]));
-          ++ng;
-          TRC_ADD(10, tr_r);
+        for (int c = 0; c < 8; ++c) {
+          const uint4 v = lds_u128(kt + sw128_off(row, c));
+          r[4 * c] = v.x, r[4 * c + 1] = v.y, r[4 * c + 2] = v.z, r[4 * c + 3] = v.w;
         }
-      }
-      cont = is.next_same_unit(item);
-      if (!cont) {
+        uint32_t hi[32];
+#pragma unroll
+        for (int c = 0; c < 32; ++c) hi[c] = bf16x2_mul(r[c], r[c]);
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&imgfree[p]));
-        ++nrun;
+        if (lane == 0) mbar_arrive(smem_u32(&empty[st]));  // the tile is in registers
+        TRC_T(tr_a);
+        if (it >= 2 && !mbar_wait(smem_u32(&aempty[ab]), ((it >> 1) & 1) ^ 1, ws, abort)) goto conv_done;
+        TRC_ADD(8, tr_a);
+        TRC_T(tr_b);
+        tc_fence_after();
+        const uint32_t a = tmem + KB_ACC_COLS + ab * KB_A_COLS + 32 * half + lanes;
+        tmem_st_32x32b_x32(a, hi);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) r[c] = bf16x2_fma(r[c], r[c], bf16x2_neg(hi[c]));  // lo, exact
+        tmem_st_32x32b_x32(a + 64, r);
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&afull[ab]));
+        TRC_ADD(9, tr_b);
       }
     }
-  kappa_done:
+  conv_done:
     TRC_ADD(11, tr_all);
-    if (warp == KB_KAPPA_WARP0 && lane == 0) TRC_PUT(ws, TR_K_KPASS, 12);
-  } else if (warp >= KB_READ_WARP0 && warp < KB_READ_WARP0 + 4) {
-    // ------------------------------------------ logits readout + stats ----
+    if (warp == KB_CONV_WARP0 && lane == 0) TRC_PUT(ws, TR_K_KPASS, 12);
+  } else if (warp >= KB_READ_WARP0) {
+    // ------------------------------------------------ readout + stats -----
     const int quarter = warp & 3;
     const int y = quarter * 32 + lane;        // token row (tensor-memory lane)
     const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
@@ -400,8 +356,8 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
     bool bad = false, cont = false;
     float run_m[G], run_s[G];
     Item item;
-    // time accounting (trace builds, first readout warp): 12 waits for logits, 13 the
-    // readout of a tile (with 15, its wait for the kappa partials), 14 the whole loop
+    // time accounting (trace builds, first readout warp): 12 waits for an accumulator, 13
+    // the readout of a tile, 14 the whole loop
     TRC_DECL(TR_CTA_SLOTS);
     TRC_T(tr_all);
     for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); is.next(item);) {
@@ -414,42 +370,46 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
       }
       float* lkp = ws.lk + (int64_t)item.plane * dm.Ntot * (2 * G);
       for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
-        const int ab = it % KB_NACC;
+        const int ac = it % NACC;
         TRC_T(tr_f);
-        if (!mbar_wait(smem_u32(&accfull[ab]), (it / KB_NACC) & 1, ws, abort)) break;  // abort: see below
+        if (!mbar_wait(smem_u32(&accfull[ac]), (it / NACC) & 1, ws, abort)) break;  // abort: see below
         TRC_ADD(12, tr_f);
         TRC_T(tr_b);
         tc_fence_after();
-        float dv[C::NB];
-        if constexpr (C::NB == 16) tmem_ld16(tmem + ab * C::NB + lanes, dv);
-        else tmem_ld32(tmem + ab * C::NB + lanes, dv);
+        // NB columns of logit parts, then NB of kappa parts per channel group:
+        // part p of head h in column p G + h
+        const uint32_t src = tmem + ac * C::ACC + lanes;
+        float row[2 * G];  // logits, then kappa; the small parts first
+        {
+          constexpr int PS = NB == 16 ? G : 8;  // part p of head h at dv[p PS + h]
+          float dv[NB == 16 ? 16 : 24];
+          auto load = [&](uint32_t col) {
+            if constexpr (NB == 16) tmem_ld16(col, dv);
+            else tmem_ld8x3(col, G, dv);
+          };
+          float low[G];
+          load(src);
+#pragma unroll
+          for (int h = 0; h < G; ++h) row[h] = dv[h] + (dv[PS + h] + dv[2 * PS + h]);
+#pragma unroll
+          for (int g = 1; g <= C::KG; ++g) {
+            load(src + g * NB);
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+              row[G + h] = g == 1 ? dv[h] : row[G + h] + dv[h];
+              low[h] = g == 1 ? dv[PS + h] + dv[2 * PS + h] : low[h] + (dv[PS + h] + dv[2 * PS + h]);
+            }
+          }
+#pragma unroll
+          for (int h = 0; h < G; ++h) row[G + h] += low[h];
+        }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&accempty[ab]));
-        // kappa of this warp's 32 tokens: the four partials of the tile's group
-        // (the group's slot holds [token subset][writer][G][32]), added in writer order
-        const uint32_t ng = it >> 1;  // the tile is the ng-th of group it % 2
-        const int ks = (int)(it & 1) * C::SLOTS + (int)(ng % C::SLOTS);
-        TRC_T(tr_k);
-        if (!mbar_wait(smem_u32(&kready[ks]), (ng / C::SLOTS) & 1, ws, abort)) break;  // abort: see below
-        TRC_ADD(15, tr_k);
-        const float* slot = kred + ks * C::SLOT_FLOATS;
-        float row[2 * G];  // logits, then kappa
-#pragma unroll
-        for (int h = 0; h < G; ++h) {
-          float v = 0.f;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) v += slot[((quarter * 4 + q) * G + h) * 32 + lane];
-          row[G + h] = v;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&kfree[ks]));
-        const int64_t tok = t + y;
-        if (tok < item.t1) {
+        if (lane == 0) mbar_arrive(smem_u32(&accempty[ac]));
+        if (t + y < item.t1) {
 #pragma unroll
           for (int h = 0; h < G; ++h) {
-            const float lg = dv[h] + dv[G + h] + dv[2 * G + h];
-            row[h] = lg;
+            const float lg = row[h];
             bad |= !isfinite(lg) || !isfinite(row[G + h]);
             // branch-free online update: one of the two exponentials is exp(0);
             // both arguments are <= 0, where the fast exponential's relative
@@ -458,8 +418,26 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
             run_s[h] = run_s[h] * __expf(run_m[h] - mn) + __expf(lg - mn);
             run_m[h] = mn;
           }
-          store_floats<2 * G, LkAlign<G>::ROW>(lkp + tok * (2 * G), row);
         }
+        // the warp's rows are contiguous in global memory: through shared memory,
+        // so that each store instruction writes whole lines (a lane's own row
+        // written by itself costs 2 G / V instructions of 32 partial sectors)
+        constexpr int V = LkAlign<G>::ROW;
+        float* wrows = rows + quarter * 32 * 2 * G;
+        store_floats<2 * G, V>(wrows + lane * 2 * G, row);
+        __syncwarp();
+        const int64_t left = item.t1 - t - 32 * quarter;
+        const int nf = (int)(left < 0 ? 0 : (left < 32 ? left : 32)) * 2 * G;
+        float* dst = lkp + (t + 32 * quarter) * (2 * G);
+#pragma unroll
+        for (int e = 0; e < 2 * G / V; ++e) {
+          const int f = (lane + 32 * e) * V;
+          if (f < nf) {
+            if constexpr (V == 4) *(float4*)(dst + f) = *(const float4*)(wrows + f);
+            else *(float2*)(dst + f) = *(const float2*)(wrows + f);
+          }
+        }
+        __syncwarp();
         TRC_ADD(13, tr_b);
       }
       // ---- softmax statistics of a run, at its last chunk; the run's other
@@ -496,7 +474,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
     }
   read_done:
     TRC_ADD(14, tr_all);
-    if (warp == KB_READ_WARP0 && lane == 0) TRC_PUT(ws, TR_K_KPASS, 16);
+    if (warp == KB_READ_WARP0 && lane == 0) TRC_PUT(ws, TR_K_KPASS, 15);
     if (bad) flag(ws, ST_NONFINITE);
   }
   tc_fence_before();

@@ -504,3 +504,27 @@ def test_full_size_full_covariance():
         check_unit(ev, t, wl, params, 0, layer, g, check_w=False)
     del ev, t
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("G", range(1, 9))
+@pytest.mark.parametrize("scale", (1.0, 1e-12, 1e6))
+def test_kappa_of_every_group_size_at_tile_edges(G, scale):
+    """kappa through the linear surrogate's weights, w = (1/d) sum_h kappa_h, for requests that end
+    before, on and after a tile's edge and keys far from 1. All terms are positive, squares and
+    products are exact, so the error is that of lambda in float32 ((w + 3) 2^-24 relative: two sums
+    over the window) and of at most 16 truncated and 8 rounded additions (2^-23 each at most). The
+    keys stay below 1e7, so that w < 1e15 and the squares of A's entries, w^2 n^2, below float32's
+    3e38 in the kernels that follow."""
+    wl = Workload("t", 1, 2 * G, 2, (129, 1, 128, 127, 385), 16, 8, seed=300 + G)
+    t = generate(wl, "cuda")
+    t.k.mul_(scale)
+    ev = evict(make_cache(t, wl), wl.budget, jacap_params(linear_weighting=1))
+    w = ev.intermediates()["weights"].double()
+    cu = t.cu_seqlens.tolist()
+    bound = (16 + 3) * 2.0 ** -24 + (16 + 8) * 2.0 ** -23
+    for s in range(len(wl.seqlens)):
+        q = t.q_win[s, 0].double().view(2, G, 16, 128)
+        lam = (q - q.mean(2, keepdim=True)).square().mean(2).sum(1)  # [2, 128], summed over the heads
+        k2 = t.k[0, :, cu[s]:cu[s + 1]].double().square()
+        ref = torch.einsum("gnc,gc->gn", k2, lam) / 128
+        assert bool(((w[0, :, cu[s]:cu[s + 1]] - ref).abs() <= bound * ref).all())
