@@ -24,7 +24,7 @@ inline size_t align_up(size_t x) { return (x + ALIGN - 1) & ~(ALIGN - 1); }
 struct Carve {
   size_t status, plan, chunks, counters, mu, lam, qdev, lk, cstats, ustats, w, gpart, pflag, gram, minv,
       minv_img, total;
-  size_t units, trace, trace_cta;
+  size_t units, trace, trace_cta, base, runs, sched;
 };
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -126,6 +126,9 @@ Carve carve(const Dims& dm) {
   c.gram = o; o = align_up(o + units * D * D * 4);
   c.minv = o; o = align_up(o + units * D * D * 4);
   c.minv_img = o; o = align_up(o + units * 65536);
+  c.base = o;  // the static scratch's limit applies to the sections up to here (jacap_static.cu)
+  c.runs = o; o = align_up(o + 2 * (size_t)dm.c_cap * 16);
+  c.sched = o; o = align_up(o + 32 + 2 * ((size_t)dm.S + 2) * 4);  // run counters, then the run prefixes
 #ifdef JACAP_TRACE
   c.trace = o; o = align_up(o + units * TR_SLOTS * 8);  // trace builds: the fused schedule's timeline,
   c.trace_cta = o; o = align_up(o + (size_t)TR_KERNELS * TR_CTAS * TR_CTA_SLOTS * 8);  // then the CTA accounting
@@ -143,6 +146,9 @@ Ws make_ws(void* base, const Carve& c) {
   ws.status = (uint32_t*)(b + c.status);
   ws.plan = (int32_t*)(b + c.plan);
   ws.chunks = (int4*)(b + c.chunks);
+  ws.runs = (int4*)(b + c.runs);
+  ws.sched = (int32_t*)(b + c.sched);
+  ws.rplan = ws.sched + 8;
   ws.gcount = (int32_t*)(b + c.counters);
   ws.fdone = ws.gcount + c.units;  // right after gcount: the plan kernel zeroes 2 x units words
   ws.mu = (float*)(b + c.mu);
@@ -306,6 +312,25 @@ int pick_schedule(const jacap_layout* L, const jacap_params* P, const Dims& dm, 
   return 2;
 }
 
+// The runs of the streaming kernels (RunStream). Up to 24 tiles per SM: one
+// equal run each. Otherwise about eight runs per SM, of 8 to 64 tiles (a run
+// costs an image and a set of statistics, ~1.5 us beside ~0.75 us per tile), and
+// the last 36 tiles' worth per SM in runs of 8 tiles (at least a chunk).
+void pick_runs(Dims& dm, int64_t items, int sms) {
+  const int64_t planes = (int64_t)dm.L * dm.Hkv, per_plane = std::max<int64_t>(1, items / planes);
+  const int64_t ct = dm.chunk / TILE, q = items * ct / sms;  // tiles per chunk and per SM
+  dm.big_planes = (int)planes;
+  if (q <= 24) {
+    dm.run_chunks[0] = dm.run_chunks[1] = (int)std::max<int64_t>(1, (items + sms - 1) / sms);
+    return;
+  }
+  const int64_t small = std::max<int64_t>(1, 8 / ct);
+  dm.run_chunks[0] = (int)std::max(small, std::min<int64_t>(64, q / 8) / ct);
+  dm.run_chunks[1] = (int)small;
+  if (dm.run_chunks[0] > small)
+    dm.big_planes = (int)std::max<int64_t>(0, planes - ((36 + ct - 1) / ct * sms + per_plane - 1) / per_plane);
+}
+
 // Work items of the pass (plane x chunk): exact for one request, otherwise the
 // capacity bound (the device computes the exact count from cu_seqlens).
 int64_t pass_items(const jacap_layout* L, const Dims& dm) {
@@ -314,6 +339,13 @@ int64_t pass_items(const jacap_layout* L, const Dims& dm) {
 }
 
 }  // namespace
+
+size_t jacap::workspace_base(const jacap_layout* layout) {
+  if (check_layout(layout) != JACAP_OK) return 0;
+  Dims dm;
+  make_dims(layout, nullptr, dm);
+  return carve(dm).base;
+}
 
 extern "C" {
 
@@ -394,6 +426,8 @@ jacap_status score_pass(const jacap_layout* layout, const jacap_params* params, 
   const bool bf = layout->dtype == JACAP_BF16;
   if (!encode_kv_map(&kmap, layout, k) || !encode_kv_map(&vmap, layout, v)) return JACAP_ERR_CUDA;
   const int64_t items = pass_items(layout, dm);
+  if (items >= ((int64_t)1 << 31)) return JACAP_ERR_UNSUPPORTED;
+  pick_runs(dm, items, sms);
   const int dt = bf ? 1 : 0;
   const int32_t* cu = layout->cu_seqlens;
   // hook(i): the boundary before kernel i (optional timing event; with

@@ -47,6 +47,8 @@ struct Dims {
   int keep_tiles;     // fused: V tiles of each Gram item loaded with the L2 evict_last policy (the score
                       // role reads them again soon after); the item's other tiles are loaded evict_first
   int run_items;      // fused: consecutive items a role's CTA takes at a time (one partial Gram per run)
+  int run_chunks[2];  // separate kernels: chunks per run (at most) of the first big_planes planes, and of the
+  int big_planes;     // planes after them, see RunStream
 };
 
 // Rows per split part of the full-covariance query image of one KV head's
@@ -62,7 +64,10 @@ __host__ __device__ constexpr int kfull_rows_padded(int G, int W) {
 struct Ws {
   uint32_t* status;   // [16] status word + first failing unit
   int32_t* plan;      // [0] = chunks per plane C_tot, [1 .. S+1] = chunk prefix per request
+  int32_t* rplan;     // two lists of runs, list m at m (S + 2): [0] = runs per plane, [1 .. S+1] = run prefix
   int4* chunks;       // [c_cap] chunk r of every plane: {t0, t1, request, r}
+  int4* runs;         // [2][c_cap] run r of every plane, for each list: {t0, t1, request, first chunk}
+  int32_t* sched;     // [8] next run of each streaming kernel beyond the first one of each CTA (SCHED_*)
   int32_t* gcount;    // [units] fused schedule: Gram progress of a unit (each item adds 1 for its weights
                       // and 1 for its partial Gram; complete at 2 x the unit's chunk count)
   int32_t* fdone;     // [units] fused schedule: 1 once the unit's factor (G, L^{-1} and its image) is written
@@ -189,6 +194,35 @@ struct ItemStream {
   }
 };
 
+// Runs dealt to the CTAs of a streaming kernel as they become free. A run is a
+// sequence of consecutive chunks of one unit (accumulators, images and softmax
+// statistics carry over within it). The list of runs is fixed by the layout:
+// first the big_planes planes in long runs, then the other planes in short ones,
+// so that the CTAs finish close together. Which
+// CTA takes a run is decided while the kernel runs (CTA b starts with run b, then
+// each takes the next one from a counter), so no result depends on it: every
+// sum is over the chunks of a run.
+// Why: with equal shares the CTAs of an HBM-bound pass finish far apart, as the
+// SMs do not get equal shares of the bandwidth (K pass over 32 x 8 x 32768 tokens:
+// 281 to 396 us of equal work, 335 on average). Dealt: K pass 0.402 -> 0.352 ms
+// there, 1.51 -> 1.34 ms over 131072 tokens, 1.39 -> 1.12 ms over 16 requests of
+// 2K to 64K tokens (8 layers); scores 1.117 -> 1.070 ms over those. The Gram keeps
+// equal contiguous shares: a run's end drains its accumulators and leaves a
+// partial for the factor (dealt, it took 0.414 instead of 0.394 ms), and so does
+// the full-covariance K pass, whose one image buffer a new run waits for.
+enum { SCHED_KPASS = 0, SCHED_SCORE = 1 };
+constexpr int RQ_SLOTS = 4;
+struct __align__(16) RunRec {
+  int32_t t0, t1, seq, c0;       // tokens [t0, t1) of the plane's token axis, request, first chunk
+  int32_t plane, nc, pad0, pad1; // plane (-1: no more runs), chunks
+};
+// The producer thread of a CTA takes the runs and hands them to the CTA's other
+// roles through a ring of records in shared memory.
+struct RunQueue {
+  RunRec rec[RQ_SLOTS];
+  uint64_t full[RQ_SLOTS], empty[RQ_SLOTS];
+};
+
 // Largest GQA group (query heads per KV head) the kernels are compiled for.
 constexpr int G_MAX = 8;
 
@@ -269,15 +303,17 @@ __device__ __forceinline__ void softmax_merge(float& m, float& s, float m2, floa
   m = M;
 }
 
-// Butterfly merge of (m, s) over the 32 lanes of a warp; every lane ends with
-// the warp total (same value on every lane, fixed order: deterministic).
+// Merge of (m, s) over the 32 lanes of a warp: the maximum, then the sums scaled
+// to it (one exponential per lane). Every lane ends with the warp total (the same
+// value on every lane, fixed order: deterministic).
 __device__ __forceinline__ void softmax_warp_merge(float& m, float& s) {
+  float M = m;
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-    softmax_merge(m, s, m2, s2);
-  }
+  for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+  s = m == -INFINITY ? 0.f : s * expf(m - M);
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  m = M;
 }
 
 // ------------------------------------------------------------------ PTX ----
@@ -517,6 +553,138 @@ static __device__ __noinline__ bool wait_count(const int32_t* p, int target, con
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
+
+// ------------------------------------------------------------- run queue --
+// One thread, before the CTA's first barrier; `consumers`: the arrivals that
+// free a slot (one per role thread or role warp that reads the queue).
+__device__ __forceinline__ void run_queue_init(RunQueue* q, int consumers) {
+  for (int i = 0; i < RQ_SLOTS; ++i) {
+    mbar_init(smem_u32(&q->full[i]), 1);
+    mbar_init(smem_u32(&q->empty[i]), consumers);
+  }
+}
+
+// The runs of a CTA, chunk by chunk, as one of its roles sees them. PRODUCER:
+// the thread that takes the runs. When it starts on one it claims the next one (an
+// atomic add and a table read, ~1.5 us that its ring of tiles covers) and publishes
+// it, so that the roles that prepare a run (the images) see it a run ahead, and no
+// CTA holds more than one run that it has not started. Otherwise a consumer: a whole warp (`solo` false; all lanes call
+// next() together) or a single thread.
+template <bool PRODUCER>
+struct RunStream {
+  const Dims& dm;
+  const Ws& ws;
+  RunQueue* q;
+  volatile int* abort;
+  bool solo;
+  bool fresh = false;   // the last next() took (or tried to take) a new run
+  bool failed = false;  // ... and its wait failed
+  uint32_t i = 0;       // runs published (producer) or taken
+  int c = 0, c_end = 0, plane = 0, seq = 0, t = 0, t_end = 0;
+  int sched, rtot, stot;
+  int64_t nbig, nall, nxt;
+  RunRec ahead;  // (producer) the run published last, not yet started
+
+  __device__ __forceinline__ RunStream(const Dims& dm_, const Ws& ws_, RunQueue* q_, volatile int* abort_, bool solo_,
+                                       int sched_ = 0)
+      : dm(dm_), ws(ws_), q(q_), abort(abort_), solo(solo_), sched(sched_) {
+    if (PRODUCER) {
+      rtot = ws.rplan[0];
+      stot = ws.rplan[dm.S + 2];
+      nbig = (int64_t)dm.big_planes * rtot;
+      nall = nbig + (int64_t)(dm.L * dm.Hkv - dm.big_planes) * stot;
+      nxt = blockIdx.x;
+      publish();
+    }
+  }
+  // (producer) the record of run nxt into the queue and `ahead`
+  __device__ __forceinline__ void publish() {
+    const int s = i % RQ_SLOTS;
+    RunRec r;
+    r.plane = -1;
+    if (nxt < nall) {
+      const bool big = nxt < nbig;
+      const uint32_t n = (uint32_t)(big ? nxt : nxt - nbig), per = (uint32_t)(big ? rtot : stot);
+      const uint32_t p = n / per;  // fewer than 2^31 chunks in all planes (checked by the host)
+      r.plane = (int)p + (big ? 0 : dm.big_planes);
+      const int4 rec = (ws.runs + (big ? 0 : dm.c_cap))[n - p * per];
+      r.t0 = rec.x, r.t1 = rec.y, r.seq = rec.z, r.c0 = rec.w;
+      r.nc = (rec.y - rec.x + dm.chunk - 1) / dm.chunk;
+#ifdef JACAP_CHECKED
+      // checked build: a record outside the cache ends this CTA's runs and is
+      // reported (ST_INVALID) instead of being streamed
+      if (r.t0 < 0 || r.t1 <= r.t0 || r.t1 > dm.Ntot || r.seq < 0 || r.seq >= dm.S || r.c0 < 0 ||
+          r.c0 + r.nc > ws.plan[0] || r.plane >= dm.L * dm.Hkv) {
+        atomicOr(ws.status, 1u);
+        r.plane = -1;
+      }
+#endif
+    }
+    ahead = r;
+    if (i >= RQ_SLOTS && !mbar_wait(smem_u32(&q->empty[s]), ((i / RQ_SLOTS) & 1) ^ 1, ws, abort)) {
+      failed = true;
+      return;
+    }
+    q->rec[s] = r;
+    mbar_arrive(smem_u32(&q->full[s]));
+    ++i;
+  }
+  __device__ __forceinline__ bool take(RunRec& r) {
+    if constexpr (PRODUCER) {
+      r = ahead;
+      if (failed || r.plane < 0) return false;
+      nxt = (int64_t)gridDim.x + atomicAdd(ws.sched + sched, 1);
+      publish();
+      return true;
+    } else {
+      const int s = i % RQ_SLOTS;
+      if (!mbar_wait(smem_u32(&q->full[s]), (i / RQ_SLOTS) & 1, ws, abort)) {
+        failed = true;
+        return false;
+      }
+      r = q->rec[s];
+      if (!solo) __syncwarp();
+      if (solo || (threadIdx.x & 31) == 0) mbar_arrive(smem_u32(&q->empty[s]));
+      ++i;
+      return r.plane >= 0;
+    }
+  }
+  __device__ __forceinline__ bool next(Item& it) {
+    fresh = c == c_end;
+    if (fresh) {
+      RunRec r;
+      if (!take(r)) return false;
+      plane = r.plane, seq = r.seq, t = r.t0, t_end = r.t1, c = r.c0, c_end = r.c0 + r.nc;
+    }
+    it.plane = plane;
+    it.seq = seq;
+    it.cidx = c;
+    it.t0 = t;
+    const int t1 = t_end - t > dm.chunk ? t + dm.chunk : t_end;
+    it.t1 = t1;
+    t = t1;
+    ++c;
+    return true;
+  }
+  // whether the run goes on after the item last returned by next()
+  __device__ __forceinline__ bool next_same_unit(const Item&) const { return c < c_end; }
+};
+
+// The work of a role: the runs dealt by the CTA's producer, or (the fused
+// schedule's roles, part `part` of `parts`) strided items.
+template <bool FUSED, bool PRODUCER>
+struct RoleStream : RunStream<PRODUCER> {
+  __device__ __forceinline__ RoleStream(const Dims& dm, const Ws& ws, RunQueue* q, volatile int* abort, bool solo,
+                                        int sched, int, int)
+      : RunStream<PRODUCER>(dm, ws, q, abort, solo, sched) {}
+};
+template <bool PRODUCER>
+struct RoleStream<true, PRODUCER> : ItemStream {
+  static constexpr bool fresh = false, failed = false;
+  __device__ __forceinline__ RoleStream(const Dims& dm, const Ws& ws, RunQueue*, volatile int*, bool, int, int part,
+                                        int parts)
+      : ItemStream(dm, ws, part, parts, true) {}
+};
 
 // ------------------------------------------------------------ tcgen05 ----
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {

@@ -3,9 +3,14 @@
 // the kernel was enqueued).
 #pragma once
 
+#include "jacap.h"
 #include "jacap_dev.cuh"
 
 namespace jacap {
+
+// Bytes of the workspace of a layout without the run tables at its end (0 for
+// an invalid layout).
+size_t workspace_base(const jacap_layout* layout);
 
 // Tracing: built with -DJACAP_NVTX (JACAP_NVTX=1 in the environment of the
 // build), the host side marks each kernel's launch with an NVTX range named

@@ -17,11 +17,17 @@
 #include <mutex>
 
 #include "jacap.h"
+#include "jacap_internal.h"
 
 namespace {
 
 // The scratch, one copy per device context (the module is loaded per context).
-static __device__ __align__(256) unsigned char g_static_scratch[JACAP_STATIC_SCRATCH_BYTES];
+// JACAP_STATIC_SCRATCH_BYTES is the limit on a layout's workspace without its
+// run tables; those take at most 48 bytes per chunk and request on top, and a
+// layout within the limit has at most 1024 of each (64 KB of partial Gram per
+// chunk; a request adds a chunk).
+constexpr size_t SCRATCH_BYTES = (size_t)JACAP_STATIC_SCRATCH_BYTES + 65536;
+static __device__ __align__(256) unsigned char g_static_scratch[SCRATCH_BYTES];
 
 constexpr int MAX_DEVICES = 64;
 struct Slot {
@@ -86,14 +92,15 @@ jacap_status jacap_score_static(const jacap_layout* layout, const jacap_params* 
   // An invalid or unsupported layout: jacap_score reports which, from its
   // host checks, before it looks at the (absent) workspace.
   if (need == 0) return jacap_score(layout, params, q_win, k, v, scores, nullptr, 0, stream);
-  if (need > (size_t)JACAP_STATIC_SCRATCH_BYTES) return JACAP_ERR_WORKSPACE;
+  if (jacap::workspace_base(layout) > (size_t)JACAP_STATIC_SCRATCH_BYTES || need > SCRATCH_BYTES)
+    return JACAP_ERR_WORKSPACE;
   void* ws = scratch_for_current_device();
   if (ws == nullptr) return JACAP_ERR_CUDA;
   if (scratch_out != nullptr) *scratch_out = ws;
   // jacap_score's first kernel clears the status word (the only state that
   // must start at zero); every other section of the workspace is written
   // before it is read within one pass.
-  return jacap_score(layout, params, q_win, k, v, scores, ws, (size_t)JACAP_STATIC_SCRATCH_BYTES, stream);
+  return jacap_score(layout, params, q_win, k, v, scores, ws, SCRATCH_BYTES, stream);
 }
 
 }  // extern "C"

@@ -27,7 +27,8 @@
 // group of four warps at G = 4, and grew with G. Measured, both kinds, K pass
 // alone (events): 32 layers x 8 KV heads x 32768 tokens, G = 4: 0.403 -> 0.385
 // ms; 40 x 8 x 9001, G = 5: 0.202 -> 0.147 ms; 28 x 4 x 20011, G = 7: 0.209 ->
-// 0.136 ms. What bounds it now is HBM (6.3 TB/s of K and rows at G = 4).
+// 0.136 ms; and with the runs dealt as CTAs become free (RunStream) 0.352, 0.137
+// and 0.122 ms. What bounds it now is HBM (6.9 TB/s of K and rows at G = 4).
 //
 // Warp roles: 0 TMA producer; 1 issues the MMAs; 2 builds the mu' and lambda
 // images of each unit a CTA reaches (double-buffered, one run of the unit's
@@ -59,9 +60,9 @@ struct KbCfg {
   static constexpr int IMG_BYTES = 2 * IMG_ATOM;       // one image; a run has two (mu', lambda)
   static constexpr uint32_t IDESC = idesc_bf16_f32(128, NB, 0, 0);
   static constexpr size_t smem_for(int stages) {
-    return 1024 + (size_t)stages * KB_TILE_BYTES + 4 * IMG_BYTES + TILE * 2 * G * 4 + 4 * 2 * G * 4 + 256;
+    return 1024 + (size_t)stages * KB_TILE_BYTES + 4 * IMG_BYTES + TILE * 2 * G * 4 + 8 * 2 * G * 4 + 256;  // + barriers
   }
-  static constexpr int STAGES = smem_for(6) <= 232448 ? 6 : 5;  // K tiles in flight
+  static constexpr int STAGES = smem_for(6) + 512 <= 232448 ? 6 : 5;  // K tiles in flight
   static constexpr size_t SMEM = smem_for(STAGES);
 };
 
@@ -123,8 +124,8 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
   uint8_t* tiles = smem;
   uint8_t* img = tiles + KB_STAGES * KB_TILE_BYTES;  // [parity][mu', lambda][IMG_BYTES]
   float* rows = (float*)(img + 4 * C::IMG_BYTES);     // [TILE][2G] the tile's rows on their way out
-  float* red = rows + TILE * 2 * G;                   // [4 readout warps][2G]
-  uint64_t* full = (uint64_t*)(red + 4 * 2 * G);
+  float* red = rows + TILE * 2 * G;                   // [run parity][4 readout warps][2G]
+  uint64_t* full = (uint64_t*)(red + 8 * 2 * G);
   uint64_t* empty = full + KB_STAGES;
   uint64_t* afull = empty + KB_STAGES;   // [2] the tile's A operands are in tensor memory
   uint64_t* aempty = afull + 2;          // [2] the MMAs have read them
@@ -135,11 +136,13 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
   static_assert((2 * KB_STAGES + 4 + 2 * NACC + 4) * 8 <= 256, "barriers");
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort, s_skip;
+  __shared__ RunQueue s_queue;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     s_abort = 0;
     s_skip = status_failed(ws) ? 1 : 0;
+    run_queue_init(&s_queue, 2 + KB_CONV_WARPS + 4);  // MMA, builder, convert and readout warps
     for (int i = 0; i < KB_STAGES; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
       mbar_init(smem_u32(&empty[i]), KB_CONV_WARPS + 1);  // and the MMAs' commit
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
       // time accounting (trace builds): 0 waits for a free stage, 1 the whole loop
       TRC_DECL(TR_CTA_SLOTS);
       TRC_T(tr_all);
-      for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); ok && is.next(item);) {
+      for (RunStream<true> is(dm, ws, &s_queue, abort, true, SCHED_KPASS); ok && is.next(item);) {
         const int l = item.plane / dm.Hkv, g = item.plane % dm.Hkv;
         for (int64_t t = item.t0; t < item.t1; t += TILE) {
           const int st = it % KB_STAGES;
@@ -215,7 +218,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
       // free accumulator, 5 the whole loop, 6 tiles
       TRC_DECL(TR_CTA_SLOTS);
       TRC_T(tr_all);
-      for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); ok && is.next(item);) {
+      for (RunStream<false> is(dm, ws, &s_queue, abort, true); ok && is.next(item);) {
         if (!cont) {
           p = nrun & 1;
           TRC_T(tr_i);
@@ -278,7 +281,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
     uint32_t nrun = 0;
     bool cont = false;
     Item item;
-    for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); is.next(item);) {
+    for (RunStream<false> is(dm, ws, &s_queue, abort, false); is.next(item);) {
       const bool same = cont;
       cont = is.next_same_unit(item);
       if (same) continue;  // the run's images are in place
@@ -308,7 +311,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
     TRC_T(tr_all);
     // Every wait is bounded and the warps meet at no named barrier, so a warp
     // whose wait failed (the abort flag is set) leaves on its own.
-    for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); is.next(item);) {
+    for (RunStream<false> is(dm, ws, &s_queue, abort, false); is.next(item);) {
       for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
         const int st = it % KB_STAGES, ab = it & 1;
         TRC_T(tr_f);
@@ -354,13 +357,18 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
     const int rw = warp - KB_READ_WARP0;
     uint32_t it = 0;
     bool bad = false, cont = false;
+    int par = 0;
     float run_m[G], run_s[G];
     Item item;
     // time accounting (trace builds, first readout warp): 12 waits for an accumulator, 13
     // the readout of a tile, 14 the whole loop
     TRC_DECL(TR_CTA_SLOTS);
     TRC_T(tr_all);
-    for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); is.next(item);) {
+    for (RunStream<false> is(dm, ws, &s_queue, abort, false);;) {
+      if (!is.next(item)) {  // no more runs, or a failed wait: the four warps leave together (see below)
+        named_barrier_any(1, 128, is.failed);
+        break;
+      }
       if (!cont) {  // a new run of the unit's consecutive chunks: fresh statistics
 #pragma unroll
         for (int h = 0; h < G; ++h) {
@@ -455,22 +463,24 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
       for (int h = 0; h < G; ++h) {
         softmax_warp_merge(run_m[h], run_s[h]);
         if (lane == 0) {
-          red[rw * 2 * G + h] = run_m[h];
-          red[rw * 2 * G + G + h] = run_s[h];
+          red[(par * 4 + rw) * 2 * G + h] = run_m[h];
+          red[(par * 4 + rw) * 2 * G + G + h] = run_s[h];
         }
       }
-      // a warp that met an abort still arrives here; the barrier ORs the flag,
-      // so all four leave together
+      // One barrier per run, and one before leaving: a warp that met an abort, or
+      // could not take its next run, still arrives at it; the barrier ORs the
+      // flag, so all four leave together.
       if (named_barrier_any(1, 128, *abort != 0)) goto read_done;
       if (rw == 0 && lane < G) {
         const int h = lane;
         float m = -INFINITY, ssum = 0.f;
-        for (int j = 0; j < 4; ++j) softmax_merge(m, ssum, red[j * 2 * G + h], red[j * 2 * G + G + h]);
+        for (int j = 0; j < 4; ++j)
+          softmax_merge(m, ssum, red[(par * 4 + j) * 2 * G + h], red[(par * 4 + j) * 2 * G + G + h]);
         float* cs = ws.cstats + (((int64_t)item.plane * dm.c_cap + item.cidx) * G + h) * 2;
         cs[0] = m;
         cs[1] = ssum;
       }
-      named_barrier_sync(1, 128);
+      par ^= 1;  // the next run's partials go elsewhere: no second barrier
     }
   read_done:
     TRC_ADD(14, tr_all);
@@ -489,7 +499,7 @@ template <int G>
 static cudaError_t launch_g(const CUtensorMap& kmap, const Dims& dm, const Ws& ws, const int32_t* cu, int grid,
                             cudaStream_t st) {
   constexpr size_t smem = KbCfg<G>::SMEM;
-  static_assert(smem <= 232448, "shared memory budget");
+  static_assert(smem + 512 <= 232448, "shared memory budget");  // 512: the static variables
   cudaError_t e = cudaFuncSetAttribute(kpass_bf16_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   JACAP_TRY(launch_pdl(dm.pdl != 0, kpass_bf16_kernel<G>, grid, KB_THREADS, smem, st, kmap, dm, ws, cu));

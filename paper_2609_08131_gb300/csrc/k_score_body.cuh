@@ -71,11 +71,13 @@ __device__ __forceinline__ void score_bf16_body(const CUtensorMap* vmap_p, const
   float* s_part = (float*)(stages + SC_STAGES * SC_TILE_BYTES + 144);  // [2][128] second group's partial sums
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort, s_skip;
+  __shared__ RunQueue s_queue;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     s_abort = 0;
     s_skip = status_failed(ws) ? 1 : 0;
+    run_queue_init(&s_queue, 2 + 8);  // MMA, image and epilogue warps
     for (int i = 0; i < SC_STAGES; ++i) {
       mbar_init(smem_u32(&vfull[i]), 1);
       mbar_init(smem_u32(&vempty[i]), 1);
@@ -114,7 +116,7 @@ __device__ __forceinline__ void score_bf16_body(const CUtensorMap* vmap_p, const
       // time accounting (trace builds): 0 waits for a free stage, 1 the whole loop
       TRC_DECL(TR_CTA_SLOTS);
       TRC_T(tr_all);
-      for (ItemStream is(dm, ws, part, parts, FUSED); ok && is.next(item);) {
+      for (RoleStream<FUSED, true> is(dm, ws, &s_queue, abort, true, SCHED_SCORE, part, parts); ok && is.next(item);) {
         const int l = item.plane / dm.Hkv, g = item.plane % dm.Hkv;
         for (int64_t t = item.t0; t < item.t1; t += TILE) {
           const int st = it % SC_STAGES;
@@ -149,7 +151,7 @@ __device__ __forceinline__ void score_bf16_body(const CUtensorMap* vmap_p, const
       uint32_t nrun = 0;
       bool cont = false;
       Item item;
-      for (ItemStream is(dm, ws, part, parts, FUSED); is.next(item);) {
+      for (RoleStream<FUSED, false> is(dm, ws, &s_queue, abort, true, SCHED_SCORE, part, parts); is.next(item);) {
         const bool same = cont;
         cont = is.next_same_unit(item);
         if (same) continue;
@@ -185,7 +187,7 @@ __device__ __forceinline__ void score_bf16_body(const CUtensorMap* vmap_p, const
       // accumulator, 4 for a V tile, 5 the whole loop, 6 tiles
       TRC_DECL(TR_CTA_SLOTS);
       TRC_T(tr_all);
-      for (ItemStream is(dm, ws, part, parts, FUSED); ok && is.next(item);) {
+      for (RoleStream<FUSED, false> is(dm, ws, &s_queue, abort, true, SCHED_SCORE, part, parts); ok && is.next(item);) {
         if (!cont) {
           mp = nrun % SC_IMGS;
           TRC_T(tr_m);
@@ -264,7 +266,13 @@ __device__ __forceinline__ void score_bf16_body(const CUtensorMap* vmap_p, const
     // 8 reading and reducing it, 9 the rest of the tile, 10 the whole loop
     TRC_DECL(TR_CTA_SLOTS);
     TRC_T(tr_all);
-    for (ItemStream is(dm, ws, part, parts, FUSED); is.next(item);) {
+    for (RoleStream<FUSED, false> is(dm, ws, &s_queue, abort, false, SCHED_SCORE, part, parts);;) {
+      if (!is.next(item)) {
+        // no more runs, or a failed wait: the two warps of a lane quarter leave
+        // together (the partner may be at its next tile's barrier)
+        if (!FUSED) named_barrier_any(1 + quarter, 64, is.failed);
+        break;
+      }
       bool unit_ok = true;
       if (FUSED && !cont && grp == 0) {  // the unit's weights are complete once its factor is published
         if (lane == 0) unit_ok = wait_count(ws.fdone + (int64_t)item.plane * dm.S + item.seq, 1, ws, abort);

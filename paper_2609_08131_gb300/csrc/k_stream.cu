@@ -2,7 +2,8 @@
 //
 //  plan_kernel          clears the status word, validates cu_seqlens and lays
 //                       out the work items (chunks of `chunk` tokens that never
-//                       straddle requests) in the chunk table.
+//                       straddle requests) in the chunk table, and runs of them
+//                       in the run table.
 //  window_stats_kernel  mu_h and the diagonal of Lambda_Q from the last w queries
 //                       of each query head (Sec. 3.4 last paragraph; App. B.2).
 //  kpass_kernel         (float32 caches; bf16 caches use k_kpass.cu) one
@@ -18,29 +19,53 @@
 namespace jacap {
 
 // The pass's first kernel, one block: clears the status word, validates
-// cu_seqlens and lays out the chunks (thread 0), then writes the chunk table:
-// record r = {t0, t1, request, r} for the C_tot chunks of a plane.
+// cu_seqlens and counts the chunks and runs of each request (warp 0), then writes
+// the chunk table, record r = {t0, t1, request, r} for the C_tot chunks of a
+// plane, and its two lists of runs, {t0, t1, request, first chunk} each.
 __global__ void __launch_bounds__(256) plan_kernel(Dims dm, Ws ws, const int32_t* __restrict__ cu) {
   pdl_wait();
-  __shared__ int s_ctot;
+  __shared__ int s_ctot, s_rtot[2];
   if (threadIdx.x < 16) ws.status[threadIdx.x] = 0u;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 8) ws.sched[threadIdx.x] = 0;
+  int32_t* cpre = ws.plan + 1;          // [S + 1] chunk prefix
+  __syncthreads();  // the status word is clear
+  if (threadIdx.x < 32) {  // warp 0: 32 requests at a time
+    const int lane = threadIdx.x;
     bool ok = (cu[0] == 0) && ((int64_t)cu[dm.S] == dm.Ntot);
-    int32_t acc = 0;
-    ws.plan[1] = 0;
-    for (int s = 0; s < dm.S; ++s) {
-      const int32_t n = cu[s + 1] - cu[s];
+    int32_t cacc = 0, racc[2] = {0, 0};
+    for (int s0 = 0; s0 < dm.S; s0 += 32) {
+      const int s = s0 + lane;
+      const int32_t n = s < dm.S ? cu[s + 1] - cu[s] : 0;
       if (n < 0) ok = false;
-      const int32_t c = n > 0 ? (n + dm.chunk - 1) / dm.chunk : 0;
-      acc += c;
-      ws.plan[2 + s] = acc;
+      const int32_t c = n > 0 ? (n - 1) / dm.chunk + 1 : 0;
+      int32_t v[3] = {c, (c + dm.run_chunks[0] - 1) / dm.run_chunks[0], (c + dm.run_chunks[1] - 1) / dm.run_chunks[1]};
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1)  // inclusive scans
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          const int32_t x = __shfl_up_sync(0xffffffffu, v[e], o);
+          if (lane >= o) v[e] += x;
+        }
+      if (s < dm.S) {
+        cpre[s + 1] = cacc + v[0];
+        for (int m = 0; m < 2; ++m) ws.rplan[m * (dm.S + 2) + 2 + s] = racc[m] + v[1 + m];
+      }
+      cacc += __shfl_sync(0xffffffffu, v[0], 31);
+      for (int m = 0; m < 2; ++m) racc[m] += __shfl_sync(0xffffffffu, v[1 + m], 31);
     }
-    if (!ok || acc > dm.c_cap) {
-      atomicOr(ws.status, ST_INVALID);
-      acc = 0;
+    ok = __all_sync(0xffffffffu, ok) && cacc <= dm.c_cap;
+    if (lane == 0) {
+      if (!ok) {
+        atomicOr(ws.status, ST_INVALID);
+        cacc = racc[0] = racc[1] = 0;
+      }
+      cpre[0] = 0;
+      ws.plan[0] = s_ctot = cacc;
+      for (int m = 0; m < 2; ++m) {
+        ws.rplan[m * (dm.S + 2)] = s_rtot[m] = racc[m];
+        ws.rplan[m * (dm.S + 2) + 1] = 0;
+      }
     }
-    ws.plan[0] = acc;
-    s_ctot = acc;
   }
   // the fused schedule's per-unit progress counters (gcount, then fdone)
   const int64_t units = (int64_t)dm.L * dm.Hkv * dm.S;
@@ -53,17 +78,32 @@ __global__ void __launch_bounds__(256) plan_kernel(Dims dm, Ws ws, const int32_t
     for (int64_t i = threadIdx.x; i < (int64_t)TR_KERNELS * TR_CTAS * TR_CTA_SLOTS; i += blockDim.x) ws.trace_cta[i] = 0;
 #endif
   __syncthreads();
-  const int ctot = s_ctot;
-  for (int r = threadIdx.x; r < ctot; r += blockDim.x) {
-    // largest s with prefix[s] <= r (prefix is plan[1 .. S+1], nondecreasing)
+  // largest s with pre[s] <= r (the prefixes do not decrease)
+  auto request_of = [&](const int32_t* pre, int r) {
     int lo = 0, hi = dm.S - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (ws.plan[1 + mid] <= r) lo = mid; else hi = mid - 1;
+      if (pre[mid] <= r) lo = mid; else hi = mid - 1;
     }
-    const int64_t t0 = (int64_t)cu[lo] + (int64_t)(r - ws.plan[1 + lo]) * dm.chunk;
-    const int64_t t1 = min((int64_t)cu[lo + 1], t0 + (int64_t)dm.chunk);
-    ws.chunks[r] = make_int4((int)t0, (int)t1, lo, r);
+    return lo;
+  };
+  const int ctot = s_ctot;
+  for (int r = threadIdx.x; r < ctot; r += blockDim.x) {
+    const int s = request_of(cpre, r);
+    const int64_t t0 = (int64_t)cu[s] + (int64_t)(r - cpre[s]) * dm.chunk;
+    const int64_t t1 = min((int64_t)cu[s + 1], t0 + (int64_t)dm.chunk);
+    ws.chunks[r] = make_int4((int)t0, (int)t1, s, r);
+  }
+  // a request's chunks in as few runs of at most run_chunks as hold them, of nearly equal lengths
+  for (int e = threadIdx.x; e < s_rtot[0] + s_rtot[1]; e += blockDim.x) {
+    const int m = e < s_rtot[0] ? 0 : 1, r = e - m * s_rtot[0];
+    const int32_t* rpre = ws.rplan + m * (dm.S + 2) + 1;
+    const int s = request_of(rpre, r);
+    const int64_t nc = cpre[s + 1] - cpre[s], k = rpre[s + 1] - rpre[s], j = r - rpre[s];
+    const int64_t c0 = j * nc / k, c1 = (j + 1) * nc / k;
+    const int64_t t0 = (int64_t)cu[s] + c0 * dm.chunk;
+    const int64_t t1 = min((int64_t)cu[s + 1], (int64_t)cu[s] + c1 * dm.chunk);
+    ws.runs[m * dm.c_cap + r] = make_int4((int)t0, (int)t1, s, cpre[s] + (int)c0);
   }
 }
 
