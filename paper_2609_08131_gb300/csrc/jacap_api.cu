@@ -331,6 +331,14 @@ void pick_runs(Dims& dm, int64_t items, int sms) {
     dm.big_planes = (int)std::max<int64_t>(0, planes - ((36 + ct - 1) / ct * sms + per_plane - 1) / per_plane);
 }
 
+// Partial Grams of a unit: every chunk (float32), or one per CTA that its chunks
+// are spread over (bf16, contiguous shares).
+int partials_per_unit(const Dims& dm, int64_t items, int sms, bool bf) {
+  const int64_t units = (int64_t)dm.L * dm.Hkv * dm.S, chunks = std::max<int64_t>(1, items / units);
+  if (!bf) return (int)std::min<int64_t>(chunks, 1 << 20);
+  return (int)std::min<int64_t>(chunks, std::min<int64_t>(items, sms) / units + 1);
+}
+
 // Work items of the pass (plane x chunk): exact for one request, otherwise the
 // capacity bound (the device computes the exact count from cu_seqlens).
 int64_t pass_items(const jacap_layout* L, const Dims& dm) {
@@ -487,7 +495,8 @@ jacap_status score_pass(const jacap_layout* layout, const jacap_params* params, 
   if ((st = hook(4)) != JACAP_OK ||
       (st = map_cuda(launch_gram(vmap, dm, w, dt, v, cu, persistent_grid(items, sms, bf ? 1 : 4), s))) != JACAP_OK)
     return st;
-  if ((st = hook(5)) != JACAP_OK || (st = map_cuda(launch_factor(dm, w, out_factor, s))) != JACAP_OK) return st;
+  if ((st = hook(5)) != JACAP_OK || (st = map_cuda(launch_factor(dm, w, out_factor, partials_per_unit(dm, items, sms, bf), sms, s))) != JACAP_OK)
+    return st;
   if ((st = hook(6)) != JACAP_OK ||
       (st = map_cuda(launch_score(vmap, dm, w, dt, v, cu, scores, persistent_grid(items, sms, bf ? 1 : 2), s))) !=
           JACAP_OK)

@@ -79,7 +79,9 @@ cudaError_t launch_unit_stats(const Dims& dm, const Ws& ws, cudaStream_t st);
 cudaError_t launch_weights(const Dims& dm, const Ws& ws, const int32_t* cu, int grid, cudaStream_t st);
 cudaError_t launch_gram(const CUtensorMap& vmap, const Dims& dm, const Ws& ws, int dtype, const void* v,
                         const int32_t* cu, int grid, cudaStream_t st);
-cudaError_t launch_factor(const Dims& dm, const Ws& ws, const float* out_factor, cudaStream_t st);
+// `partials`: about how many partial Grams a unit has.
+cudaError_t launch_factor(const Dims& dm, const Ws& ws, const float* out_factor, int partials, int sms,
+                          cudaStream_t st);
 cudaError_t launch_score(const CUtensorMap& vmap, const Dims& dm, const Ws& ws, int dtype, const void* v,
                          const int32_t* cu, float* scores, int grid, cudaStream_t st);
 // The fused schedule (k_fused.cu): CTAs of the factor, Gram and score roles.

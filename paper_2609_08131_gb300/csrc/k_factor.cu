@@ -6,30 +6,40 @@
 //  L^{-1}   where A = L L^T.
 //
 // Since v^T A^{-1} v = ||L^{-1} v||^2, the score pass needs only L^{-1}
-// (Eq. 10). It is obtained by Gaussian forward elimination of [A | I] without
-// pivoting (safe: A is symmetric positive definite): after step j the pivot
-// p_j = A_jj and the right block holds X = Lt^{-1}, where A = Lt U with Lt
-// unit lower triangular and U = Diag(p) Lt^T, so L = Lt Diag(p)^{1/2} and
-// L^{-1} = Diag(p)^{-1/2} X.
+// (Eq. 10). It is obtained by block forward elimination of [A | I] without
+// pivoting (safe: A is symmetric positive definite), four rows at a time, in
+// place in registers: a thread holds the tile of rows 8 ty .. + 7 and columns
+// 4 cx .. + 3 of one 128 x 128 array, whose column c holds A until its block is
+// eliminated and the inverse's part afterwards; the 272 tiles that reach the
+// diagonal or lie below it are dealt to 9 warps row by row, so that few lanes
+// idle and whole warps leave as the elimination goes down. Step b (block rows and
+// columns 4 b .. 4 b + 3, Cholesky factor L_b of the pivot block):
+//   u_c = L_b^{-1} A_cb^T  (c below the block)
+//   u_c = L_b^{-1} Z_bc    (c before it): the final rows of L^{-1}
+//   u_c = column of L_b^{-1} (c in it)
+//   Z_rc -= u_r . u_c      for every row r below the block and c <= r (from 0 in the block's columns)
+// The array holds A - I, and each pivot block gets its I when its turn comes: where
+// G is small beside I (long caches), the updates round at G's size and not at 1's.
+// The tiles that own the vectors leave them in shared memory when they have made
+// their update of the step before, the pivot's owner L_b^{-1}; threads 0-127 turn
+// one vector each into u (two barriers a step), and every tile below makes the
+// same rank-4 update.
 //
-// Both blocks share one 128 x 128 register array Z: column c holds A until
-// step c eliminates it, and afterwards Y_c = -p_c X_{., c}. In that scaling
-// the eliminated value A_ic (= m_i p_c with m_i = A_ic / p_c) already equals
-// Y_ic, so step j updates every active row i > j by the same fused
-// multiply-add Z_i. -= m_i r with r_c = A_cj (c > j, lower triangle of A by
-// symmetry), r_j = 0 and r_c = Z_jc (c < j, row j of Y): one barrier and at
-// most 64 multiply-adds per thread. At the end X_ic = -Y_ic / p_c. Thread
-// (ty, tx) of the 8 x 32 grid owns rows ty + 8 a and columns 4 tx .. 4 tx + 3;
-// with 256 threads two units share an SM, so their barrier latencies overlap.
-// The multipliers use 1/p_j from the approximate hardware reciprocal refined by
-// one Newton-Raphson step (x <- x (2 - p x)), which is accurate to about one ulp.
+// Bound: the chain of the 32 steps, 1360 cycles each alone on an SM (barriers 170,
+// vectors left and turned into u 500, the pivot block's four reciprocals 170, the
+// update 520, of which the reads of u from shared memory are the larger part) and
+// 840 (700) per unit with two (three) CTAs on an SM. Measured against blocked
+// 32 x 32 eliminations of one warp each, with the blocks in shared memory: 256
+// units 0.055 -> 0.045 ms, 448 units 0.082 -> 0.061, 1024 units 0.173 -> 0.135;
+// output directions, 128 units, 0.124 -> 0.082 ms. 8 x 8 tiles whose owners formed
+// u themselves took 0.061 and 0.192 ms (two lanes a warp formed eight vectors each).
 //
 // With output directions u = W v (Sec. 3.1) the capacity matrix I + sum w u u^T
 // lives in the output space; with a 128 x 128 factor F of W^T W (F^T F = W^T W)
 // it reduces exactly to M = I + F G F^T, and u^T A^{-1} u = ||L_M^{-1} F v||^2.
-// That variant forms F G F^T from shared-memory copies of G and F (three
-// SIMT float32 products of 128 x 128 matrices), factors M as below and writes
-// T = L_M^{-1} F in place of L^{-1}.
+// That variant (PROJ) forms F G F^T with two float32 products of the same 8 x 8
+// register tiles (operands in shared memory), factors M as above and writes
+// T = L_M^{-1} F, a third product, in place of L^{-1}.
 //
 // L^{-1} is written twice: as float32 (used by the float32 score pass and
 // exposed for tests) and as a bf16 hi/lo pair laid out exactly as the
@@ -39,320 +49,472 @@
 // rows further (hi and lo interleaved by 16-row blocks, so the rows a K-step
 // of the triangular product needs are contiguous), so hi + lo carries ~16
 // significant bits. The output-direction variant (T = L_M^{-1} F, a full
-// matrix) keeps hi in rows 0-127 and lo in rows 128-255.
+// matrix) keeps hi in rows 0-127 and lo in rows 128-255. Both go straight from the
+// tiles' registers.
 #include "jacap_dev.cuh"
 #include "jacap_internal.h"
-#include "k_factor_body.cuh"
 
 namespace jacap {
 
-constexpr int FA_LD = D + 1;
-// PROJ: two padded 128 x 128 float32 matrices (R0: G, then F G, then L^{-1},
-// then the image staging; R1: F); otherwise the staging matrix only.
-template <bool PROJ>
-constexpr size_t factor_smem_bytes() { return (size_t)(PROJ ? 2 : 1) * D * FA_LD * sizeof(float); }
+constexpr int FT_TILES = 272;     // tiles (ty, cx), cx <= 2 ty + 1
+constexpr int FT_THREADS = 288;
 
-template <bool PROJ>
-__global__ void __launch_bounds__(FA_THREADS, PROJ ? 1 : 2)
-    factor_kernel(Dims dm, Ws ws, const float* __restrict__ out_factor) {
-  pdl_wait();
-  extern __shared__ float Ms[];  // [D][FA_LD]: L^{-1} staged for the bf16 image (PROJ: R0, then R1)
-  __shared__ __align__(16) float colA[2][D];
-  __shared__ __align__(16) float rowY[2][D];
-  __shared__ float piv[D];
-  __shared__ int s_skip, s_bad;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    s_skip = status_failed(ws) ? 1 : 0;
-    s_bad = 0;
+// A step's vectors: raw by index, u by component (ut) and negated by row (ur,
+// with 16 bytes between the tile rows, so that a warp's rows fall in different
+// banks).
+struct FtSmem {
+  float4 raw[D];
+  float4 linv[4];
+  float ut[4][D];
+  float4 ur[D + D / 8];
+  int list[FT_THREADS];
+  int cnt[FT_THREADS / 32];
+  int skip;
+};
+
+using Tile = float2[8][2];  // 8 rows of two column pairs
+
+__device__ __forceinline__ float4 tile_row(const Tile& T, int i) { return make_float4(T[i][0].x, T[i][0].y, T[i][1].x, T[i][1].y); }
+__device__ __forceinline__ float& tile_at(Tile& T, int i, int c) {  // i, c known after unrolling
+  return (c & 1) ? T[i][c >> 1].y : T[i][c >> 1].x;
+}
+
+// 1 / sqrt(x): the hardware's approximation refined by one Newton-Raphson step;
+// 1 / x likewise.
+__device__ __forceinline__ float rsqrt_nr(float x) {
+  const float y = rsqrtf(x);
+  return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
+}
+__device__ __forceinline__ float rcp_nr(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return fmaf(y, fmaf(-x, y, 1.f), y);
+}
+
+// L_b^{-1} of the pivot block in rows O .. O + 3 of its tile, to which the 1 of I
+// is added here. The chain from one
+// pivot to the next is a reciprocal, a product and a multiply-add (the block's
+// L D L^T); the square roots follow beside it.
+template <int O>
+__device__ __forceinline__ void pivot_block(Tile& T, FtSmem& sm, bool& bad) {
+  const float d0 = fmaxf(1.f + tile_at(T, O, 0), 1e-30f);
+  const float r0 = rcp_nr(d0);
+  const float a10 = tile_at(T, O + 1, 0), a20 = tile_at(T, O + 2, 0), a30 = tile_at(T, O + 3, 0);
+  const float l10 = a10 * r0, l20 = a20 * r0, l30 = a30 * r0;
+  const float d1 = fmaxf(1.f + fmaf(-l10, a10, tile_at(T, O + 1, 1)), 1e-30f);
+  const float a21 = fmaf(-l20, a10, tile_at(T, O + 2, 1)), a31 = fmaf(-l30, a10, tile_at(T, O + 3, 1));
+  const float r1 = rcp_nr(d1);
+  const float l21 = a21 * r1, l31 = a31 * r1;
+  const float d2 = fmaxf(1.f + fmaf(-l21, a21, fmaf(-l20, a20, tile_at(T, O + 2, 2))), 1e-30f);
+  const float a32 = fmaf(-l31, a21, fmaf(-l30, a20, tile_at(T, O + 3, 2)));
+  const float r2 = rcp_nr(d2);
+  const float l32 = a32 * r2;
+  const float d3 =
+      fmaxf(1.f + fmaf(-l32, a32, fmaf(-l31, a31, fmaf(-l30, a30, tile_at(T, O + 3, 3)))), 1e-30f);
+  // a pivot that is not positive, or not finite, shows here (NaN takes 1e-30 too)
+  bad |= !(fminf(fminf(d0, d1), fminf(d2, d3)) > 1e-30f) || !isfinite(d0) || !isfinite(d1) || !isfinite(d2) || !isfinite(d3);
+  const float i0 = rsqrt_nr(d0), i1 = rsqrt_nr(d1), i2 = rsqrt_nr(d2), i3 = rsqrt_nr(d3);
+  // the inverse of the unit lower factor, rows scaled by D^{-1/2}
+  const float x20 = fmaf(l21, l10, -l20), x31 = fmaf(l32, l21, -l31);
+  const float x30 = fmaf(-l32, x20, fmaf(l31, l10, -l30));
+  sm.linv[0] = make_float4(i0, 0.f, 0.f, 0.f);
+  sm.linv[1] = make_float4(-l10 * i1, i1, 0.f, 0.f);
+  sm.linv[2] = make_float4(x20 * i2, -l21 * i2, i2, 0.f);
+  sm.linv[3] = make_float4(x30 * i3, x31 * i3, -l32 * i3, i3);
+}
+
+template <int O>
+__device__ __forceinline__ void leave_rows(Tile& T, FtSmem& sm, int ty) {
+#pragma unroll
+  for (int i = O; i < O + 4; ++i) {
+    sm.raw[8 * ty + i] = tile_row(T, i);
+    T[i][0] = T[i][1] = make_float2(0.f, 0.f);
   }
-  __syncthreads();
-  if (s_skip) return;
+}
+
+// The vectors of step b = 2 p + H from their owners, and its pivot block.
+template <int H>
+__device__ __forceinline__ void leave_vectors(Tile& T, FtSmem& sm, int p, int ty, int cx, bool& bad) {
+  const int b = 2 * p + H;
+  if (cx == b && ty >= p) {
+    // rows below the block; their part of the block's columns starts from 0
+    if (ty > p) {
+      leave_rows<0>(T, sm, ty);
+      leave_rows<4>(T, sm, ty);
+    } else {
+      pivot_block<4 * H>(T, sm, bad);
+      if (H == 0) leave_rows<4>(T, sm, ty);
+    }
+  } else if (ty == p && cx < b) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      sm.raw[4 * cx + v] = make_float4(tile_at(T, 4 * H, v), tile_at(T, 4 * H + 1, v), tile_at(T, 4 * H + 2, v),
+                                       tile_at(T, 4 * H + 3, v));
+  }
+}
+
+// Rows O .. O + 3 of the tile: Z_rc -= u_r . u_c. The loads of the rows' vectors
+// are in flight together.
+template <int O>
+__device__ __forceinline__ void update_rows(Tile& T, const FtSmem& sm, const float2 (&uc)[4][2], int ty) {
+  float4 a[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) a[i] = sm.ur[9 * ty + O + i];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float x = j == 0 ? a[i].x : (j == 1 ? a[i].y : (j == 2 ? a[i].z : a[i].w));
+#pragma unroll
+      for (int c = 0; c < 2; ++c) T[O + i][c] = __ffma2_rn(make_float2(x, x), uc[j][c], T[O + i][c]);
+    }
+}
+
+template <int H>
+__device__ __forceinline__ void eliminate_step(Tile& T, FtSmem& sm, int p, int ty, int cx, int tid, bool& bad) {
+  const int b = 2 * p + H;
+  named_barrier_sync(1, FT_THREADS);
+  if (tid < D) {
+    const float4 m0 = sm.linv[0], m1 = sm.linv[1], m2 = sm.linv[2], m3 = sm.linv[3];
+    float4 x = sm.raw[tid];
+    const int e = tid - 4 * b;  // in the block: a unit vector
+    if (e >= 0 && e < 4) x = make_float4(e == 0 ? 1.f : 0.f, e == 1 ? 1.f : 0.f, e == 2 ? 1.f : 0.f, e == 3 ? 1.f : 0.f);
+    const float u0 = m0.x * x.x;
+    const float u1 = fmaf(m1.y, x.y, m1.x * x.x);
+    const float u2 = fmaf(m2.z, x.z, fmaf(m2.y, x.y, m2.x * x.x));
+    const float u3 = fmaf(m3.w, x.w, fmaf(m3.z, x.z, fmaf(m3.y, x.y, m3.x * x.x)));
+    sm.ut[0][tid] = u0;
+    sm.ut[1][tid] = u1;
+    sm.ut[2][tid] = u2;
+    sm.ut[3][tid] = u3;
+    sm.ur[tid + (tid >> 3)] = make_float4(-u0, -u1, -u2, -u3);
+  }
+  named_barrier_sync(1, FT_THREADS);
+  if (ty >= p) {
+    float2 uc[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 a = *(const float4*)&sm.ut[j][4 * cx];
+      uc[j][0] = make_float2(a.x, a.y), uc[j][1] = make_float2(a.z, a.w);
+    }
+    if (ty > p) {
+      update_rows<0>(T, sm, uc, ty);
+      update_rows<4>(T, sm, uc, ty);
+    } else {  // the block's rows are final; below it in the tile: rows 4 .. 7 (H == 0)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) T[4 * H + j][0] = uc[j][0], T[4 * H + j][1] = uc[j][1];
+      if (H == 0) update_rows<4>(T, sm, uc, ty);
+    }
+    if (H == 0) leave_vectors<1>(T, sm, p, ty, cx, bad);
+    else if (p < 15) leave_vectors<0>(T, sm, p + 1, ty, cx, bad);
+  }
+}
+
+// T (the tiles of A - I) -> L^{-1}'s, by FT_THREADS threads (the last ones without a tile: ty = -1).
+__device__ __forceinline__ void eliminate(Tile& T, FtSmem& sm, int ty, int cx, int tid, bool& bad) {
+  if (ty >= 0) leave_vectors<0>(T, sm, 0, ty, cx, bad);
+#pragma unroll 1
+  for (int p = 0; p < 16; ++p) {
+    eliminate_step<0>(T, sm, p, ty, cx, tid, bad);
+    eliminate_step<1>(T, sm, p, ty, cx, tid, bad);
+  }
+}
+
+// PROJ: two 128 x 128 float32 matrices, 16-byte rows.
+constexpr int FT_LD = D + 4;
+constexpr size_t FT_PROJ_SMEM = (size_t)2 * D * FT_LD * sizeof(float);
+
+// acc = P Q (row-major, stride FT_LD), 8 x 8 outputs per thread of a 16 x 16 grid:
+// rows 8 ty .., columns 8 tx ..
+using Acc = float2[8][4];
+__device__ __forceinline__ void tile_product(Acc& acc, const float* P, const float* Q, int ty, int tx) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int m = 0; m < D; m += 4) {
+    float2 q[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 a = *(const float4*)(Q + (m + j) * FT_LD + 8 * tx);
+      const float4 b = *(const float4*)(Q + (m + j) * FT_LD + 8 * tx + 4);
+      q[j][0] = make_float2(a.x, a.y), q[j][1] = make_float2(a.z, a.w);
+      q[j][2] = make_float2(b.x, b.y), q[j][3] = make_float2(b.z, b.w);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float4 x = *(const float4*)(P + (8 * ty + i) * FT_LD + m);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        acc[i][c] = __ffma2_rn(make_float2(x.x, x.x), q[0][c], acc[i][c]);
+        acc[i][c] = __ffma2_rn(make_float2(x.y, x.y), q[1][c], acc[i][c]);
+        acc[i][c] = __ffma2_rn(make_float2(x.z, x.z), q[2][c], acc[i][c]);
+        acc[i][c] = __ffma2_rn(make_float2(x.w, x.w), q[3][c], acc[i][c]);
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void store_acc(const Acc& T, float* dst, int ld, int ty, int tx) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float* r = dst + (int64_t)(8 * ty + i) * ld + 8 * tx;
+    *(float4*)r = make_float4(T[i][0].x, T[i][0].y, T[i][1].x, T[i][1].y);
+    *(float4*)(r + 4) = make_float4(T[i][2].x, T[i][2].y, T[i][3].x, T[i][3].y);
+  }
+}
+__device__ __forceinline__ void store_acc_t(const Acc& T, float* dst, int ld, int ty, int tx) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    auto at = [&](int i) { return (c & 1) ? T[i][c >> 1].y : T[i][c >> 1].x; };
+    float* r = dst + (int64_t)(8 * tx + c) * ld + 8 * ty;
+    *(float4*)r = make_float4(at(0), at(1), at(2), at(3));
+    *(float4*)(r + 4) = make_float4(at(4), at(5), at(6), at(7));
+  }
+}
+
+// Four consecutive values of a row as the image's hi and lo (8 bytes each).
+__device__ __forceinline__ void split4(const float4 x, uint2& hi, uint2& lo) {
+  hi.x = pack_bf16x2(x.x, x.y), hi.y = pack_bf16x2(x.z, x.w);
+  lo.x = pack_bf16x2(x.x - bf16lo(hi.x), x.y - bf16hi(hi.x));
+  lo.y = pack_bf16x2(x.z - bf16lo(hi.y), x.w - bf16hi(hi.y));
+}
+// Image offset of channels 4 cx .. + 3 of image row ir.
+__device__ __forceinline__ uint32_t img_off(uint32_t ir, int cx) {
+  return (cx >> 4) * 32768u + sw128_off(ir, (cx & 15) >> 1) + 8u * (cx & 1);
+}
+
+template <bool PROJ, int CTAS>
+__global__ void __launch_bounds__(FT_THREADS, CTAS)
+    factor_kernel(Dims dm, Ws ws, const float* __restrict__ out_factor, int reduced) {
+  pdl_wait();
+  extern __shared__ __align__(16) float fmat[];  // PROJ: R0, R1
+  __shared__ FtSmem sm;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // tile of this thread: tiles 0 .. ty (ty + 1) - 1 lie in the tile rows above ty
+  int ty = (int)((sqrtf(4.f * (float)tid + 1.f) - 1.f) * 0.5f);
+  while (ty * (ty + 1) > tid) --ty;
+  while ((ty + 1) * (ty + 2) <= tid) ++ty;
+  const int cx = tid - ty * (ty + 1);
+  if (tid >= FT_TILES) ty = -1;
+  const bool own = ty >= 0;
   const int u = blockIdx.x;
   const int plane = u / dm.S, s = u % dm.S;
-  const int ch0 = ws.plan[1 + s], ch1 = ws.plan[2 + s];
-  const int ty = tid >> 5, tx = tid & 31;
-  const int c0 = 4 * tx;
+  if (tid == 0) sm.skip = status_failed(ws) ? 1 : 0;
+  const int ch0 = ws.plan[1 + s], ch1 = reduced ? min(ch0 + 1, (int)ws.plan[2 + s]) : (int)ws.plan[2 + s];
+  __syncthreads();
+  if (sm.skip) return;
+  bool bad = false;
 
-  // A = I + sum of partial Grams (chunk order)
-  float2 z[FA_ROWS][2];  // columns (c0, c0+1) and (c0+2, c0+3) as packed pairs
+  // G's tiles: the sum of the unit's partials, in chunk order, straight from
+  // global memory (layout: (m, n) at ((n / 32) D + m) 32 + n % 32)
+  Tile T;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) T[i][0] = T[i][1] = make_float2(0.f, 0.f);
   {
-    const float* gp = ws.gpart + ((int64_t)plane * dm.c_cap) * D * D;
+    const float* gp = ws.gpart + ((int64_t)plane * dm.c_cap) * D * D + ((cx >> 3) * D + 8 * ty) * 32 + (cx & 7) * 4;
+    const int32_t* pf = ws.pflag + (int64_t)plane * dm.c_cap;
+    for (int base = ch0; base < ch1; base += FT_THREADS) {
+      // the chunks that hold a partial (the first one of every run)
+      const int ch = base + tid;
+      const bool has = ch < ch1 && pf[ch] != 0;
+      const uint32_t b = __ballot_sync(0xffffffffu, has);
+      if (lane == 0) sm.cnt[warp] = __popc(b);
+      __syncthreads();
+      int at = 0, n = 0;
+#pragma unroll
+      for (int w = 0; w < FT_THREADS / 32; ++w) {
+        if (w < warp) at += sm.cnt[w];
+        n += sm.cnt[w];
+      }
+      if (has) sm.list[at + __popc(b & ((1u << lane) - 1u))] = ch;
+      __syncthreads();
+      if (own)
+        for (int k = 0; k < n; ++k) {
+          const float* src = gp + (int64_t)sm.list[k] * D * D;
+          float4 v[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = *(const float4*)(src + i * 32);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            T[i][0].x += v[i].x, T[i][0].y += v[i].y;
+            T[i][1].x += v[i].z, T[i][1].y += v[i].w;
+          }
+        }
+      __syncthreads();  // the list is read before the next round writes it
+    }
+  }
+  // G, both triangles (a diagonal tile's part above the diagonal is there as it is)
+  if (own) {
     float* gout = ws.gram + (int64_t)u * D * D;
 #pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a) z[a][0] = z[a][1] = make_float2(0.f, 0.f);
-    const int32_t* pf = ws.pflag + (int64_t)plane * dm.c_cap;
-    for (int ch = ch0; ch < ch1; ++ch) {  // 16 independent 16-byte loads in flight per chunk
-      if (!pf[ch]) continue;  // no partial at this chunk (it continued a run)
-      // partial layout: (m, n) at ((n / 32) D + m) 32 + n % 32; only the
-      // lower 32 x 32 blocks are stored (rows ty + 8 a lie in block a / 4)
-      const float* src = gp + (int64_t)ch * D * D + (c0 >> 5) * D * 32 + (c0 & 31);
+    for (int i = 0; i < 8; ++i) *(float4*)(gout + (8 * ty + i) * D + 4 * cx) = tile_row(T, i);
+    if (cx < 2 * ty) {
 #pragma unroll
-      for (int a = 0; a < FA_ROWS; ++a) {
-        if (a / 4 < (c0 >> 5)) continue;
-        const float4 v = *(const float4*)(src + (ty + 8 * a) * 32);
-        z[a][0].x += v.x;
-        z[a][0].y += v.y;
-        z[a][1].x += v.z;
-        z[a][1].y += v.w;
+      for (int c = 0; c < 4; ++c) {
+        float* r = gout + (4 * cx + c) * D + 8 * ty;
+        *(float4*)r = make_float4(tile_at(T, 0, c), tile_at(T, 1, c), tile_at(T, 2, c), tile_at(T, 3, c));
+        *(float4*)(r + 4) = make_float4(tile_at(T, 4, c), tile_at(T, 5, c), tile_at(T, 6, c), tile_at(T, 7, c));
       }
     }
-    // the upper blocks by symmetry, through the staging matrix
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a) {
-      const int i = ty + 8 * a;
-      if (a / 4 < (c0 >> 5)) continue;
-      Ms[i * FA_LD + c0] = z[a][0].x;
-      Ms[i * FA_LD + c0 + 1] = z[a][0].y;
-      Ms[i * FA_LD + c0 + 2] = z[a][1].x;
-      Ms[i * FA_LD + c0 + 3] = z[a][1].y;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a) {
-      const int i = ty + 8 * a;
-      if (a / 4 < (c0 >> 5))
-        z[a][0] = make_float2(Ms[c0 * FA_LD + i], Ms[(c0 + 1) * FA_LD + i]),
-        z[a][1] = make_float2(Ms[(c0 + 2) * FA_LD + i], Ms[(c0 + 3) * FA_LD + i]);
-      *(float4*)(gout + i * D + c0) = make_float4(z[a][0].x, z[a][0].y, z[a][1].x, z[a][1].y);
-    }
-    __syncthreads();
   }
+  float *R0 = fmat, *R1 = fmat + D * FT_LD;
+  const int py = tid >> 4, px = tid & 15;  // the products' grid (threads 0-255)
   if constexpr (PROJ) {
-    // M = F G F^T: G and F to shared memory (stride FA_LD), then two products
-    // with thread (ty, tx) computing rows ty + 8 a, columns tx + 32 b
-    float* R0 = Ms;
-    float* R1 = Ms + D * FA_LD;
+    // M = F G F^T: (F G)^T to R0, then M = F (F G)^T (M is symmetric), to R0
     const float* F = out_factor + (int64_t)plane * D * D;
+    if (own) {
 #pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a) {
-      const int i = ty + 8 * a;
-      R0[i * FA_LD + c0] = z[a][0].x;
-      R0[i * FA_LD + c0 + 1] = z[a][0].y;
-      R0[i * FA_LD + c0 + 2] = z[a][1].x;
-      R0[i * FA_LD + c0 + 3] = z[a][1].y;
-    }
-    for (int e = tid; e < D * D / 4; e += FA_THREADS) {
-      const float4 f = ((const float4*)F)[e];
-      const int r = e / (D / 4), c = (e % (D / 4)) * 4;
-      R1[r * FA_LD + c] = f.x;
-      R1[r * FA_LD + c + 1] = f.y;
-      R1[r * FA_LD + c + 2] = f.z;
-      R1[r * FA_LD + c + 3] = f.w;
-    }
-    __syncthreads();
-    float acc[FA_ROWS][4];
-    // T1 = F G: T1[i][c] = sum_m F[i][m] G[m][c]
+      for (int i = 0; i < 8; ++i) *(float4*)(R0 + (8 * ty + i) * FT_LD + 4 * cx) = tile_row(T, i);
+      if (cx < 2 * ty) {
 #pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-#pragma unroll 2
-    for (int m = 0; m < D; ++m) {
-      float g[4];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) g[b] = R0[m * FA_LD + tx + 32 * b];
-#pragma unroll
-      for (int a = 0; a < FA_ROWS; ++a) {
-        const float f = R1[(ty + 8 * a) * FA_LD + m];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(f, g[b], acc[a][b]);
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) R0[(ty + 8 * a) * FA_LD + tx + 32 * b] = acc[a][b];
-    __syncthreads();
-    // M = T1 F^T: M[i][c] = sum_m T1[i][m] F[c][m]
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-#pragma unroll 2
-    for (int m = 0; m < D; ++m) {
-      float f[4];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) f[b] = R1[(tx + 32 * b) * FA_LD + m];
-#pragma unroll
-      for (int a = 0; a < FA_ROWS; ++a) {
-        const float t = R0[(ty + 8 * a) * FA_LD + m];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(t, f[b], acc[a][b]);
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) R0[(ty + 8 * a) * FA_LD + tx + 32 * b] = acc[a][b];
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a) {
-      const int i = ty + 8 * a;
-      z[a][0] = make_float2(R0[i * FA_LD + c0], R0[i * FA_LD + c0 + 1]);
-      z[a][1] = make_float2(R0[i * FA_LD + c0 + 2], R0[i * FA_LD + c0 + 3]);
-    }
-    __syncthreads();
-  }
-  {
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a) {
-      const int i = ty + 8 * a;
-      z[a][0].x += (i == c0 ? 1.f : 0.f);
-      z[a][0].y += (i == c0 + 1 ? 1.f : 0.f);
-      z[a][1].x += (i == c0 + 2 ? 1.f : 0.f);
-      z[a][1].y += (i == c0 + 3 ? 1.f : 0.f);
-    }
-  }
-
-  // forward elimination, step j = 8 jh + jl (jl unrolled so the register
-  // column of the pivot column is a compile-time constant)
-#pragma unroll 1
-  for (int jh = 0; jh < 16; ++jh) {
-#pragma unroll
-    for (int jl = 0; jl < 8; ++jl) {
-      const int j = 8 * jh + jl;
-      const int buf = j & 1;
-      if (tx == (j >> 2)) {  // owners of column j: rows ty + 8 a, register column j % 4 = jl % 4
-#pragma unroll
-        for (int a = 0; a < FA_ROWS; ++a) {
-          const float2 zp = z[a][(jl & 3) >> 1];
-          colA[buf][ty + 8 * a] = (jl & 1) ? zp.y : zp.x;
-        }
-      }
-      if (ty == jl) {  // owners of row j (register row jh)
-        float2 r01 = make_float2(0.f, 0.f), r23 = r01;
-#pragma unroll
-        for (int a = 0; a < FA_ROWS; ++a)
-          if (a == jh) {
-            r01 = z[a][0];
-            r23 = z[a][1];
-          }
-        *(float4*)&rowY[buf][c0] = make_float4(r01.x, r01.y, r23.x, r23.y);
-      }
-      __syncthreads();
-      const float pj = colA[buf][j];
-      if (tid == 0) piv[j] = pj;
-      const float inv_p = recip_nr(pj);
-      const float4 ca = *(const float4*)&colA[buf][c0];
-      const float4 ry = *(const float4*)&rowY[buf][c0];
-      const float cav[4] = {ca.x, ca.y, ca.z, ca.w}, ryv[4] = {ry.x, ry.y, ry.z, ry.w};
-      float r[4];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) r[b] = c0 + b > j ? cav[b] : (c0 + b == j ? 0.f : ryv[b]);
-      const float2 r01 = make_float2(r[0], r[1]), r23 = make_float2(r[2], r[3]);
-#pragma unroll
-      for (int a = 0; a < FA_ROWS; ++a) {
-        if (ty + 8 * a > j) {  // active rows (uniform over the warp)
-          const float m = colA[buf][ty + 8 * a] * inv_p;
-          const float2 nm = make_float2(-m, -m);
-          z[a][0] = __ffma2_rn(nm, r01, z[a][0]);
-          z[a][1] = __ffma2_rn(nm, r23, z[a][1]);
+        for (int c = 0; c < 4; ++c) {
+          float* r = R0 + (4 * cx + c) * FT_LD + 8 * ty;
+          *(float4*)r = make_float4(tile_at(T, 0, c), tile_at(T, 1, c), tile_at(T, 2, c), tile_at(T, 3, c));
+          *(float4*)(r + 4) = make_float4(tile_at(T, 4, c), tile_at(T, 5, c), tile_at(T, 6, c), tile_at(T, 7, c));
         }
       }
     }
+    for (int e = tid; e < D * D / 4; e += FT_THREADS)
+      *(float4*)(R1 + (e >> 5) * FT_LD + (e & 31) * 4) = ((const float4*)F)[e];
+    Acc acc;
+    __syncthreads();
+    if (tid < 256) tile_product(acc, R1, R0, py, px);
+    __syncthreads();
+    if (tid < 256) store_acc_t(acc, R0, FT_LD, py, px);
+    __syncthreads();
+    if (tid < 256) tile_product(acc, R1, R0, py, px);
+    __syncthreads();
+    if (tid < 256) store_acc(acc, R0, FT_LD, py, px);
+    __syncthreads();
+    if (own) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 v = *(const float4*)(R0 + (8 * ty + i) * FT_LD + 4 * cx);
+        T[i][0] = make_float2(v.x, v.y), T[i][1] = make_float2(v.z, v.w);
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
-
-  // L^{-1}_ic = X_ic / sqrt(p_i) with X_ic = -Y_ic / p_c (c < i), X_ii = 1
+  eliminate(T, sm, ty, cx, tid, bad);
+  if (own && cx >= 2 * ty) {  // zeros above the diagonal
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (4 * (cx - 2 * ty) + c > i) tile_at(T, i, c) = 0.f;
+  }
   float* mout = ws.minv + (int64_t)u * D * D;
-  float ipc[4];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) ipc[b] = 1.f / piv[c0 + b];
-#pragma unroll
-  for (int a = 0; a < FA_ROWS; ++a) {
-    const int i = ty + 8 * a;
-    const float d = piv[i];
-    if (!(d > 0.f) || !isfinite(d)) s_bad = 1;
-    const float sc = 1.f / sqrtf(fmaxf(d, 1e-30f));
-    const float zv[4] = {z[a][0].x, z[a][0].y, z[a][1].x, z[a][1].y};
-    float x[4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = c0 + b;
-      x[b] = c < i ? (-zv[b] * ipc[b]) * sc : (c == i ? sc : 0.f);
-      if (!isfinite(x[b])) s_bad = 1;
-      Ms[i * FA_LD + c] = x[b];
-    }
-    if constexpr (!PROJ) *(float4*)(mout + i * D + c0) = make_float4(x[0], x[1], x[2], x[3]);
-  }
-  __syncthreads();
-  if constexpr (PROJ) {
-    // T = L_M^{-1} F: T[i][c] = sum_{m <= i} L^{-1}[i][m] F[m][c] (L^{-1} now in R0 = Ms)
-    const float* R1 = Ms + D * FA_LD;
-    float acc[FA_ROWS][4];
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-#pragma unroll 2
-    for (int m = 0; m < D; ++m) {
-      float f[4];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) f[b] = R1[m * FA_LD + tx + 32 * b];
-#pragma unroll
-      for (int a = 0; a < FA_ROWS; ++a) {
-        const float l = Ms[(ty + 8 * a) * FA_LD + m];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(l, f[b], acc[a][b]);
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < FA_ROWS; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int i = ty + 8 * a, c = tx + 32 * b;
-        if (!isfinite(acc[a][b])) s_bad = 1;
-        Ms[i * FA_LD + c] = acc[a][b];
-        mout[i * D + c] = acc[a][b];
-      }
-    __syncthreads();
-  }
-  // bf16 hi/lo image: 2 K-atoms (channels 0-63, 64-127) x 256 rows x 128 B
   uint8_t* img = ws.minv_img + (int64_t)u * 65536;
-  for (int e = tid; e < 256 * 16; e += FA_THREADS) {
-    const int n = e / 16, cc = e % 16;  // row n, 8-channel chunk cc
-    const int r = n & 127;
-    const bool lo = n >= 128;
-    uint32_t wv[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float x0 = Ms[r * FA_LD + cc * 8 + 2 * q];
-      const float x1 = Ms[r * FA_LD + cc * 8 + 2 * q + 1];
-      const uint32_t h = pack_bf16x2(x0, x1);
-      wv[q] = lo ? pack_bf16x2(x0 - bf16lo(h), x1 - bf16hi(h)) : h;
+  if constexpr (PROJ) {  // T = L_M^{-1} F
+    for (int e = tid; e < D * D / 4; e += FT_THREADS) {  // the tiles above the diagonal
+      const int r = e >> 5, c4 = e & 31;
+      if (c4 > 2 * (r >> 3) + 1) *(float4*)(R0 + r * FT_LD + 4 * c4) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const uint32_t off = (cc >> 3) * 32768 + sw128_off(n, cc & 7);
-    *(uint4*)(img + off) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+    if (own) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) *(float4*)(R0 + (8 * ty + i) * FT_LD + 4 * cx) = tile_row(T, i);
+    }
+    __syncthreads();
+    if (tid < 256) {
+      Acc acc;
+      tile_product(acc, R0, R1, py, px);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t n = 8 * py + i;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float4 x = make_float4(acc[i][2 * h].x, acc[i][2 * h].y, acc[i][2 * h + 1].x, acc[i][2 * h + 1].y);
+          bad |= !isfinite(x.x) || !isfinite(x.y) || !isfinite(x.z) || !isfinite(x.w);
+          *(float4*)(mout + n * D + 8 * px + 4 * h) = x;
+          uint2 hi, lo;
+          split4(x, hi, lo);
+          *(uint2*)(img + img_off(n, 2 * px + h)) = hi;
+          *(uint2*)(img + img_off(n + 128, 2 * px + h)) = lo;
+        }
+      }
+    }
+  } else {
+    if (own) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t n = 8 * ty + i;
+        const float4 x = tile_row(T, i);
+        bad |= !isfinite(x.x) || !isfinite(x.y) || !isfinite(x.z) || !isfinite(x.w);
+        *(float4*)(mout + n * D + 4 * cx) = x;
+        uint2 hi, lo;
+        split4(x, hi, lo);
+        const uint32_t ir = 32 * (n >> 4) + (n & 15);
+        *(uint2*)(img + img_off(ir, cx)) = hi;
+        *(uint2*)(img + img_off(ir + 16, cx)) = lo;
+      }
+    }
+    // zeros: float32 above the tiles; in the image the score pass reads row n up
+    // to channel 16 (n / 16) + 15, so only the tile pair right of an even tile row
+    for (int e = tid; e < D * D / 4; e += FT_THREADS) {
+      const int r = e >> 5, c4 = e & 31, t = r >> 3;
+      if (c4 <= 2 * t + 1) continue;
+      *(float4*)(mout + r * D + 4 * c4) = make_float4(0.f, 0.f, 0.f, 0.f);
+      if ((t & 1) == 0 && c4 <= 2 * t + 3) {
+        const uint32_t ir = 32 * (r >> 4) + (r & 15);
+        *(uint2*)(img + img_off(ir, c4)) = make_uint2(0u, 0u);
+        *(uint2*)(img + img_off(ir + 16, c4)) = make_uint2(0u, 0u);
+      }
+    }
   }
-  __syncthreads();
-  if (tid == 0 && s_bad) flag(ws, ST_NONFINITE);
+  if (bad) flag(ws, ST_NONFINITE);
 }
 
-__global__ void __launch_bounds__(FB_THREADS, 2) factor_blocked_kernel(Dims dm, Ws ws) {
+// The partials of each unit summed into the first one (at its first chunk), by
+// one CTA per unit and lower 32 x 32 block: for a few units with many partials,
+// which the factor's one CTA per unit would add one after the other (~0.6 us each;
+// this launch costs about 4 us, hence from six partials on).
+constexpr int FR_THREADS = 256;
+__global__ void __launch_bounds__(FR_THREADS) gram_reduce_kernel(Dims dm, Ws ws) {
   pdl_wait();
-  factor_blocked_cta<false>(dm, ws, blockIdx.x, gridDim.x);
+  __shared__ int s_skip;
+  const int tid = threadIdx.x;
+  if (tid == 0) s_skip = status_failed(ws) ? 1 : 0;
+  const int u = blockIdx.x / 10, blk = blockIdx.x % 10;
+  const int nb = blk < 4 ? 0 : (blk < 7 ? 1 : (blk < 9 ? 2 : 3));             // column block
+  const int I = nb + blk - (nb == 0 ? 0 : (nb == 1 ? 4 : (nb == 2 ? 7 : 9)));  // row block >= nb
+  const int plane = u / dm.S, s = u % dm.S;
+  const int ch0 = ws.plan[1 + s], ch1 = ws.plan[2 + s];
+  __syncthreads();
+  if (s_skip || ch0 >= ch1) return;
+  float* gp = ws.gpart + ((int64_t)plane * dm.c_cap) * D * D + (nb * D + 32 * I) * 32 + 4 * tid;
+  const int32_t* pf = ws.pflag + (int64_t)plane * dm.c_cap;
+  float4 acc = *(const float4*)(gp + (int64_t)ch0 * D * D);
+  constexpr int N = 8;  // loads in flight
+  for (int c = ch0 + 1; c < ch1; c += N) {
+    float4 v[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c + k < ch1 && pf[c + k] != 0) v[k] = *(const float4*)(gp + (int64_t)(c + k) * D * D);
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) acc.x += v[k].x, acc.y += v[k].y, acc.z += v[k].z, acc.w += v[k].w;
+  }
+  *(float4*)(gp + (int64_t)ch0 * D * D) = acc;
 }
 
-template <bool PROJ>
-static cudaError_t launch_factor_t(const Dims& dm, const Ws& ws, const float* out_factor, cudaStream_t st) {
-  constexpr size_t smem = factor_smem_bytes<PROJ>();
-  cudaError_t e = cudaFuncSetAttribute(factor_kernel<PROJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_factor(const Dims& dm, const Ws& ws, const float* out_factor, int partials, int sms,
+                          cudaStream_t st) {
   const int units = dm.L * dm.Hkv * dm.S;
-  JACAP_TRY(launch_pdl(dm.pdl != 0, factor_kernel<PROJ>, units, FA_THREADS, smem, st, dm, ws, out_factor));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_factor(const Dims& dm, const Ws& ws, const float* out_factor, cudaStream_t st) {
-  if (out_factor != nullptr) return launch_factor_t<true>(dm, ws, out_factor, st);
-  cudaError_t e = cudaFuncSetAttribute(factor_blocked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)FB_SMEM);
-  if (e != cudaSuccess) return e;
-  JACAP_TRY(launch_pdl(dm.pdl != 0, factor_blocked_kernel, dm.L * dm.Hkv * dm.S, FB_THREADS, FB_SMEM, st, dm, ws));
+  const int reduced = partials >= 6 ? 1 : 0;
+  if (reduced) JACAP_TRY(launch_pdl(dm.pdl != 0, gram_reduce_kernel, units * 10, FR_THREADS, 0, st, dm, ws));
+  if (out_factor != nullptr) {
+    auto kern = factor_kernel<true, 1>;
+    JACAP_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FT_PROJ_SMEM));
+    JACAP_TRY(launch_pdl(dm.pdl != 0, kern, units, FT_THREADS, FT_PROJ_SMEM, st, dm, ws, out_factor, reduced));
+  } else {
+    // three CTAs per SM (72 registers a thread) finish 17 % more units in the
+    // same time than two (96), but each later: worth it beyond one wave of two
+    auto kern = units > 2 * sms ? factor_kernel<false, 3> : factor_kernel<false, 2>;
+    JACAP_TRY(launch_pdl(dm.pdl != 0, kern, units, FT_THREADS, 0, st, dm, ws, out_factor, reduced));
+  }
   return cudaGetLastError();
 }
 

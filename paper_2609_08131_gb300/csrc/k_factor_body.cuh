@@ -1,6 +1,7 @@
-// k_factor_body.cuh - the blocked factor as a device function: the kernel
-// of k_factor.cu and the factor role of the fused schedule (k_fused.cu)
-// both run it. See k_factor.cu for what it computes.
+// k_factor_body.cuh - the factor role of the fused schedule (k_fused.cu); see
+// k_factor.cu for what it computes. The fused kernel's threads have 96 registers
+// and its CTA five stages of shared memory for the partials, so this one keeps the
+// matrix in shared memory (the kernel of k_factor.cu keeps it in registers).
 #pragma once
 
 #include "jacap_dev.cuh"
@@ -19,8 +20,7 @@ __device__ __forceinline__ float recip_nr(float p) {
 // ------------------------------------------------------------ blocked ------
 // The proxy path (u = v) factors A with a blocked right-looking Cholesky on
 // 32 x 32 blocks (I, J = 0..3) and inverts the factor blockwise, so the
-// sequential part is four 32-step eliminations inside one warp instead of
-// 128 block-wide steps:
+// sequential part is four 32-step eliminations inside one warp:
 //  for K = 0..3:
 //    T_KK = L_KK^{-1}   one warp: the forward elimination above on the 32 x 32
 //                       block A_KK (its lower triangle), X_KK -> T_KK
@@ -43,23 +43,16 @@ constexpr int FB_BLK = 32 * FB_LD;    // floats per block
 // XT (XT_JI at tri(I, J); S_IJ^T there until X_IJ replaces it)
 // 10 lower blocks of A and 10 of XT, then the elimination's buffers (192 floats)
 constexpr int FB_ELIM = 192;
-constexpr size_t FB_SMEM = ((size_t)20 * FB_BLK + FB_ELIM) * sizeof(float);
 
 __device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }  // block (i, j), j <= i
 // a partial Gram's lower blocks staged in shared memory: column block nb,
 // rows 32 nb .. 127, 32 floats per row, after the segments of blocks < nb
 __host__ __device__ constexpr int fb_seg(int nb) { return 32 * (128 * nb - 16 * nb * (nb - 1)); }
 constexpr int FB_STAGE = fb_seg(4);  // floats per stage (10 blocks of 32 x 32)
-static_assert(2 * FB_STAGE <= 20 * FB_BLK, "the staging ring fits in the A and XT blocks");
-// partials in flight: 2 in the factor kernel (two CTAs per SM), 5 in the fused
-// schedule's factor role (one CTA per SM, the shared memory of the Gram role)
-template <bool FUSED> __host__ __device__ constexpr int fb_stages() { return FUSED ? 5 : 2; }
+constexpr int FB_STAGES = 5;  // partials in flight (one CTA per SM, the shared memory of the Gram role)
 // floats before the elimination buffers: the A and XT blocks, or the staging ring if that is longer
-template <bool FUSED> __host__ __device__ constexpr int fb_elim_at() {
-  return 20 * FB_BLK > fb_stages<FUSED>() * FB_STAGE ? 20 * FB_BLK : fb_stages<FUSED>() * FB_STAGE;
-}
-static_assert(fb_elim_at<false>() == 20 * FB_BLK, "the factor kernel's shared memory");
-constexpr size_t FB_FUSED_SMEM = ((size_t)fb_elim_at<true>() + FB_ELIM) * sizeof(float);
+constexpr int FB_ELIM_AT = 20 * FB_BLK > FB_STAGES * FB_STAGE ? 20 * FB_BLK : FB_STAGES * FB_STAGE;
+constexpr size_t FB_FUSED_SMEM = ((size_t)FB_ELIM_AT + FB_ELIM) * sizeof(float);
 
 // The barrier of the factor's FB_THREADS threads (named barrier 1: in the
 // fused schedule the factor runs on the first FB_THREADS threads of a larger CTA).
@@ -304,18 +297,16 @@ __device__ __forceinline__ void inv_accumulate(float* As, float* XT, int P, int 
 
 // Units first, first + stride, ... of the CTA, one after the other, by its
 // first FB_THREADS threads (further threads of the CTA must not call this).
-// FUSED: the role of the fused schedule (k_fused.cu): each unit waits until
-// the Gram role has completed it (6 progress counts per chunk), reads the
-// partials with the L2 evict_first policy, and is published (fdone) once
-// G, L^{-1} and the image are visible device-wide.
-template <bool FUSED>
+// Each unit waits until the Gram role has completed it (6 progress counts per
+// chunk), reads the partials with the L2 evict_first policy, and is published
+// (fdone) once G, L^{-1} and the image are visible device-wide.
 __device__ __forceinline__ void factor_blocked_cta(const Dims& dm, const Ws& ws, int first, int stride) {
   extern __shared__ __align__(16) float fsm[];
   float* As = fsm;                // tri(I, J): A_IJ, then L_IJ (I > J) / T_II (I == J)
   float* XT = fsm + 10 * FB_BLK;  // tri(I, J): XT_JI = (L^{-1})_IJ^T
-  constexpr int NST = fb_stages<FUSED>();
+  constexpr int NST = FB_STAGES;
   __shared__ __align__(8) uint64_t s_full[NST];
-  float* s_elim = fsm + fb_elim_at<FUSED>();  // the elimination's row and column buffers, pivots, reciprocals
+  float* s_elim = fsm + FB_ELIM_AT;  // the elimination's row and column buffers, pivots, reciprocals
   __shared__ int s_skip, s_bad, s_np;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -327,7 +318,7 @@ __device__ __forceinline__ void factor_blocked_cta(const Dims& dm, const Ws& ws,
   if (s_skip) return;
   const int units = dm.L * dm.Hkv * dm.S;
   uint32_t kk = 0;  // partial stages consumed so far (phases of s_full across units)
-  const uint64_t drop = FUSED ? policy_evict_first() : 0;
+  const uint64_t drop = policy_evict_first();
   // time accounting (trace builds, thread 0, the elimination warp): 0 the
   // partial Grams summed into A (and G stored), 1-4 the eliminations of the
   // diagonal blocks, 5 its waits for the other warps after them, 6 panels and
@@ -347,7 +338,7 @@ __device__ __forceinline__ void factor_blocked_cta(const Dims& dm, const Ws& ws,
 
   // A = I + sum of the unit's partial Grams (chunk order) over the lower
   // 32 x 32 blocks (the partials hold only those); G to the workspace and the lower blocks of
-  // A to shared memory. The partials stream through a two-stage ring of bulk
+  // A to shared memory. The partials stream through a ring of bulk
   // copies (the 4 lower segments of one partial per stage: rows 32 nb .. 127
   // of column block nb, contiguous in the partial layout) while the threads
   // add the previous stage. Thread (ty, tx) sums rows ty + 8 a, columns
@@ -358,11 +349,10 @@ __device__ __forceinline__ void factor_blocked_cta(const Dims& dm, const Ws& ws,
     const int32_t* pf = ws.pflag + (int64_t)plane * dm.c_cap;
     if (tid == 0) {
       int np = 0;
-      if (FUSED) {  // every item of the unit has stored its weights and partial
-        if (wait_count(ws.gcount + u, 6 * (ch1 - ch0), ws, nullptr)) fence_proxy_async_global();
-        else np = -1;
-        JACAP_TRACE_MAX(ws, u, TR_FAC0);
-      }
+      // every item of the unit has stored its weights and partial
+      if (wait_count(ws.gcount + u, 6 * (ch1 - ch0), ws, nullptr)) fence_proxy_async_global();
+      else np = -1;
+      JACAP_TRACE_MAX(ws, u, TR_FAC0);
       if (np == 0)
         for (int ch = ch0; ch < ch1; ++ch) np += pf[ch] != 0;
       s_np = np;
@@ -384,8 +374,7 @@ __device__ __forceinline__ void factor_blocked_cta(const Dims& dm, const Ws& ws,
       for (int nb = 0; nb < 4; ++nb) {
         const uint32_t sd = smem_u32(dst + fb_seg(nb) * 4), bytes = (D - 32 * nb) * 32 * 4;
         const float* sp = src + (nb * D + 32 * nb) * 32;
-        if (FUSED) bulk_g2s_hint(sd, sp, bytes, smem_u32(&s_full[st]), drop);
-        else bulk_g2s(sd, sp, bytes, smem_u32(&s_full[st]));
+        bulk_g2s_hint(sd, sp, bytes, smem_u32(&s_full[st]), drop);
       }
     };
     if (tid == 0) {
@@ -565,14 +554,13 @@ __device__ __forceinline__ void factor_blocked_cta(const Dims& dm, const Ws& ws,
   }
   kk += (uint32_t)unit_np;
   if (tid == 0 && s_bad) flag(ws, ST_NONFINITE);
-  if (FUSED) {  // G, L^{-1} and the image are visible device-wide: publish the unit
-    fence_proxy_async_global();
-    __threadfence();
-    fb_all();
-    if (tid == 0) {
-      st_release_gpu(ws.fdone + u, 1);
-      JACAP_TRACE_MAX(ws, u, TR_FAC1);
-    }
+  // G, L^{-1} and the image are visible device-wide: publish the unit
+  fence_proxy_async_global();
+  __threadfence();
+  fb_all();
+  if (tid == 0) {
+    st_release_gpu(ws.fdone + u, 1);
+    JACAP_TRACE_MAX(ws, u, TR_FAC1);
   }
   TRC_ADD(8, tr_o);
   TRC_ADD(10, tr_unit);

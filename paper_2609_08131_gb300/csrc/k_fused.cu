@@ -40,7 +40,6 @@ constexpr int FU_THREADS = GR_THREADS;
 template <int G>
 constexpr size_t fused_smem_bytes() {
   constexpr size_t a = GrCfg<G, 1024>::SMEM, b = score_bf16_smem_bytes<false>(), c = FB_FUSED_SMEM;
-  static_assert(FB_SMEM <= FB_FUSED_SMEM, "the factor's blocks fit in its staging ring");
   return a > b ? (a > c ? a : c) : (b > c ? b : c);
 }
 
@@ -51,7 +50,7 @@ __global__ void __launch_bounds__(FU_THREADS, 1)
   pdl_wait();
   const int b = blockIdx.x;
   if (b < nf) {
-    if (threadIdx.x < FB_THREADS) factor_blocked_cta<true>(dm, ws, b, nf);
+    if (threadIdx.x < FB_THREADS) factor_blocked_cta(dm, ws, b, nf);
   } else if (b < nf + ng) {
     gram_bf16_body<G, true>(&vmap, dm, ws, b - nf, ng);
   } else {

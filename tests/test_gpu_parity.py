@@ -554,3 +554,26 @@ def test_packed_requests_score_as_each_request_alone(layers, lens):
                     wl.budget)
         got, ref = ev.scores[:, :, cu[s]:cu[s + 1]].double(), one.scores.double()
         assert bool(((got - ref).abs() <= 2e-5 * ref).all())
+
+
+@pytest.mark.parametrize("layers, hkv, lens, tau", [
+    (1, 2, (20000,), 10.0),          # a few units of many partial Grams, summed by the launch before
+    (1, 2, (20000,), 0.2),           # ... with a Gram far from 0
+    (1, 1, (1, 0, 3, 130), 0.2),     # units of few tokens, one without any
+    (20, 8, (300, 129), 1.0),        # more units than two CTAs per SM hold at once
+])
+def test_factor_inverts_the_capacity_matrix(layers, hkv, lens, tau):
+    """X = L^{-1} as the factor writes it against A = I + G (G as it summed it): X A X^T = I within
+    the bound of a backward stable factor and triangular inverse, 4 n 2^-24 cond(A) with n = 128,
+    and X is lower triangular with zeros above. (The factor reads G's lower triangle; within a
+    diagonal tile the products v_a (w v_b) of the other one are rounded on the other side.)"""
+    wl = Workload("t", layers, 4 * hkv, hkv, lens, 16, 16, seed=91)
+    t = generate(wl, "cuda")
+    ev = evict(make_cache(t, wl), wl.budget, jacap_params(tau=tau))
+    x = ev.intermediates()
+    G, X = x["gram"].double(), x["chol_inv"].double()
+    assert bool((X.triu(1) == 0).all())
+    A = G.tril() + G.tril(-1).mT + torch.eye(128, dtype=torch.float64, device="cuda")
+    cond = torch.linalg.cond(A)
+    err = (X @ A @ X.mT - torch.eye(128, dtype=torch.float64, device="cuda")).abs().amax((-2, -1))
+    assert bool((err <= 4 * 128 * 2.0 ** -24 * cond).all()), (err / cond).max()
