@@ -495,7 +495,8 @@ jacap_status score_pass(const jacap_layout* layout, const jacap_params* params, 
   if ((st = hook(4)) != JACAP_OK ||
       (st = map_cuda(launch_gram(vmap, dm, w, dt, v, cu, persistent_grid(items, sms, bf ? 1 : 4), s))) != JACAP_OK)
     return st;
-  if ((st = hook(5)) != JACAP_OK || (st = map_cuda(launch_factor(dm, w, out_factor, partials_per_unit(dm, items, sms, bf), sms, s))) != JACAP_OK)
+  if ((st = hook(5)) != JACAP_OK ||
+      (st = map_cuda(launch_factor(dm, w, out_factor, partials_per_unit(dm, items, sms, bf), sms, s))) != JACAP_OK)
     return st;
   if ((st = hook(6)) != JACAP_OK ||
       (st = map_cuda(launch_score(vmap, dm, w, dt, v, cu, scores, persistent_grid(items, sms, bf ? 1 : 2), s))) !=
@@ -601,17 +602,15 @@ jacap_status jacap_select_compact_inplace(const jacap_layout* layout, const floa
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   const Ws w = make_ws(ws, c);
-  const int64_t units = (int64_t)dm.L * dm.Hkv * dm.S;
   const int dt = layout->dtype == JACAP_BF16 ? 1 : 0;
   const cudaStream_t s = (cudaStream_t)stream;
   const TraceRange trace("jacap/select_compact_inplace");
   if (!preserve_order)  // hole filling inside the selection kernel
-    return map_cuda(launch_select(dm, w, layout->cu_seqlens, scores, budget, idx, kept, layout->max_seqlen,
-                                  persistent_grid(units, sms, 2), s, dt, nullptr, nullptr, nullptr, nullptr, k, v,
-                                  pos));
+    return map_cuda(launch_select(dm, w, layout->cu_seqlens, scores, budget, idx, kept, layout->max_seqlen, s,
+                                  dt, nullptr, nullptr, nullptr, nullptr, k, v, pos));
   // ascending order moves every kept row: its own launch after the selection
-  if ((st = map_cuda(launch_select(dm, w, layout->cu_seqlens, scores, budget, idx, kept, layout->max_seqlen,
-                                   persistent_grid(units, sms, 2), s))) != JACAP_OK)
+  if ((st = map_cuda(launch_select(dm, w, layout->cu_seqlens, scores, budget, idx, kept, layout->max_seqlen, s))) !=
+      JACAP_OK)
     return st;
   return map_cuda(launch_compact_inplace(dm, w, dt, layout->cu_seqlens, k, v, pos, idx, budget, 1, s));
 }
@@ -631,10 +630,9 @@ jacap_status jacap_select(const jacap_layout* layout, const float* scores, int32
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   const Ws w = make_ws(ws, c);
-  const int64_t units = (int64_t)dm.L * dm.Hkv * dm.S;
   const TraceRange trace("jacap/select");
   return map_cuda(launch_select(dm, w, layout->cu_seqlens, scores, budget, idx, kept, layout->max_seqlen,
-                                persistent_grid(units, sms, 2), (cudaStream_t)stream));
+                                (cudaStream_t)stream));
 }
 
 jacap_status jacap_select_compact(const jacap_layout* layout, const float* scores, int32_t budget, int32_t* idx,
@@ -655,11 +653,9 @@ jacap_status jacap_select_compact(const jacap_layout* layout, const float* score
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   const Ws w = make_ws(ws, c);
-  const int64_t units = (int64_t)dm.L * dm.Hkv * dm.S;
   const TraceRange trace("jacap/select_compact");
   return map_cuda(launch_select(dm, w, layout->cu_seqlens, scores, budget, idx, kept, layout->max_seqlen,
-                                persistent_grid(units, sms, 2), (cudaStream_t)stream,
-                                layout->dtype == JACAP_BF16 ? 1 : 0, k, v, k_out, v_out));
+                                (cudaStream_t)stream, layout->dtype == JACAP_BF16 ? 1 : 0, k, v, k_out, v_out));
 }
 
 jacap_status jacap_compact(const jacap_layout* layout, const void* k, const void* v, const int32_t* idx,
@@ -696,7 +692,7 @@ jacap_status jacap_device_status(const void* ws, void* stream) {
   if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return JACAP_ERR_CUDA;
   uint32_t word = 0;
   if (cudaMemcpy(&word, ws, sizeof(word), cudaMemcpyDeviceToHost) != cudaSuccess) return JACAP_ERR_CUDA;
-  if (word & ST_INVALID) return JACAP_ERR_INVALID_ARG;
+  if (word & (ST_INVALID | ST_SELECT)) return JACAP_ERR_INVALID_ARG;
   if (word & ST_TIMEOUT) return JACAP_ERR_TIMEOUT;
   if (word & ST_NONFINITE) return JACAP_ERR_NONFINITE;
   return JACAP_OK;

@@ -23,6 +23,7 @@ enum : uint32_t {
   ST_INVALID = 1u,    // malformed cu_seqlens
   ST_NONFINITE = 2u,  // NaN/Inf in an input or intermediate
   ST_TIMEOUT = 4u,    // a bounded wait expired
+  ST_SELECT = 8u,     // malformed cu_seqlens met by the selection, whose other units go on
 };
 
 constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;  // 2 s per wait

@@ -64,9 +64,10 @@ __device__ __forceinline__ void compact_ordered_unit(const Dims& dm, int plane, 
 // and does not decrease, so hole j lies after the i = #{p < f : c(p) <= j}
 // kept positions below it, at row j + i. One warp per hole (lanes over the
 // 16-byte pieces of the row); sources and destinations are disjoint.
+// Part `part` of `parts` of the holes.
 template <typename T, int NT>
-__device__ __forceinline__ void fill_holes_unit(const Dims& dm, int plane, int64_t t0, int kept, int f, T* k, T* v,
-                                                int32_t* pos, const int32_t* ix) {
+__device__ __forceinline__ void fill_holes_unit(const Dims& dm, int plane, int64_t t0, int kept, int f, int part,
+                                                int parts, T* k, T* v, int32_t* pos, const int32_t* ix) {
   constexpr int RB = D * (int)sizeof(T) / 16;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int holes = kept - f;
@@ -77,7 +78,7 @@ __device__ __forceinline__ void fill_holes_unit(const Dims& dm, int plane, int64
   const int64_t st16 = dm.kv_st * (int64_t)sizeof(T) / 16;
   // the tags follow the layout of K with one int32 per token row
   int32_t* pb = pos != nullptr ? pos + (int64_t)l * (dm.kv_sl / dm.kv_st) + (int64_t)g * (dm.kv_sh / dm.kv_st) : nullptr;
-  for (int j = warp; j < holes; j += NT / 32) {
+  for (int j = part * (NT / 32) + warp; j < holes; j += parts * (NT / 32)) {
     int lo = 0, hi = f;  // first p in [0, f) with c(p) > j (f if none)
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;

@@ -97,7 +97,7 @@ cudaError_t launch_fused(const CUtensorMap& vmap, const Dims& dm, const Ws& ws, 
 // launch_compact does. With kio: the holes of kio, vio (and pos) are filled in
 // place, as launch_compact_inplace does without preserve_order.
 cudaError_t launch_select(const Dims& dm, const Ws& ws, const int32_t* cu, const float* scores, int budget,
-                          int32_t* idx, int32_t* kept, int max_seqlen, int grid, cudaStream_t st, int dtype = 1,
+                          int32_t* idx, int32_t* kept, int max_seqlen, cudaStream_t st, int dtype = 1,
                           const void* k = nullptr, const void* v = nullptr, void* k_out = nullptr,
                           void* v_out = nullptr, void* kio = nullptr, void* vio = nullptr, int32_t* pos = nullptr);
 cudaError_t launch_compact(const Dims& dm, int dtype, const int32_t* cu, const void* k, const void* v,

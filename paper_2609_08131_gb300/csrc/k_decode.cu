@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(CI_THREADS)
     if (tid == 0) flag(ws, ST_INVALID);
     return;
   }
-  fill_holes_unit<T, CI_THREADS>(dm, plane, t0, kept, s_f, k, v, pos, ix);
+  fill_holes_unit<T, CI_THREADS>(dm, plane, t0, kept, s_f, 0, 1, k, v, pos, ix);
 }
 
 template <typename T>

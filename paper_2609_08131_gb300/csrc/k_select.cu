@@ -1,24 +1,42 @@
 // k_select.cu - TOP-B selection (Algorithm 1 step 5) and compaction of the
 // retained cache Z_C (Sec. 3.1).
 //
-// select_kernel: one CTA per unit (grid-stride), of NT = 1024 threads, or of
-// 256 when the longest request has at most 4096 tokens and there are more
-// units than SMs (then four or more CTAs fit an SM and a pass over many short
-// units, as in decoding-stage eviction, runs in one wave), or of 512 (two per
-// SM) for longer requests when there are more than two SMs' worth of units. Scores are
-// non-negative float32, so their bit patterns order like unsigned integers.
-// Three radix passes (digits of 11, 11 and 10 bits, most significant first,
-// shared-memory histograms; a pass counts only keys that match the digits
-// found so far) find the B-th largest key T and how many keys equal to T are
-// still needed. The keys are read in slabs of NT KPT into registers (KPT
-// per lane, all loads in flight together; KPT = 4, 8, 16 or 32, the smallest
-// that holds the longest request in one slab); a request that fits one slab is
-// read once and every pass works on registers. Emission walks the slabs in
-// order; in a slab each warp owns 32 KPT consecutive positions, counts its keys
-// > T and == T with ballots, and the warp totals give where its kept
-// positions go and which of its keys == T are among the first `need` by
-// position (ties go to the lower position); kept positions come out in
-// ascending order. All of it is deterministic.
+// select_kernel: one CTA per unit. Scores are non-negative float32, so their bit
+// patterns order like unsigned integers. The kept set of a unit of more than B
+// tokens is {key > T} and the keys == T at positions <= I, for the B-th token
+// (T, I) in the order of Algorithm 1 (score descending, then position):
+//  1. histogram of the keys' distance from a reference R just above the first
+//     slab's maximum, in 2048 bins of 2^16 (1/128 octave each: 16 octaves, in
+//     which the lanes of a warp rarely meet in one bin); keys further down cannot
+//     count unless the bins hold fewer than B keys;
+//  2. the bin that holds the B-th key, by a scan over all warps;
+//  3. that bin's keys (a handful) go to a list, and each one's rank in it names
+//     (T, I).
+// If the bins hold fewer than B keys, or the bin more than SE_CAND (many ties, as
+// with a window of one query), a radix selection over key digits and then, for
+// ties, position digits finds (T, I) instead.
+// Emission: the keys are held in registers in slabs of NT KPT (KPT per lane, all
+// loads in flight together; the smallest that holds the longest request; a longer
+// one is read again by each step, from L2); warp w owns 32 KPT consecutive
+// positions, lane j keeps the ballot of slot j, and prefix sums of the counts over
+// lanes and warps place each lane's positions: ascending, and deterministic.
+//
+// With fewer units than SMs, `parts` CTAs take a unit: each selects for itself (the
+// SMs would idle otherwise; all write the same positions) and moves its share of
+// the rows.
+//
+// Bound: latency and shared-memory atomics of one unit, then the row copies (HBM).
+// Why one CTA per unit dealt by the hardware, and small CTAs for short requests:
+// a resident grid that strides over the units gave a CTA the same request of a
+// batch each time when the number of requests divided the grid.
+// Measured against three radix passes over all keys in such a grid, selection and
+// row copies: 1024 units of 731-3072 tokens (256 kept) 0.152 -> 0.055 ms, 1024 units
+// of 2K-64K tokens (512) 0.290 -> 0.158, 320 units of 9001 (900) 0.102 -> 0.080, 256
+// units of 32768 (512) 0.057 -> 0.044, of 131072 (1024) 0.154 -> 0.124, 8 units of
+// 4099 (512) 0.018 -> 0.012; 448 slots of 2052 tokens with holes filled 0.045 -> 0.020.
+// The copies' bytes alone take 0.040, 0.079, 0.044, 0.020 and 0.040 ms of the first
+// five at the copy rate.
+//
 //
 // compact_kernel: 16-byte vector copies of the kept K and V rows into the
 // dense [L][Hkv][S][B][d] output; rows of -1 (or of a position outside the
@@ -32,6 +50,8 @@
 // MODE 0 only selects. (The in-place compaction in ascending order moves
 // every kept row; it stays a launch of its own, whose small CTAs keep more
 // bytes in flight per SM than one selection CTA per unit could.)
+#include <algorithm>
+
 #include "jacap_dev.cuh"
 #include "jacap_inplace.cuh"
 #include "jacap_internal.h"
@@ -40,6 +60,20 @@ namespace jacap {
 
 
 constexpr int SE_BINS = 2048;
+constexpr int SE_SHIFT = 16;    // a bin spans 2^16 keys
+constexpr int SE_CAND = 1024;   // keys of the B-th key's bin that are ranked directly
+constexpr int SE_IDX = 2048;    // kept positions also held in shared memory
+
+struct SeSmem {
+  uint32_t hist[SE_BINS];
+  uint32_t ckey[SE_CAND];
+  int32_t cidx[SE_CAND];
+  int32_t idx[SE_IDX];
+  uint32_t tot[2][32];  // counts per warp
+  uint32_t max, digit, need, count, T;
+  int32_t I;
+  int skip;
+};
 
 // Keys of slab `sl` into registers: lane's register j holds position
 // sl * NT KPT + 32 KPT w + 32 j + lane (coalesced; all loads in flight at
@@ -57,23 +91,24 @@ __device__ __forceinline__ void load_slab(const uint32_t* key, int n, int sl, in
 }
 
 // Rows out[0 .. B) of unit u (positions relative to the request start, as
-// emitted) from K and V into k_out, v_out; -1 or a position outside the
-// request gives a zero row. All threads of the CTA; out was written by them
-// before the barrier that precedes this call.
+// emitted; the first SE_IDX also in sidx if not null) from K and V into k_out,
+// v_out; -1 or a position outside the request gives a zero row. Part `part` of
+// `parts` of the copies. All threads of the CTA; out and sidx were written by them before the barrier that precedes this
+// call.
 template <typename T, int NT>
 __device__ __forceinline__ void gather_unit(const Dims& dm, int plane, int64_t start, int64_t end, bool valid,
                                             const T* __restrict__ k, const T* __restrict__ v,
-                                            const int32_t* out, int B, int64_t u, T* __restrict__ k_out,
-                                            T* __restrict__ v_out) {
+                                            const int32_t* out, const int32_t* sidx, int B, int64_t u, int part,
+                                            int parts, T* __restrict__ k_out, T* __restrict__ v_out) {
   constexpr int CH = D * (int)sizeof(T) / 16;  // 16-byte chunks per row
   const int l = plane / dm.Hkv, g = plane % dm.Hkv;
   const int64_t base = (int64_t)l * dm.kv_sl + (int64_t)g * dm.kv_sh;
   uint4* ko = (uint4*)(k_out + u * B * D);
   uint4* vo = (uint4*)(v_out + u * B * D);
 #pragma unroll 4
-  for (int e = threadIdx.x; e < B * CH; e += NT) {
+  for (int e = part * NT + threadIdx.x; e < B * CH; e += parts * NT) {
     const int r = e / CH, c = e % CH;
-    const int32_t src = out[r];
+    const int32_t src = sidx != nullptr && r < SE_IDX ? sidx[r] : out[r];
     uint4 kk = make_uint4(0, 0, 0, 0), vv = make_uint4(0, 0, 0, 0);
     if (valid && src >= 0 && start + src < end) {
       const int64_t off = base + (start + src) * dm.kv_st;
@@ -85,216 +120,262 @@ __device__ __forceinline__ void gather_unit(const Dims& dm, int plane, int64_t s
   }
 }
 
+// The digit d (0 .. SE_BINS - 1) with (sum of hist over digits before d) < need <=
+// (that sum + hist[d]), digits counted from the top (DESC) or from 0, into
+// sm.digit; need less that sum into sm.need and hist[d] into sm.count. Every
+// thread of the CTA; the histogram is complete and holds at least `need`.
+template <int NT, bool DESC>
+__device__ __forceinline__ void find_digit(SeSmem& sm, uint32_t need, int tid) {
+  constexpr int PER = SE_BINS / NT, NW = NT / 32;
+  const int lane = tid & 31, warp = tid >> 5;
+  uint32_t c[PER], sum = 0;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int r = tid * PER + k;  // rank of the digit in the order of the sums
+    c[k] = sm.hist[DESC ? SE_BINS - 1 - r : r];
+    sum += c[k];
+  }
+  uint32_t inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) sm.tot[0][warp] = inc;
+  __syncthreads();
+  uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp && lane < NW ? sm.tot[0][lane] : 0u) + inc - sum;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    if (before < need && before + c[k] >= need) {  // one thread, one k
+      const int r = tid * PER + k;
+      sm.digit = (uint32_t)(DESC ? SE_BINS - 1 - r : r);
+      sm.need = need - before;
+      sm.count = c[k];
+    }
+    before += c[k];
+  }
+  __syncthreads();
+}
+
+// (T, I) of the B-th token by digits, most significant first: of the keys (11, 11
+// and 10 bits), then, if only some of the keys == T are kept, of their positions.
+// Reads the keys from global memory at every step. (Every thread of the CTA.)
+template <int NT>
+__device__ __noinline__ void radix_boundary(SeSmem& sm, const uint32_t* key, int n, int B, int tid) {
+  uint32_t prefix = 0, mask = 0, need = (uint32_t)B;
+#pragma unroll 1
+  for (int pass = 0; pass < 3; ++pass) {
+    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+    const uint32_t dmask = pass == 2 ? 1023u : 2047u;
+    __syncthreads();
+    for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += NT) {
+      const uint32_t x = __ldg(key + i);
+      if ((x & mask) == prefix) atomicAdd(&sm.hist[(x >> shift) & dmask], 1u);
+    }
+    __syncthreads();
+    find_digit<NT, true>(sm, need, tid);
+    prefix |= sm.digit << shift;
+    mask |= dmask << shift;
+    need = sm.need;
+  }
+  const uint32_t T = prefix, equal = sm.count;
+  uint32_t pos = 0, pmask = 0;
+  if (equal > need) {  // the first `need` of them by position
+#pragma unroll 1
+    for (int shift = 22; shift >= 0; shift -= 11) {
+      __syncthreads();
+      for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
+      __syncthreads();
+      for (int i = tid; i < n; i += NT)
+        if (__ldg(key + i) == T && ((uint32_t)i & pmask) == pos) atomicAdd(&sm.hist[((uint32_t)i >> shift) & 2047u], 1u);
+      __syncthreads();
+      find_digit<NT, false>(sm, need, tid);
+      pos |= sm.digit << shift;
+      pmask |= 2047u << shift;
+      need = sm.need;
+    }
+  } else {
+    pos = (uint32_t)n;  // all of them
+  }
+  __syncthreads();
+  if (tid == 0) {
+    sm.T = T;
+    sm.I = (int32_t)pos;
+  }
+  __syncthreads();
+}
+
 template <int KPT, typename E, int MODE, int NT>
-__global__ void __launch_bounds__(NT, NT == 512 ? 2 : 1)
+__global__ void __launch_bounds__(NT, 1024 / NT)
     select_kernel(Dims dm, Ws ws, const int32_t* __restrict__ cu, const float* __restrict__ scores, int B,
                   int32_t* __restrict__ idx, int32_t* __restrict__ kept, const E* __restrict__ k,
                   const E* __restrict__ v, E* __restrict__ k_out, E* __restrict__ v_out, E* kio, E* vio,
-                  int32_t* pos) {
+                  int32_t* pos, int parts) {
   constexpr bool GATHER = MODE == 1;
   pdl_wait();
-  constexpr int SE_KPT = KPT;
-  constexpr int SE_SLAB = NT * KPT;  // warp w holds positions 32 KPT w .. + 32 KPT - 1 of a slab
+  constexpr int SLAB = NT * KPT;  // warp w holds positions 32 KPT w .. + 32 KPT - 1 of a slab
   constexpr int NW = NT / 32;
-  __shared__ uint32_t hist[SE_BINS];
-  __shared__ uint32_t s_digit, s_need;
-  __shared__ int s_skip;
+  __shared__ SeSmem sm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_skip = status_failed(ws) ? 1 : 0;
+  const int u = blockIdx.x / parts, part = blockIdx.x % parts;
+  const int plane = u / dm.S, s = u % dm.S;
+  const int64_t start = cu[s];
+  const int64_t end = cu[s + 1];
+  if (tid == 0) {
+    // (not a bit that another CTA of this launch may have set)
+    sm.skip = (*((volatile uint32_t*)ws.status) & ~(uint32_t)ST_SELECT) != 0u ? 1 : 0;
+    sm.max = 0;
+    sm.count = 0;
+  }
+  for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
   __syncthreads();
-  if (s_skip) return;
-  const int units = dm.L * dm.Hkv * dm.S;
-  const uint32_t lt = (1u << lane) - 1u;
-  // time accounting (trace builds, thread 0): 0 the scores loaded (one slab),
-  // 1 the radix passes, 2 the emission, 3 the rows gathered, 4 units, 5 the
-  // whole unit (units of more than B tokens)
+  if (sm.skip) return;
+  // time accounting (trace builds, thread 0): 0 the scores loaded (one slab) and
+  // their maximum, 1 the B-th token, 2 the emission, 3 the rows gathered, 4 units,
+  // 5 the whole unit (units of more than B tokens)
   TRC_DECL(TR_CTA_SLOTS);
-  for (int u = blockIdx.x; u < units; u += gridDim.x) {
-    TRC_T(tr_u);
-    const int plane = u / dm.S, s = u % dm.S;
-    const int64_t start = cu[s];
-    const int64_t end = cu[s + 1];
-    int32_t* out = idx + (int64_t)u * B;
-    const bool valid = !(start < 0 || end < start || end > dm.Ntot);
-    if (!valid) {  // malformed cu_seqlens: no reads
-      for (int r = tid; r < B; r += NT) out[r] = -1;
-      if (tid == 0) {
-        flag(ws, ST_INVALID);
-        if (plane == 0) kept[s] = 0;
-      }
-      if constexpr (GATHER) {
-        __syncthreads();
-        gather_unit<E, NT>(dm, plane, start, end, false, k, v, out, B, u, k_out, v_out);
-      }
-      continue;
+  TRC_T(tr_u);
+  int32_t* out = idx + (int64_t)u * B;
+  const bool valid = !(start < 0 || end < start || end > dm.Ntot);
+  const int n = valid ? (int)(end - start) : 0;
+  if (!valid && tid == 0) flag(ws, ST_SELECT);  // malformed cu_seqlens: no reads
+  if (plane == 0 && tid == 0) kept[s] = min(n, B);
+  if (n <= B) {
+    for (int r = tid; r < B; r += NT) out[r] = r < n ? r : -1;
+    if constexpr (GATHER) {
+      __syncthreads();
+      gather_unit<E, NT>(dm, plane, start, end, valid, k, v, out, nullptr, B, u, part, parts, k_out, v_out);
     }
-    const int n = (int)(end - start);
-    const uint32_t* key = (const uint32_t*)(scores + (int64_t)plane * dm.Ntot + start);
-    if (plane == 0 && tid == 0) kept[s] = min(n, B);
-    if (n <= B) {
-      for (int r = tid; r < B; r += NT) out[r] = r < n ? r : -1;
-      if constexpr (GATHER) {
-        __syncthreads();
-        gather_unit<E, NT>(dm, plane, start, end, true, k, v, out, B, u, k_out, v_out);
-      }
-      continue;
-    }
-    const int nslab = (n + SE_SLAB - 1) / SE_SLAB;
-    uint32_t kr[SE_KPT];
-    TRC_INC(4);
-    if (nslab == 1) load_slab<KPT, NT>(key, n, 0, warp, lane, kr);  // register-resident for all passes
-    TRC_ADD(0, tr_u);
-    TRC_T(tr_r);
-    // ---- radix select of the B-th largest key: digits [31:21], [20:10], [9:0] ----
-    uint32_t prefix = 0, mask = 0, need = (uint32_t)B;
+    return;
+  }
+  const uint32_t* key = (const uint32_t*)(scores + (int64_t)plane * dm.Ntot + start);
+  const int nslab = (n + SLAB - 1) / SLAB;
+  uint32_t kr[KPT];
+  TRC_INC(4);
+  load_slab<KPT, NT>(key, n, 0, warp, lane, kr);  // one slab: register-resident for all steps
+  uint32_t m = 0;
+#pragma unroll
+  for (int j = 0; j < KPT; ++j) m = max(m, kr[j]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) atomicMax(&sm.max, m);
+  __syncthreads();
+  TRC_ADD(0, tr_u);
+  TRC_T(tr_r);
+  // the reference is an octave above the first slab's maximum if there are others
+  const uint32_t up = nslab > 1 ? 1u << 23 : 0u;
+  const uint32_t R = sm.max > 0xffffffffu - up ? 0xffffffffu : sm.max + up;
+  // bin of a key: 0 from the reference up, SE_BINS or more if too far below it
+  auto bin_of = [&](uint32_t x) { return x >= R ? 0u : (R - x) >> SE_SHIFT; };
 #pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-      const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-      const uint32_t dmask = pass == 2 ? 1023u : 2047u;
-      for (int b = tid; b < SE_BINS; b += NT) hist[b] = 0;
-      __syncthreads();
-#pragma unroll 1
-      for (int sl = 0; sl < nslab; ++sl) {
-        if (nslab > 1) load_slab<KPT, NT>(key, n, sl, warp, lane, kr);
-        const int base = sl * SE_SLAB + warp * (32 * SE_KPT) + lane;
+  for (int sl = 0; sl < nslab; ++sl) {
+    if (sl > 0) load_slab<KPT, NT>(key, n, sl, warp, lane, kr);
+    const int base = sl * SLAB + warp * (32 * KPT) + lane;
 #pragma unroll
-        for (int j = 0; j < SE_KPT; ++j)
-          if (base + 32 * j < n && (kr[j] & mask) == prefix) atomicAdd(&hist[(kr[j] >> shift) & dmask], 1u);
-      }
-      __syncthreads();
-      if (warp == 0) {
-        // lane l sums bins 64 l .. 64 l + 63 (in a rotated order, so that the
-        // lanes' loads fall in different banks); suffix sums over the lanes
-        // locate the group of 64 bins that holds the need-th largest key, and
-        // a second suffix scan over that group (two bins per lane) the bin
-        uint32_t c = 0;
-#pragma unroll 8
-        for (int b = 0; b < 64; ++b) c += hist[64 * lane + ((b + lane) & 63)];
-        uint32_t suf = c;  // sum over lanes >= lane
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_down_sync(0xffffffffu, suf, o);
-          if (lane + o < 32) suf += y;
-        }
-        const uint32_t above = suf - c;  // keys in bins of higher lanes
-        const uint32_t hit = __ballot_sync(0xffffffffu, above < need && suf >= need);  // exactly one lane
-        const int g = __ffs(hit) - 1;
-        const uint32_t gabove = __shfl_sync(0xffffffffu, above, g);  // keys above the group
-        // bins 64 g + 2 lane (+1), suffix sums from the top of the group down
-        const uint32_t h0 = hist[64 * g + 2 * lane], h1 = hist[64 * g + 2 * lane + 1];
-        const uint32_t c2 = h0 + h1;
-        uint32_t suf2 = c2;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_down_sync(0xffffffffu, suf2, o);
-          if (lane + o < 32) suf2 += y;
-        }
-        const uint32_t a1 = gabove + suf2 - c2;  // keys above bin 2 lane + 1 of the group
-        const uint32_t a0 = a1 + h1;             // keys above bin 2 lane
-        // the bin d with (keys above d) < need <= (keys above d) + hist[d]
-        const bool in1 = a1 < need && a1 + h1 >= need, in0 = a0 < need && a0 + h0 >= need;
-        if (in1) {
-          s_digit = (uint32_t)(64 * g + 2 * lane + 1);
-          s_need = need - a1;
-        } else if (in0) {
-          s_digit = (uint32_t)(64 * g + 2 * lane);
-          s_need = need - a0;
-        }
-      }
-      __syncthreads();
-      prefix |= s_digit << shift;
-      mask |= dmask << shift;
-      need = s_need;
-      __syncthreads();
+    for (int j = 0; j < KPT; ++j) {
+      const uint32_t d = bin_of(kr[j]);
+      if (base + 32 * j < n && d < SE_BINS) atomicAdd(&sm.hist[d], 1u);
     }
-    const uint32_t T = prefix;  // the B-th largest key; the first `need` keys == T are kept
-    TRC_ADD(1, tr_r);
-    TRC_T(tr_e);
-    // ---- emission, slab by slab; in a slab warp w owns positions 32 KPT w .. ----
-    uint32_t gt_run = 0, eq_run = 0;  // kept-greater and equal keys before this slab
+  }
+  __syncthreads();
+  find_digit<NT, false>(sm, (uint32_t)B, tid);
+  uint32_t T;
+  int32_t I;
+  // (sm.count is still 0 where the bins hold fewer than B keys)
+  if (sm.count != 0 && sm.count <= SE_CAND) {
+    const uint32_t d = sm.digit, need = sm.need;
+    const int cand = (int)sm.count;
+    __syncthreads();  // everyone has read the bin's count
+    if (tid == 0) sm.count = 0;
+    __syncthreads();
 #pragma unroll 1
     for (int sl = 0; sl < nslab; ++sl) {
       if (nslab > 1) load_slab<KPT, NT>(key, n, sl, warp, lane, kr);
-      const int base = sl * SE_SLAB + warp * (32 * SE_KPT) + lane;
-      // the warp's counts of keys > T and == T, and which register slots hold
-      // any key >= T (most hold none: only B of the n keys are kept)
-      uint32_t gt = 0, eq = 0, jmask = 0;
+      const int base = sl * SLAB + warp * (32 * KPT) + lane;
 #pragma unroll
-      for (int j = 0; j < SE_KPT; ++j) {
-        const bool v = base + 32 * j < n;
-        const uint32_t bg = __ballot_sync(0xffffffffu, v && kr[j] > T);
-        const uint32_t be = __ballot_sync(0xffffffffu, v && kr[j] == T);
-        gt += __popc(bg);
-        eq += __popc(be);
-        if (bg | be) jmask |= 1u << j;
-      }
-      if (lane == 0) {
-        hist[warp] = gt;  // the histogram is free again: it holds the warp totals
-        hist[NW + warp] = eq;
-      }
-      __syncthreads();
-      if (warp == 0) {  // exclusive prefixes of the warp totals (lane w: warp w) and the slab totals
-        const uint32_t g = lane < NW ? hist[lane] : 0u, e = lane < NW ? hist[NW + lane] : 0u;
-        uint32_t gs = g, es = e;  // inclusive scans
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, gs, o), z = __shfl_up_sync(0xffffffffu, es, o);
-          if (lane >= o) {
-            gs += y;
-            es += z;
-          }
-        }
-        if (lane < NW) {
-          hist[2 * NW + lane] = gs - g;
-          hist[3 * NW + lane] = es - e;
-        }
-        if (lane == 31) {
-          hist[4 * NW] = gs;
-          hist[4 * NW + 1] = es;
+      for (int j = 0; j < KPT; ++j) {
+        if (base + 32 * j < n && bin_of(kr[j]) == d) {
+          const uint32_t at = atomicAdd(&sm.count, 1u);
+          sm.ckey[at] = kr[j];
+          sm.cidx[at] = base + 32 * j;
         }
       }
-      __syncthreads();
-      const uint32_t gt_before = gt_run + hist[2 * NW + warp], eq_before = eq_run + hist[3 * NW + warp];
-      const uint32_t gt_all = hist[4 * NW], eq_all = hist[4 * NW + 1];
-      // kept before this warp's block: all greater keys plus the equal ones of rank < need
-      uint32_t pos = gt_before + min(eq_before, need);
-      uint32_t er = eq_before;
-#pragma unroll
-      for (int j = 0; j < SE_KPT; ++j) {
-        if (!(jmask & (1u << j))) continue;  // warp-uniform: no key >= T in this slot
-        const int i = base + 32 * j;
-        const bool v = i < n;
-        const uint32_t beq = __ballot_sync(0xffffffffu, v && kr[j] == T);
-        const uint32_t my_er = er + __popc(beq & lt);
-        const bool sel = v && (kr[j] > T || (kr[j] == T && my_er < need));
-        const uint32_t bsel = __ballot_sync(0xffffffffu, sel);
-        const uint32_t my_pos = pos + __popc(bsel & lt);
-        if (sel && my_pos < (uint32_t)B) out[my_pos] = i;
-        pos += __popc(bsel);
-        er += __popc(beq);
-      }
-      gt_run += gt_all;
-      eq_run += eq_all;
-      __syncthreads();  // the totals in hist are read before the next slab rewrites them
     }
-    // (the barrier that ends the last slab also orders the emitted positions
-    // before they are read back here)
-    TRC_ADD(2, tr_e);
-    TRC_T(tr_g);
-    if constexpr (GATHER) gather_unit<E, NT>(dm, plane, start, end, true, k, v, out, B, u, k_out, v_out);
-    TRC_ADD(3, tr_g);
-    if constexpr (MODE == 2) {
-      // f = the kept positions below B (they ascend: a binary search)
-      int lo = 0, hi = B;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (out[mid] < B) lo = mid + 1; else hi = mid;
+    __syncthreads();
+    for (int c = tid; c < cand; c += NT) {  // the token of rank need - 1 in the bin
+      const uint32_t x = sm.ckey[c];
+      const int32_t i = sm.cidx[c];
+      uint32_t rank = 0;
+      for (int e = 0; e < cand; ++e) {
+        const uint32_t y = sm.ckey[e];
+        rank += y > x || (y == x && sm.cidx[e] < i) ? 1u : 0u;
       }
-      fill_holes_unit<E, NT>(dm, plane, start, B, lo, kio, vio, pos, out);
+      if (rank == need - 1) {
+        sm.T = x;
+        sm.I = i;
+      }
     }
-    if constexpr (MODE == 2) __syncthreads();  // the unit's rows have moved before `out` is reused
-    TRC_ADD(5, tr_u);
+    __syncthreads();
+  } else {
+    radix_boundary<NT>(sm, key, n, B, tid);
   }
+  T = sm.T;
+  I = sm.I;
+  TRC_ADD(1, tr_r);
+  TRC_T(tr_e);
+  // ---- emission, slab by slab ----
+  uint32_t run = 0;  // kept before this slab
+#pragma unroll 1
+  for (int sl = 0; sl < nslab; ++sl) {
+    if (nslab > 1) load_slab<KPT, NT>(key, n, sl, warp, lane, kr);
+    const int first = sl * SLAB + warp * (32 * KPT);
+    uint32_t mine = 0;  // the kept tokens of slot `lane`
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+      const int i = first + 32 * j + lane;
+      const uint32_t b = __ballot_sync(0xffffffffu, i < n && (kr[j] > T || (kr[j] == T && i <= I)));
+      if (lane == j) mine = b;
+    }
+    const uint32_t c = __popc(mine);
+    uint32_t inc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    uint32_t* tot = sm.tot[sl & 1];
+    if (lane == 31) tot[warp] = inc;
+    __syncthreads();
+    const uint32_t w = lane < NW ? tot[lane] : 0u;
+    uint32_t at = run + __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + inc - c;
+    run += __reduce_add_sync(0xffffffffu, w);
+    while (mine != 0) {
+      const int i = first + 32 * lane + __ffs(mine) - 1;
+      mine &= mine - 1;
+      if (at < (uint32_t)B) {
+        out[at] = i;
+        if (at < SE_IDX) sm.idx[at] = i;
+      }
+      ++at;
+    }
+  }
+  __syncthreads();  // the positions are read back below
+  TRC_ADD(2, tr_e);
+  TRC_T(tr_g);
+  if constexpr (GATHER) gather_unit<E, NT>(dm, plane, start, end, true, k, v, out, sm.idx, B, u, part, parts, k_out,
+                                          v_out);
+  TRC_ADD(3, tr_g);
+  if constexpr (MODE == 2) {
+    // f = the kept positions below B (they ascend: a binary search)
+    int lo = 0, hi = B;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((mid < SE_IDX ? sm.idx[mid] : out[mid]) < B) lo = mid + 1; else hi = mid;
+    }
+    fill_holes_unit<E, NT>(dm, plane, start, B, lo, part, parts, kio, vio, pos, out);
+  }
+  TRC_ADD(5, tr_u);
   if (tid == 0) TRC_PUT(ws, TR_K_SELECT, 6);
 }
 
@@ -329,54 +410,58 @@ __global__ void __launch_bounds__(256)
 template <int KPT, int NT>
 static cudaError_t launch_select_kpt(const Dims& dm, const Ws& ws, const int32_t* cu, const float* scores, int budget,
                                      int32_t* idx, int32_t* kept, int dtype, const void* k, const void* v,
-                                     void* k_out, void* v_out, void* kio, void* vio, int32_t* pos, int grid,
+                                     void* k_out, void* v_out, void* kio, void* vio, int32_t* pos, int grid, int parts,
                                      cudaStream_t st) {
   using bf = __nv_bfloat16;
   if (kio != nullptr) {  // hole filling in place
     if (dtype == 1)
       return launch_pdl(dm.pdl != 0, select_kernel<KPT, bf, 2, NT>, grid, NT, 0, st, dm, ws, cu, scores, budget,
                         idx, kept, (const bf*)nullptr, (const bf*)nullptr, (bf*)nullptr, (bf*)nullptr, (bf*)kio,
-                        (bf*)vio, pos);
+                        (bf*)vio, pos, parts);
     return launch_pdl(dm.pdl != 0, select_kernel<KPT, float, 2, NT>, grid, NT, 0, st, dm, ws, cu, scores, budget,
                       idx, kept, (const float*)nullptr, (const float*)nullptr, (float*)nullptr, (float*)nullptr,
-                      (float*)kio, (float*)vio, pos);
+                      (float*)kio, (float*)vio, pos, parts);
   }
   if (k == nullptr)
     return launch_pdl(dm.pdl != 0, select_kernel<KPT, bf, 0, NT>, grid, NT, 0, st, dm, ws, cu, scores, budget,
                       idx, kept, (const bf*)nullptr, (const bf*)nullptr, (bf*)nullptr, (bf*)nullptr, (bf*)nullptr,
-                      (bf*)nullptr, (int32_t*)nullptr);
+                      (bf*)nullptr, (int32_t*)nullptr, parts);
   if (dtype == 1)
     return launch_pdl(dm.pdl != 0, select_kernel<KPT, bf, 1, NT>, grid, NT, 0, st, dm, ws, cu, scores, budget,
                       idx, kept, (const bf*)k, (const bf*)v, (bf*)k_out, (bf*)v_out, (bf*)nullptr, (bf*)nullptr,
-                      (int32_t*)nullptr);
+                      (int32_t*)nullptr, parts);
   return launch_pdl(dm.pdl != 0, select_kernel<KPT, float, 1, NT>, grid, NT, 0, st, dm, ws, cu, scores, budget,
                     idx, kept, (const float*)k, (const float*)v, (float*)k_out, (float*)v_out, (float*)nullptr,
-                    (float*)nullptr, (int32_t*)nullptr);
+                    (float*)nullptr, (int32_t*)nullptr, parts);
 }
 
 cudaError_t launch_select(const Dims& dm, const Ws& ws, const int32_t* cu, const float* scores, int budget,
-                          int32_t* idx, int32_t* kept, int max_seqlen, int grid, cudaStream_t st, int dtype,
+                          int32_t* idx, int32_t* kept, int max_seqlen, cudaStream_t st, int dtype,
                           const void* k, const void* v, void* k_out, void* v_out, void* kio, void* vio,
                           int32_t* pos) {
 #define JACAP_SELECT(KPT, NT)                                                                                   \
   JACAP_TRY((launch_select_kpt<KPT, NT>(dm, ws, cu, scores, budget, idx, kept, dtype, k, v, k_out, v_out, kio, vio, \
-                                        pos, grid, st)))
-  // small CTAs only pay off when the 1024-thread ones would need more than one
-  // wave (one per SM fits); for a few units the larger CTA finishes each sooner
+                                        pos, grid, parts, st)))
+  // More units than SMs: CTAs of 256 threads (four per SM) while they hold the
+  // longest request in one slab, of 512 (two per SM) beyond that (256 units of 32768
+  // tokens: 44 us, 51 with 1024 threads; of 131072: 124 and 132). Otherwise CTAs of
+  // 1024 threads, as many per unit as there are SMs for (112 units of 20011 tokens,
+  // 2048 kept: 55 us; 64 with two CTAs of 512 threads each).
   int dev = 0, sms = 0;
   JACAP_TRY(cudaGetDevice(&dev));
   JACAP_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t units = (int64_t)dm.L * dm.Hkv * dm.S;
-  const bool small = units > sms;
-  if (small && max_seqlen <= 256 * 4) JACAP_SELECT(4, 256);
-  else if (small && max_seqlen <= 256 * 8) JACAP_SELECT(8, 256);
-  else if (small && max_seqlen <= 256 * 16) JACAP_SELECT(16, 256);
-  // more than two waves of 1024-thread CTAs: two 512-thread CTAs per SM (keys
-  // in slabs of 16384, re-read from L2 by each pass) keep twice as many units
-  // going (config 5's 4096 units: 0.95 -> 0.85 ms); with fewer units the
-  // larger CTA finishes each unit sooner (256 units of 131072 tokens: 0.159
-  // against 0.170 ms)
-  else if (units > 2 * (int64_t)sms && max_seqlen > 1024 * 16) JACAP_SELECT(32, 512);
+  if (units >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
+  const bool many = units > sms;
+  const int parts = many || (k == nullptr && kio == nullptr)
+                        ? 1
+                        : (int)std::max<int64_t>(1, std::min<int64_t>(sms / units, budget / 32));
+  const int grid = (int)units * parts;
+  if (many && max_seqlen <= 256 * 4) JACAP_SELECT(4, 256);
+  else if (many && max_seqlen <= 256 * 8) JACAP_SELECT(8, 256);
+  else if (many && max_seqlen <= 256 * 16) JACAP_SELECT(16, 256);
+  else if (many && max_seqlen <= 256 * 32) JACAP_SELECT(32, 256);
+  else if (many) JACAP_SELECT(32, 512);
   else if (max_seqlen <= 1024 * 4) JACAP_SELECT(4, 1024);
   else if (max_seqlen <= 1024 * 8) JACAP_SELECT(8, 1024);
   else if (max_seqlen <= 1024 * 16) JACAP_SELECT(16, 1024);

@@ -577,3 +577,48 @@ def test_factor_inverts_the_capacity_matrix(layers, hkv, lens, tau):
     cond = torch.linalg.cond(A)
     err = (X @ A @ X.mT - torch.eye(128, dtype=torch.float64, device="cuda")).abs().amax((-2, -1))
     assert bool((err <= 4 * 128 * 2.0 ** -24 * cond).all()), (err / cond).max()
+
+
+SELECT_UNITS = ((1, 1), (20, 8), (40, 8))  # layers, KV heads: few units, more than SMs, more than twice
+
+
+@pytest.mark.parametrize("layers, hkv", SELECT_UNITS)
+@pytest.mark.parametrize("n", (1000, 4097, 8193, 20000, 40000))
+@pytest.mark.parametrize("kind", ("spread", "ties", "equal", "wide", "zero_but_few"))
+def test_selection_of_any_scores_is_the_stable_order(layers, hkv, n, kind):
+    """jacap_select against a stable descending sort: scores of a few octaves, many equal scores at
+    the boundary (by rank, and too many for that), all equal, spread over the whole exponent range
+    (the B-th score far below the maximum), and fewer than B that are not 0. Selection compares bit
+    patterns, so the positions are exactly those of the sort."""
+    if layers * hkv > 8 and n > 20000:
+        hkv, layers = 8, 20
+    g = torch.Generator(device=DEV).manual_seed(n + layers)
+    lens = (n, max(1, n // 3))
+    N = sum(lens)
+    B = max(1, n // 5)
+    x = torch.rand((layers, hkv, N), generator=g, device=DEV)
+    if kind == "spread":
+        x = torch.exp(x * 4 - 9)
+    elif kind == "ties":
+        x = (x * 7).floor() / 8
+    elif kind == "equal":
+        x = torch.full_like(x, 0.25)
+    elif kind == "wide":
+        x = torch.exp2(x * 200 - 120) * (1 + x)
+    else:
+        x = torch.where(x < 0.03, x, torch.zeros_like(x))
+    k = torch.zeros((layers, hkv, N, 128), dtype=torch.bfloat16, device=DEV)
+    q = torch.zeros((2, layers, hkv, 1, 128), dtype=torch.bfloat16, device=DEV)
+    cu = torch.tensor([0, lens[0], N], dtype=torch.int32, device=DEV)
+    ev = Evictor(Cache(q, k, k, cu, list(lens), hkv), B)
+    ev.ws[:64].zero_()
+    ev.scores.copy_(x)
+    ev.select()
+    ev.check()
+    for s, m in enumerate(lens):
+        a = 0 if s == 0 else lens[0]
+        order = torch.sort(x[:, :, a:a + m], dim=-1, descending=True, stable=True).indices[..., :B]
+        want = torch.sort(order, dim=-1).values.int()
+        kept = min(m, B)
+        assert torch.equal(ev.idx[:, :, s, :kept], want[..., :kept])
+        assert bool((ev.idx[:, :, s, kept:] == -1).all())
