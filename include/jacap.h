@@ -318,6 +318,26 @@ jacap_status jacap_stats_update(const jacap_layout* layout, const void* q_new, i
                                 float* stats, int32_t* counts, void* stream);
 
 /*
+ * jacap_append is one decode step of every request in one launch: request s's
+ * new token goes to row lengths[s] of its slot in k, v and (its id ids[s]) pos,
+ * and its query is merged into the running statistics as jacap_stats_update
+ * does. The layout holds the slots as num_seqs requests of max_seqlen rows each
+ * (total_tokens = num_seqs * max_seqlen); window is 1 and the q strides are those
+ * of q_new.
+ *
+ *   k_new, v_new  device pointers, element (s, l, g, c) at s strides[0] + l
+ *                 strides[1] + g strides[2] + c of k_new (strides[3 .. 5] for
+ *                 v_new), in the layout's dtype, 16-byte aligned rows
+ *   lengths, ids  HOST arrays [num_seqs], read during the call; 0 <= lengths[s]
+ *                 < max_seqlen
+ *   pos           as in jacap_compact_inplace, or NULL
+ */
+jacap_status jacap_append(const jacap_layout* layout, const void* k_new, const void* v_new,
+                          const int64_t* strides, const void* q_new, const int32_t* lengths,
+                          const int32_t* ids, void* k, void* v, int32_t* pos, float* stats,
+                          int32_t* counts, void* stream);
+
+/*
  * jacap_score_timed with the query statistics taken from running statistics
  * (as kept by jacap_stats_update) instead of a query window: per query head
  * mu = mean and lambda = M2 / n (M2 / (n - 1) with cov_unbiased), n = counts.

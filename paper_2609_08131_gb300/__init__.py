@@ -105,6 +105,9 @@ _SIGS = {
                                          _P, _P, _P, ctypes.c_size_t, _P, ctypes.POINTER(ctypes.c_void_p),
                                          ctypes.c_int32]),
     "jacap_stats_update": (ctypes.c_int, [ctypes.POINTER(jacap_layout), _P, ctypes.c_int32, _P, _P, _P]),
+    "jacap_append": (ctypes.c_int, [ctypes.POINTER(jacap_layout), _P, _P, ctypes.POINTER(ctypes.c_int64), _P,
+                                    ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32), _P, _P, _P, _P,
+                                    _P, _P]),
     "jacap_compact_inplace": (ctypes.c_int, [ctypes.POINTER(jacap_layout), _P, _P, _P, _P, ctypes.c_int32,
                                              ctypes.c_int32, _P, ctypes.c_size_t, _P]),
     "jacap_selftest_wait": (ctypes.c_int, [_P, ctypes.c_size_t, ctypes.c_int64, _P]),
@@ -178,6 +181,15 @@ def jacap_score_stats(layout, params, stats, counts, k, v, scores, ws, ws_bytes,
 
 def jacap_stats_update(layout, q_new, reset, stats, counts, stream) -> int:
     return lib().jacap_stats_update(ctypes.byref(layout), q_new, int(reset), stats, counts, stream)
+
+
+def jacap_append(layout, k_new, v_new, strides, q_new, lengths, ids, k, v, pos, stats, counts, stream) -> int:
+    """``strides``: six element strides (request, layer, head of k_new, then of v_new); ``lengths``,
+    ``ids``: sequences of ints, one per request."""
+    n = len(lengths)
+    return lib().jacap_append(ctypes.byref(layout), k_new, v_new, (ctypes.c_int64 * 6)(*strides), q_new,
+                              (ctypes.c_int32 * n)(*map(int, lengths)), (ctypes.c_int32 * n)(*map(int, ids)), k, v, pos, stats, counts,
+                              stream)
 
 
 def jacap_selftest_wait(ws, ws_bytes, limit_ns, stream) -> int:

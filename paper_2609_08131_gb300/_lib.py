@@ -122,6 +122,7 @@ EXPORTS = [
     "jacap_score_out",
     "jacap_score_stats",
     "jacap_stats_update",
+    "jacap_append",
     "jacap_compact_inplace",
     "jacap_select_compact_inplace",
     "jacap_select",

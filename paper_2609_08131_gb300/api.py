@@ -15,6 +15,7 @@ from . import (
     JACAP_BF16,
     JACAP_F32,
     JACAP_OK,
+    jacap_append,
     jacap_compact,
     jacap_device_status,
     jacap_evict_host,
@@ -463,6 +464,13 @@ class DecodeEvictor:
         full = [s for s in range(self.S) if self.lengths[s] >= self.cap]
         if full:
             raise RuntimeError(f"request {full[0]} is full; evict it first")
+        if self._one_launch(k_new, v_new, q_new, stream):
+            _check(jacap_append(self.step_layout, _ptr(k_new), _ptr(v_new), k_new.stride()[:3] + v_new.stride()[:3],
+                                _ptr(q_new), self.lengths, self.next_id, _ptr(self._k), _ptr(self._v),
+                                _ptr(self._pos), _ptr(self.stats), _ptr(self.counts), _stream(stream)), "jacap_append")
+            self.lengths = [n + 1 for n in self.lengths]
+            self.next_id = [n + 1 for n in self.next_id]
+            return [s for s in range(self.S) if self.lengths[s] >= self.cap]
         dev = self._k.device
         rows = torch.tensor(self.lengths, dtype=torch.long, device=dev)
         reqs = torch.arange(self.S, device=dev)
@@ -475,6 +483,21 @@ class DecodeEvictor:
         self.next_id = [n + 1 for n in self.next_id]
         self.merge_queries(q_new, stream)
         return [s for s in range(self.S) if self.lengths[s] >= self.cap]
+
+    def _one_launch(self, k_new, v_new, q_new, stream) -> bool:
+        """Whether jacap_append takes this step: plain tensors of the slots' dtype, device and exact
+        shapes with 16-byte aligned rows, nothing to differentiate, and the stream that the indexed
+        copies would run on. Otherwise the step is made of indexed copies and jacap_stats_update."""
+        if stream is not None and stream != torch.cuda.current_stream(self._k.device):
+            return False
+        if torch.cuda.is_current_stream_capturing():  # the rows' numbers would be frozen in the graph
+            return False
+        el16 = 16 // self._k.element_size()
+        for t, heads in ((k_new, self.Hkv), (v_new, self.Hkv), (q_new, self.Hq)):
+            if (type(t) is not torch.Tensor or t.dtype != self.dtype or t.device != self._k.device or t.requires_grad
+                    or tuple(t.shape) != (self.S, self.L, heads, 128) or t.stride(3) != 1 or t.data_ptr() % 16):
+                return False
+        return q_new.is_contiguous() and all(n % el16 == 0 for n in k_new.stride()[:3] + v_new.stride()[:3])
 
     def merge_queries(self, q_new, stream=None):
         """Merge one decode step's queries [S, L, Hq, 128] into the running statistics."""

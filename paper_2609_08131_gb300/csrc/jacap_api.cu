@@ -560,6 +560,38 @@ jacap_status jacap_stats_update(const jacap_layout* layout, const void* q_new, i
                                       (cudaStream_t)stream));
 }
 
+jacap_status jacap_append(const jacap_layout* layout, const void* k_new, const void* v_new, const int64_t* strides,
+                          const void* q_new, const int32_t* lengths, const int32_t* ids, void* k, void* v,
+                          int32_t* pos, float* stats, int32_t* counts, void* stream) {
+  jacap_status st = check_layout(layout);
+  if (st != JACAP_OK) return st;
+  if (k_new == nullptr || v_new == nullptr || strides == nullptr || q_new == nullptr || lengths == nullptr ||
+      ids == nullptr || k == nullptr || v == nullptr || stats == nullptr || counts == nullptr)
+    return JACAP_ERR_INVALID_ARG;
+  if (layout->window != 1 || layout->total_tokens != (int64_t)layout->num_seqs * layout->max_seqlen)
+    return JACAP_ERR_INVALID_ARG;
+  if (!aligned16(k_new) || !aligned16(v_new) || !aligned16(q_new) || !aligned16(k) || !aligned16(v) ||
+      !aligned16(stats) || ((uintptr_t)counts & 3u) != 0 || ((uintptr_t)pos & 3u) != 0 || !pos_layout_ok(layout, pos))
+    return JACAP_ERR_INVALID_ARG;
+  const int64_t el16 = layout->dtype == JACAP_BF16 ? 8 : 4;  // elements per 16 bytes
+  AppendArgs a = {};
+  for (int i = 0; i < 6; ++i) {
+    if (strides[i] < 0 || strides[i] % el16 != 0) return JACAP_ERR_INVALID_ARG;
+    a.strides[i] = strides[i];
+  }
+  for (int s = 0; s < layout->num_seqs; ++s)
+    if (lengths[s] < 0 || lengths[s] >= layout->max_seqlen) return JACAP_ERR_INVALID_ARG;
+  if ((int64_t)layout->num_layers * layout->num_kv_heads * 256 >= ((int64_t)1 << 31)) return JACAP_ERR_INVALID_ARG;
+  int sms = 0;
+  if ((st = check_device(&sms)) != JACAP_OK) return st;
+  Dims dm;
+  make_dims(layout, nullptr, dm);
+  a.k_new = k_new, a.v_new = v_new, a.q_new = q_new;
+  a.slot_rows = layout->max_seqlen;
+  a.k = k, a.v = v, a.pos = pos, a.stats = stats, a.counts = counts;
+  return map_cuda(launch_append(dm, layout->dtype == JACAP_BF16 ? 1 : 0, a, lengths, ids, (cudaStream_t)stream));
+}
+
 jacap_status jacap_compact_inplace(const jacap_layout* layout, void* k, void* v, int32_t* pos, const int32_t* idx,
                                    int32_t budget, int32_t preserve_order, void* ws, size_t ws_bytes, void* stream) {
   jacap_status st = check_layout(layout);

@@ -104,6 +104,18 @@ cudaError_t launch_compact(const Dims& dm, int dtype, const int32_t* cu, const v
                            const int32_t* idx, int budget, void* k_out, void* v_out, cudaStream_t st);
 cudaError_t launch_stats_update(const Dims& dm, int dtype, const void* q, float* stats, int32_t* counts, int reset,
                                 cudaStream_t st);
+// One decode step (jacap_append): new rows, slots and running statistics.
+struct AppendArgs {
+  const void *k_new, *v_new, *q_new;
+  int64_t strides[6];
+  int64_t slot_rows;
+  void *k, *v;
+  int32_t* pos;
+  float* stats;
+  int32_t* counts;
+};
+cudaError_t launch_append(const Dims& dm, int dtype, const AppendArgs& a, const int32_t* lengths, const int32_t* ids,
+                          cudaStream_t st);
 cudaError_t launch_stats_moments(const Dims& dm, const Ws& ws, const float* stats, const int32_t* counts,
                                  cudaStream_t st);
 cudaError_t launch_compact_inplace(const Dims& dm, const Ws& ws, int dtype, const int32_t* cu, void* k, void* v,

@@ -308,3 +308,38 @@ def test_many_slots_fill_their_holes_with_the_small_selection_ctas():
                 sel = torch.as_tensor(_arrangement(gidx, B, False), dtype=torch.long, device=DEV)
                 assert_rows_bitwise(kb[layer, g][sel], ev.k[s, layer, g, :B])
                 assert_rows_bitwise(vb[layer, g][sel], ev.v[s, layer, g, :B])
+
+
+@pytest.mark.parametrize("dtype", (torch.bfloat16, torch.float32))
+@pytest.mark.parametrize("S, L, Hq, Hkv", [(1, 2, 7, 1), (3, 1, 8, 8), (300, 1, 4, 2)])
+def test_a_step_in_one_launch_is_the_step_by_indexed_copies(dtype, S, L, Hq, Hkv):
+    """append() through jacap_append (contiguous and strided rows) against the indexed copies and
+    jacap_stats_update that it stands for: the same bytes in every buffer. (300 requests take two
+    launches.)"""
+    g = torch.Generator(device="cuda").manual_seed(5)
+
+    def randn(*shape):
+        return torch.randn(*shape, generator=g, device="cuda").to(dtype)
+
+    decs = [DecodeEvictor(S, L, Hq, Hkv, 6, 3, dtype=dtype) for _ in range(2)]
+    k0, v0, q0 = randn(S, L, Hkv, 8, 128), randn(S, L, Hkv, 8, 128), randn(S, L, Hq, 2, 128)
+    lengths = [3 + s % 4 for s in range(S)]
+    for d in decs:
+        d.start(k0, v0, q0, lengths)
+    decs[1]._one_launch = lambda *a: False
+    for step in range(3):
+        k, v, q = randn(S, L, Hkv, 128), randn(S, L, Hkv, 128), randn(S, L, Hq, 128)
+        if step == 1:  # the layout of a projection that computes K and V side by side
+            kv = randn(S, L, Hkv, 256)
+            k, v = kv[..., :128], kv[..., 128:]
+        if step == 2:
+            k = randn(Hkv, L, S, 128).permute(2, 1, 0, 3)
+        assert decs[0]._one_launch(k, v, q, None)
+        assert decs[0].append(k, v, q) == decs[1].append(k, v, q)
+    for name in ("_k", "_v", "_pos", "stats", "counts"):
+        assert torch.equal(getattr(decs[0], name), getattr(decs[1], name)), name
+    assert decs[0].lengths == decs[1].lengths and decs[0].next_id == decs[1].next_id
+    # other inputs keep the general path
+    assert not decs[0]._one_launch(k.float() if dtype == torch.bfloat16 else k.bfloat16(), v, q, None)
+    assert not decs[0]._one_launch(k, v, q, torch.cuda.Stream())
+    assert not decs[0]._one_launch(k, v, q.transpose(1, 2).contiguous().transpose(1, 2) if L > 1 else q[:, :, :1], None)
