@@ -61,7 +61,7 @@ namespace jacap {
 
 constexpr int SE_BINS = 2048;
 constexpr int SE_SHIFT = 16;    // a bin spans 2^16 keys
-constexpr int SE_CAND = 1024;   // keys of the B-th key's bin that are ranked directly
+constexpr int SE_CAND = 256;    // keys of the B-th key's bin that are ranked directly (a rank reads them all: ~3 us)
 constexpr int SE_IDX = 2048;    // kept positions also held in shared memory
 
 struct SeSmem {
@@ -157,47 +157,81 @@ __device__ __forceinline__ void find_digit(SeSmem& sm, uint32_t need, int tid) {
   __syncthreads();
 }
 
-// (T, I) of the B-th token by digits, most significant first: of the keys (11, 11
-// and 10 bits), then, if only some of the keys == T are kept, of their positions.
-// Reads the keys from global memory at every step. (Every thread of the CTA.)
-template <int NT>
-__device__ __noinline__ void radix_boundary(SeSmem& sm, const uint32_t* key, int n, int B, int tid) {
-  uint32_t prefix = 0, mask = 0, need = (uint32_t)B;
-#pragma unroll 1
-  for (int pass = 0; pass < 3; ++pass) {
-    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-    const uint32_t dmask = pass == 2 ? 1023u : 2047u;
-    __syncthreads();
-    for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
-    __syncthreads();
-    for (int i = tid; i < n; i += NT) {
-      const uint32_t x = __ldg(key + i);
-      if ((x & mask) == prefix) atomicAdd(&sm.hist[(x >> shift) & dmask], 1u);
-    }
-    __syncthreads();
-    find_digit<NT, true>(sm, need, tid);
-    prefix |= sm.digit << shift;
-    mask |= dmask << shift;
-    need = sm.need;
+// Histogram of digit(key, position) over the unit's keys from global memory (-1:
+// not counted). A warp's most frequent case, ties, makes one addition: the digit of
+// its first counted lane is added for all lanes that share it.
+template <int NT, typename F>
+__device__ __forceinline__ void digit_histogram(SeSmem& sm, const uint32_t* key, int n, int tid, F digit) {
+  __syncthreads();
+  for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
+  __syncthreads();
+  for (int i0 = 0; i0 < n; i0 += NT) {
+    const int i = i0 + tid;
+    const int d = i < n ? digit(__ldg(key + i), (uint32_t)i) : -1;
+    const uint32_t some = __ballot_sync(0xffffffffu, d >= 0);
+    if (some == 0) continue;
+    const int first = __ffs(some) - 1, d0 = __shfl_sync(0xffffffffu, d, first);
+    const uint32_t same = __ballot_sync(0xffffffffu, d == d0);
+    if ((tid & 31) == first) atomicAdd(&sm.hist[d0], (uint32_t)__popc(same));
+    else if (d >= 0 && d != d0) atomicAdd(&sm.hist[d], 1u);
   }
-  const uint32_t T = prefix, equal = sm.count;
-  uint32_t pos = 0, pmask = 0;
-  if (equal > need) {  // the first `need` of them by position
+  __syncthreads();
+}
+
+// (T, I) of the B-th token by digits, most significant first: of the distance below
+// R within its bin (known; the need-th key of it), or (bin < 0) of the whole keys;
+// then, if only some of the keys == T are kept, of their positions. (Every thread
+// of the CTA.)
+template <int NT>
+__device__ __noinline__ void radix_boundary(SeSmem& sm, const uint32_t* key, int n, uint32_t R, int bin,
+                                            uint32_t need, int tid) {
+  uint32_t T;
+  if (bin >= 0) {
+    const uint32_t hi = (uint32_t)bin << SE_SHIFT;  // distance >> 16 of the bin's keys, all of them <= R
+    digit_histogram<NT>(sm, key, n, tid, [&](uint32_t x, uint32_t) {
+      const uint32_t e = R - x;
+      return (e & ~0xffffu) == hi ? (int)((e & 0xffffu) >> 5) : -1;
+    });
+    find_digit<NT, false>(sm, need, tid);
+    need = sm.need;
+    const uint32_t mid = hi | (sm.digit << 5);
+    digit_histogram<NT>(sm, key, n, tid, [&](uint32_t x, uint32_t) {
+      const uint32_t e = R - x;
+      return (e & ~31u) == mid ? (int)(e & 31u) : -1;
+    });
+    find_digit<NT, false>(sm, need, tid);
+    need = sm.need;
+    T = R - (mid | sm.digit);
+  } else {
+    uint32_t prefix = 0, mask = 0;
 #pragma unroll 1
-    for (int shift = 22; shift >= 0; shift -= 11) {
-      __syncthreads();
-      for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
-      __syncthreads();
-      for (int i = tid; i < n; i += NT)
-        if (__ldg(key + i) == T && ((uint32_t)i & pmask) == pos) atomicAdd(&sm.hist[((uint32_t)i >> shift) & 2047u], 1u);
-      __syncthreads();
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+      const uint32_t dmask = pass == 2 ? 1023u : 2047u;
+      digit_histogram<NT>(sm, key, n, tid,
+                          [&](uint32_t x, uint32_t) { return (x & mask) == prefix ? (int)((x >> shift) & dmask) : -1; });
+      find_digit<NT, true>(sm, need, tid);
+      prefix |= sm.digit << shift;
+      mask |= dmask << shift;
+      need = sm.need;
+    }
+    T = prefix;
+  }
+  uint32_t pos = (uint32_t)n;  // all keys == T
+  if (sm.count > need) {       // the first `need` of them by position
+    uint32_t pmask = 0;
+    pos = 0;
+    // digits of 11 bits, from the highest one that a position has
+#pragma unroll 1
+    for (int shift = n > (1 << 22) ? 22 : (n > 2048 ? 11 : 0); shift >= 0; shift -= 11) {
+      digit_histogram<NT>(sm, key, n, tid, [&](uint32_t x, uint32_t i) {
+        return x == T && (i & pmask) == pos ? (int)((i >> shift) & 2047u) : -1;
+      });
       find_digit<NT, false>(sm, need, tid);
       pos |= sm.digit << shift;
       pmask |= 2047u << shift;
       need = sm.need;
     }
-  } else {
-    pos = (uint32_t)n;  // all of them
   }
   __syncthreads();
   if (tid == 0) {
@@ -318,7 +352,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     }
     __syncthreads();
   } else {
-    radix_boundary<NT>(sm, key, n, B, tid);
+    // in the bin, unless none was found or (several slabs) bin 0 reaches beyond R
+    const bool in_bin = sm.count != 0 && (nslab == 1 || sm.digit != 0);
+    const int bin = in_bin ? (int)sm.digit : -1;
+    const uint32_t need = in_bin ? sm.need : (uint32_t)B;
+    __syncthreads();  // (read before the next histogram's digit replaces them)
+    radix_boundary<NT>(sm, key, n, R, bin, need, tid);
   }
   T = sm.T;
   I = sm.I;
