@@ -47,10 +47,15 @@ __device__ __forceinline__ void load_unit_stats(const Dims& dm, const Ws& ws, in
 // read V transposed with ldmatrix, form w_i v_i = hi + lo with packed bf16
 // arithmetic and store hi and lo as two A operands; two MMAs per 16 tokens
 // accumulate v hi^T and v lo^T, in two accumulators, each chain issued by a
-// warp of its own: one thread's MMAs of N <= 128 follow each other at ~60 ns
-// here whatever their accumulators, while two issuing threads overlap theirs.
+// warp of its own.
 // The epilogue adds the two.
-// The scaling warps share nothing but the mbarriers of the pipeline. A run of
+// Bound: the arrival of V and rows (6.5 TB/s over 32 x 8 x 32768 tokens). With all
+// eight scaling warps on every tile their chain (weights, fragments, products,
+// stores, ~900 ns) set the pace; in two groups that take the tiles in turn it takes
+// half of it: 0.395 -> 0.384 ms there, 40 x 8 x 9001 (G = 5) 0.151 -> 0.143, 448
+// slots of 2052 tokens (G = 7) 0.076 -> 0.070. One MMA warp for both chains (its
+// MMAs take 495 ns a tile) measured 0.393 ms. The scaling warps share nothing but
+// the mbarriers of the pipeline. A run of
 // consecutive chunks of one unit in a CTA's item range accumulates in the
 // accumulator pair; four epilogue warps copy each finished run's Gram out
 // before the next run starts on it.
@@ -58,7 +63,6 @@ constexpr int GR_THREADS = 544;   // warp 0: TMA, 1 and 16: MMA, 2-9: scale, 10-
 constexpr int GR_MMA_LO_WARP = 16;  // issues the v lo^T chain (warp 1 the v hi^T chain)
 constexpr int GR_EPI0 = 10;       // first epilogue warp
 constexpr int GR_WEIGHT_WARP = 14;  // 14 and 15, 64 tokens of each tile each
-constexpr int GR_SCALERS = 256;
 constexpr int GR_BOX = 16384;      // {64 channels, 128 tokens} bf16, 128-byte swizzle
 constexpr int GR_V_BYTES = 2 * GR_BOX;
 constexpr int GR_W_BYTES = 512;    // the tile's weights as bf16 pairs, one word per token
@@ -74,11 +78,21 @@ template <int G, int RESERVE = 0>
 struct GrCfg {
   static constexpr int LK_BYTES = TILE * 2 * G * 4 + 16;  // a tile's logits/kappa rows (+ alignment slack)
   static constexpr size_t smem_for(int stages) {
-    return 1024 + (size_t)stages * (GR_V_BYTES + GR_W_BYTES + LK_BYTES) + 256;
+    return 1024 + (size_t)stages * (GR_V_BYTES + GR_W_BYTES + LK_BYTES) + 320;
   }
   static constexpr int VST = smem_for(6) + RESERVE + 512 <= 232448 ? 6 : 5;  // stages in flight
   static constexpr size_t SMEM = smem_for(VST);
   static_assert(SMEM + RESERVE + 512 <= 232448, "shared memory");  // 512: the static variables
+  // A group of scaling warps takes every other tile. With an odd number of stages
+  // it meets only every other use of a stage, and on a barrier per stage its parity
+  // wait could not tell "my tile landed" from "the other group's tile has not": a
+  // barrier per (tile parity, stage) then, so that every waiter sees consecutive
+  // phases.
+  static constexpr int NBAR = VST % 2 == 0 ? VST : 2 * VST;
+  static __device__ __forceinline__ int bar(uint32_t it) {
+    return VST % 2 == 0 ? (int)(it % VST) : (int)((it & 1) * VST + it % VST);
+  }
+  static __device__ __forceinline__ uint32_t parity(uint32_t it) { return (it / NBAR) & 1; }
 };
 
 // The tile's logits/kappa rows (2G floats per token): the copy starts at the
@@ -117,10 +131,10 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
   uint8_t* vring = smem;                                   // [GR_VST][GR_V_BYTES]
   uint8_t* wring = vring + GR_VST * GR_V_BYTES;            // [GR_VST][GR_W_BYTES] weight words
   uint8_t* lkring = wring + GR_VST * GR_W_BYTES;           // [GR_VST][LK_BYTES] logits/kappa rows
-  uint64_t* vfull = (uint64_t*)(lkring + GR_VST * C::LK_BYTES);
-  uint64_t* vempty = vfull + GR_VST;
-  uint64_t* wready = vempty + GR_VST;  // the weight warp has written the tile's weights
-  uint64_t* afull = wready + GR_VST;
+  uint64_t* vfull = (uint64_t*)(lkring + GR_VST * C::LK_BYTES);  // [C::NBAR]
+  uint64_t* vempty = vfull + C::NBAR;
+  uint64_t* wready = vempty + GR_VST;  // [C::NBAR] the weight warps have written the tile's weights
+  uint64_t* afull = wready + C::NBAR;
   uint64_t* aempty = afull + 2;
   uint64_t* accfull = aempty + 2;   // the run's Gram is complete in the accumulators
   uint64_t* accempty = accfull + 1; // the epilogue has read them
@@ -132,12 +146,14 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
     s_abort = 0;
     s_skip = status_failed(ws) ? 1 : 0;
     for (int i = 0; i < GR_VST; ++i) {
-      mbar_init(smem_u32(&vfull[i]), 1);
       mbar_init(smem_u32(&vempty[i]), 2);  // the two MMA warps' commits
+    }
+    for (int i = 0; i < C::NBAR; ++i) {
+      mbar_init(smem_u32(&vfull[i]), 1);
       mbar_init(smem_u32(&wready[i]), 2);  // the two weight warps
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(&afull[i]), GR_SCALERS / 32);
+      mbar_init(smem_u32(&afull[i]), 4);   // the tile's group of scaling warps
       mbar_init(smem_u32(&aempty[i]), 2);  // the two MMA warps' commits
     }
     mbar_init(smem_u32(accfull), 2);   // the two MMA warps' commits
@@ -186,7 +202,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
           TRC_ADD(0, tr_w);
           uint8_t* vt = vring + st * GR_V_BYTES;
           const LkTile lt = lk_tile<G>(dm, item, t);
-          const uint32_t bar = smem_u32(&vfull[st]);
+          const uint32_t bar = smem_u32(&vfull[C::bar(it)]);
           mbar_arrive_expect_tx(bar, GR_V_BYTES + lt.bytes);
           if (hints) {
             const uint64_t pv = (t - item.t0) < (int64_t)dm.keep_tiles * TILE ? keep : drop;
@@ -204,11 +220,11 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
       TRC_ADD(1, tr_all);
       TRC_PUT(ws, TR_K_GRAM, 2);
       for (uint32_t k = (it > (uint32_t)GR_VST ? it - GR_VST : 0); k < it; ++k)
-        mbar_wait(smem_u32(&vfull[k % GR_VST]), (k / GR_VST) & 1, ws, nullptr);
+        mbar_wait(smem_u32(&vfull[C::bar(k)]), C::parity(k), ws, nullptr);
     }
   } else if (warp == 1 || warp == GR_MMA_LO_WARP) {
     // ------------------------------------------------ MMA issuers ---------
-    if (lane == 0) {
+    if (elect_one()) {
       const bool lo = warp == GR_MMA_LO_WARP;  // the v lo^T chain
       // time accounting (trace builds): 2 waits for a scaled operand, 3 for a free
       // accumulator (run start), 4 the whole loop, 5 tiles
@@ -264,8 +280,11 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
     }
   } else if (warp < 10) {
     // ------------------------------------------------- scaling warps ------
+    // Two groups of four warps take the tiles in turn (group g those with it % 2 ==
+    // g, and operand buffer g), so that a group's chain of a tile (weights, V
+    // fragments, products, tensor-memory stores) overlaps the other's.
     const int quarter = warp & 3;        // TMEM lane quarter == channels 32 quarter .. +31
-    const int th = (warp - 2) >> 2;      // token half of each tile (blocks 4 th .. 4 th + 3)
+    const int grp = (warp - 2) >> 2;
     // ldmatrix row addresses: lane l -> matrix l / 8, row l % 8
     const int lm = lane >> 3, lr = lane & 7;
     // time accounting (trace builds, warp 2): 6 waits for V, 7 for the weights,
@@ -276,73 +295,72 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
     Item item;
     for (ItemStream is(dm, ws, part, parts, FUSED); is.next(item);) {
       for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
-        const int vs = it % GR_VST, ab = it & 1;
+        if ((int)(it & 1) != grp) continue;
+        const int vs = it % GR_VST;
         TRC_T(tr_v);
-        if (!mbar_wait(smem_u32(&vfull[vs]), (it / GR_VST) & 1, ws, abort)) goto scale_done;
+        if (!mbar_wait(smem_u32(&vfull[C::bar(it)]), C::parity(it), ws, abort)) goto scale_done;
         TRC_ADD(6, tr_v);
         TRC_T(tr_wr);
-        if (!mbar_wait(smem_u32(&wready[vs]), (it / GR_VST) & 1, ws, abort)) goto scale_done;
+        if (!mbar_wait(smem_u32(&wready[C::bar(it)]), C::parity(it), ws, abort)) goto scale_done;
         TRC_ADD(7, tr_wr);
-        // weights of this lane's token pairs (rows 2(l%4), 2(l%4)+1 of each
-        // 8-token half of its 4 blocks) as bf16 pairs; tokens past the item
-        // weigh zero
-        uint32_t wph[8], wpl[8];
-        {
-          const int nvalid = (int)(item.t1 - t < TILE ? item.t1 - t : TILE);
-          const uint32_t wsl = smem_u32(wring + vs * GR_W_BYTES);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int i0 = 16 * (4 * th + (e >> 1)) + 8 * (e & 1) + 2 * (lane & 3);
-            const uint32_t x0 = i0 < nvalid ? lds_u32(wsl + 4 * i0) : 0u;
-            const uint32_t x1 = i0 + 1 < nvalid ? lds_u32(wsl + 4 * i0 + 4) : 0u;
-            wph[e] = __byte_perm(x0, x1, 0x5410);  // (hi of token i0, hi of i0 + 1)
-            wpl[e] = __byte_perm(x0, x1, 0x7632);  // (lo, lo)
-          }
-        }
         TRC_T(tr_ae);
-        if (it >= 2 && !mbar_wait(smem_u32(&aempty[ab]), ((it >> 1) & 1) ^ 1, ws, abort)) goto scale_done;
+        if (it >= 2 && !mbar_wait(smem_u32(&aempty[grp]), ((it >> 1) & 1) ^ 1, ws, abort)) goto scale_done;
         TRC_ADD(8, tr_ae);
         TRC_T(tr_b);
         tc_fence_after();
         const uint32_t vt = smem_u32(vring + vs * GR_V_BYTES);
-        const uint32_t acol = tmem + GR_ACOL + 128 * ab;
-        // the tile's V fragments of this warp, all eight loads in flight
-        // before any arithmetic or tensor-memory store (each store orders the
-        // code around it); matrices: 0 = (tokens 0-7, ch c0..c0+7),
-        // 1 = (tokens 0-7, c0+8..), 2 = (8-15, c0..), 3 = (8-15, c0+8..)
-        uint32_t r[2][4][4];
+        const uint32_t wsl = smem_u32(wring + vs * GR_W_BYTES);
+        const uint32_t acol = tmem + GR_ACOL + 128 * grp;
 #pragma unroll
-        for (int lh = 0; lh < 2; ++lh)
+        for (int th = 0; th < 2; ++th) {  // 64 tokens: blocks 4 th .. 4 th + 3
+          // weights of this lane's token pairs (rows 2(l%4), 2(l%4)+1 of each 8-token
+          // half of the 4 blocks) as bf16 pairs (tokens past the item: zero words)
+          uint32_t wph[8], wpl[8];
 #pragma unroll
-          for (int blk = 0; blk < 4; ++blk) {
-            const int b = 4 * th + blk;  // 16-token block of the tile
-            const int c0 = quarter * 32 + lh * 16 + (lm & 1) * 8;
-            const int tokr = 16 * b + (lm >> 1) * 8 + lr;
-            const uint32_t addr = vt + (c0 >> 6) * GR_BOX + sw128_off(tokr, (c0 & 63) >> 3);
-            ldsm_x4_trans(addr, r[lh][blk][0], r[lh][blk][1], r[lh][blk][2], r[lh][blk][3]);
+          for (int e = 0; e < 8; ++e) {
+            const int i0 = 16 * (4 * th + (e >> 1)) + 8 * (e & 1) + 2 * (lane & 3);
+            const uint2 x = lds_u64(wsl + 4 * i0);
+            wph[e] = __byte_perm(x.x, x.y, 0x5410);  // (hi of token i0, hi of i0 + 1)
+            wpl[e] = __byte_perm(x.x, x.y, 0x7632);  // (lo, lo)
           }
+          // the V fragments, all eight loads in flight before any arithmetic or
+          // tensor-memory store (each store orders the code around it); matrices:
+          // 0 = (tokens 0-7, ch c0..c0+7), 1 = (tokens 0-7, c0+8..), 2 = (8-15,
+          // c0..), 3 = (8-15, c0+8..)
+          uint32_t r[2][4][4];
 #pragma unroll
-        for (int lh = 0; lh < 2; ++lh) {
-          // one 32-column slab (this warp's 4 token blocks) of hi and of lo,
-          // built in registers and written with one wide store each
-          uint32_t hi[16], lo[16];
+          for (int lh = 0; lh < 2; ++lh)
 #pragma unroll
-          for (int blk = 0; blk < 4; ++blk)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              // w v = hi + lo; registers (r0 = lanes 0-7, r1 = lanes 8-15) of
-              // columns 8 blk + 4 (q / 2) ..
-              const int e = 4 * blk + 2 * (q >> 1) + (q & 1);
-              bf16x2_scale_split(wph[2 * blk + (q >> 1)], wpl[2 * blk + (q >> 1)], r[lh][blk][q], hi[e], lo[e]);
+            for (int blk = 0; blk < 4; ++blk) {
+              const int b = 4 * th + blk;  // 16-token block of the tile
+              const int c0 = quarter * 32 + lh * 16 + (lm & 1) * 8;
+              const int tokr = 16 * b + (lm >> 1) * 8 + lr;
+              const uint32_t addr = vt + (c0 >> 6) * GR_BOX + sw128_off(tokr, (c0 & 63) >> 3);
+              ldsm_x4_trans(addr, r[lh][blk][0], r[lh][blk][1], r[lh][blk][2], r[lh][blk][3]);
             }
-          const uint32_t lanes = (uint32_t)(quarter * 32 + lh * 16) << 16;
-          tmem_st_16x128b_x8(acol + lanes + 32 * th, hi);
-          tmem_st_16x128b_x8(acol + lanes + 64 + 32 * th, lo);
+#pragma unroll
+          for (int lh = 0; lh < 2; ++lh) {
+            // one 32-column slab (4 token blocks) of hi and of lo, built in
+            // registers and written with one wide store each
+            uint32_t hi[16], lo[16];
+#pragma unroll
+            for (int blk = 0; blk < 4; ++blk)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                // w v = hi + lo; registers (r0 = lanes 0-7, r1 = lanes 8-15) of
+                // columns 8 blk + 4 (q / 2) ..
+                const int e = 4 * blk + 2 * (q >> 1) + (q & 1);
+                bf16x2_scale_split(wph[2 * blk + (q >> 1)], wpl[2 * blk + (q >> 1)], r[lh][blk][q], hi[e], lo[e]);
+              }
+            const uint32_t lanes = (uint32_t)(quarter * 32 + lh * 16) << 16;
+            tmem_st_16x128b_x8(acol + lanes + 32 * th, hi);
+            tmem_st_16x128b_x8(acol + lanes + 64 + 32 * th, lo);
+          }
         }
         tmem_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&afull[ab]));
+        if (lane == 0) mbar_arrive(smem_u32(&afull[grp]));
         TRC_ADD(9, tr_b);
       }
     }
@@ -372,7 +390,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
       for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
         const int vs = it % GR_VST;
         TRC_T(tr_v);
-        if (!mbar_wait(smem_u32(&vfull[vs]), (it / GR_VST) & 1, ws, abort)) goto weights_done;
+        if (!mbar_wait(smem_u32(&vfull[C::bar(it)]), C::parity(it), ws, abort)) goto weights_done;
         TRC_ADD(11, tr_v);
         TRC_T(tr_b);
         const LkTile lt = lk_tile<G>(dm, item, t);
@@ -408,7 +426,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
           wout[i] = word;
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&wready[vs]));
+        if (lane == 0) mbar_arrive(smem_u32(&wready[C::bar(it)]));
         TRC_ADD(12, tr_b);
       }
       if (FUSED) {  // this warp's weights of the item are stored: its share of the unit's progress
