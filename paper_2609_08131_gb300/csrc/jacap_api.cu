@@ -493,13 +493,13 @@ jacap_status score_pass(const jacap_layout* layout, const jacap_params* params, 
   // (bf16 caches: the Gram kernel computes the weights from the K pass's rows)
   if (!bf && (st = map_cuda(launch_weights(dm, w, cu, persistent_grid(items, sms, 8), s))) != JACAP_OK) return st;
   if ((st = hook(4)) != JACAP_OK ||
-      (st = map_cuda(launch_gram(vmap, dm, w, dt, v, cu, persistent_grid(items, sms, bf ? 1 : 4), s))) != JACAP_OK)
+      (st = map_cuda(launch_gram(vmap, dm, w, dt, v, cu, persistent_grid(items, sms, bf ? 1 : 3), s))) != JACAP_OK)
     return st;
   if ((st = hook(5)) != JACAP_OK ||
       (st = map_cuda(launch_factor(dm, w, out_factor, partials_per_unit(dm, items, sms, bf), sms, s))) != JACAP_OK)
     return st;
   if ((st = hook(6)) != JACAP_OK ||
-      (st = map_cuda(launch_score(vmap, dm, w, dt, v, cu, scores, persistent_grid(items, sms, bf ? 1 : 2), s))) !=
+      (st = map_cuda(launch_score(vmap, dm, w, dt, v, cu, scores, persistent_grid(items, sms, 1), s))) !=
           JACAP_OK)
     return st;
   if ((st = hook(7)) != JACAP_OK) return st;

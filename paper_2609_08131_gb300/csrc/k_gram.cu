@@ -90,74 +90,77 @@ __global__ void __launch_bounds__(GR_THREADS, 1)
 }
 
 // ------------------------------------------------------------ SIMT fp32 ---
-// float32 caches: thread t accumulates the 8x8 block (rows 8*(t/16), cols
-// 8*(t%16)) of the chunk's partial Gram over 32-token slabs staged in SMEM.
-constexpr int GF_THREADS = 256;
-constexpr int GF_SLAB = 32;
+// float32 caches: a thread accumulates one 8 x 4 tile that reaches the Gram's
+// diagonal or lies below it (272 tiles, rows 8 ty .., columns 4 cx ..; nine warps
+// spread evenly over the sub-partitions) over 128-token tiles of V in
+// shared memory, fetched with 16-byte asynchronous copies (three CTAs per SM cover
+// each other's fetches). Bound: float32 multiply-adds, 32 per token and thread
+// beside three 16-byte shared-memory reads. 8 x 4096 tokens: 0.039 -> 0.025 ms
+// against all 256 tiles over slabs of 32 tokens staged through registers.
+constexpr int GF_THREADS = 288;
+constexpr int GF_TILES = 272;
 constexpr int GF_LD = D + 4;
+constexpr size_t GF_SMEM = ((size_t)TILE * GF_LD + TILE) * sizeof(float);
 
-__global__ void __launch_bounds__(GF_THREADS)
+__global__ void __launch_bounds__(GF_THREADS, 3)
     gram_f32_kernel(Dims dm, Ws ws, const int32_t* __restrict__ cu, const float* __restrict__ v) {
   pdl_wait();
-  __shared__ __align__(16) float xs[GF_SLAB][GF_LD];  // w_i v_i (16-byte rows: GF_LD is a multiple of 4)
-  __shared__ __align__(16) float vs[GF_SLAB][GF_LD];  // v_i
-  __shared__ float wsl[GF_SLAB];
+  extern __shared__ __align__(16) float gsm[];
+  float* vs = gsm;                 // [TILE][GF_LD]
+  float* wsl = gsm + TILE * GF_LD;  // [TILE]
   __shared__ int s_skip;
   const int tid = threadIdx.x;
   if (tid == 0) s_skip = status_failed(ws) ? 1 : 0;
   __syncthreads();
   if (s_skip) return;
-  const int rb = tid / 16, cb = tid % 16;
+  // tiles 0 .. ty (ty + 1) - 1 lie in the tile rows above ty
+  int ty = (int)((sqrtf(4.f * (float)tid + 1.f) - 1.f) * 0.5f);
+  while (ty * (ty + 1) > tid) --ty;
+  while ((ty + 1) * (ty + 2) <= tid) ++ty;
+  const int cx = tid - ty * (ty + 1);
+  const bool own = tid < GF_TILES;
   Item item;
   for (ItemStream is(dm, ws, blockIdx.x, gridDim.x); is.next(item);) {
     const int l = item.plane / dm.Hkv, g = item.plane % dm.Hkv;
     const float* vbase = v + (int64_t)l * dm.kv_sl + (int64_t)g * dm.kv_sh;
-    float2 acc[8][4];  // columns (2 q, 2 q + 1) of row p, packed multiply-adds
+    float2 acc[8][2];  // columns (2 q, 2 q + 1) of row p
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
-    for (int64_t t = item.t0; t < item.t1; t += GF_SLAB) {
-      if (tid < GF_SLAB) {
-        const int64_t tok = t + tid;
-        wsl[tid] = tok < item.t1 ? ws.w[(int64_t)item.plane * dm.Ntot + tok] : 0.f;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int e = tid; e < GF_SLAB * (D / 4); e += GF_THREADS) {  // all loads in flight before the stores
+    for (int p = 0; p < 8; ++p) acc[p][0] = acc[p][1] = make_float2(0.f, 0.f);
+    for (int64_t t = item.t0; t < item.t1; t += TILE) {
+      const int nv = (int)(item.t1 - t < TILE ? item.t1 - t : TILE);
+      for (int e = tid; e < TILE * (D / 4); e += GF_THREADS) {
         const int r = e / (D / 4), c4 = (e % (D / 4)) * 4;
-        const int64_t tok = t + r;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tok < item.t1) x = *(const float4*)(vbase + tok * dm.kv_st + c4);
-        const float wt = wsl[r];
-        *(float4*)&vs[r][c4] = x;
-        *(float4*)&xs[r][c4] = make_float4(wt * x.x, wt * x.y, wt * x.z, wt * x.w);
+        cp_async16(smem_u32(vs + r * GF_LD + c4), vbase + (t + (r < nv ? r : 0)) * dm.kv_st + c4, r < nv);
       }
+      if (tid < TILE) wsl[tid] = tid < nv ? ws.w[(int64_t)item.plane * dm.Ntot + t + tid] : 0.f;
+      cp_async_commit();
+      cp_async_wait<0>();
       __syncthreads();
-#pragma unroll 4
-      for (int r = 0; r < GF_SLAB; ++r) {
-        const float4 a0 = *(const float4*)&vs[r][rb * 8], a1 = *(const float4*)&vs[r][rb * 8 + 4];
-        const float4 b0 = *(const float4*)&xs[r][cb * 8], b1 = *(const float4*)&xs[r][cb * 8 + 4];
-        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
-                             make_float2(b1.z, b1.w)};
+      if (own) {
+#pragma unroll 2
+        for (int r = 0; r < nv; ++r) {
+          const float wt = wsl[r];
+          const float4 a0 = *(const float4*)(vs + r * GF_LD + 8 * ty), a1 = *(const float4*)(vs + r * GF_LD + 8 * ty + 4);
+          const float4 b = *(const float4*)(vs + r * GF_LD + 4 * cx);
+          const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+          const float2 x[2] = {make_float2(wt * b.x, wt * b.y), make_float2(wt * b.z, wt * b.w)};  // w v of the columns
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
+          for (int p = 0; p < 8; ++p)
 #pragma unroll
-          for (int q = 0; q < 4; ++q) acc[p][q] = __ffma2_rn(make_float2(a[p], a[p]), b[q], acc[p][q]);
+            for (int q = 0; q < 2; ++q) acc[p][q] = __ffma2_rn(make_float2(a[p], a[p]), x[q], acc[p][q]);
+        }
       }
-      __syncthreads();
+      __syncthreads();  // the tile is read before the next one lands on it
     }
     float* dst = ws.gpart + ((int64_t)item.plane * dm.c_cap + item.cidx) * D * D;
     if (tid == 0) ws.pflag[(int64_t)item.plane * dm.c_cap + item.cidx] = 1;  // a partial per chunk here
-    if ((rb * 8) >> 5 < (cb * 8) >> 5) continue;  // upper 32 x 32 blocks: not read (symmetry)
+    if (own) {
 #pragma unroll
-    for (int p = 0; p < 8; ++p) {
-      // (m, n) at ((n / 32) D + m) 32 + n % 32; the 8 columns share one block
-      const int m = rb * 8 + p, n0 = cb * 8;
-      float* row = dst + ((n0 >> 5) * D + m) * 32 + (n0 & 31);
-      *(float4*)row = make_float4(acc[p][0].x, acc[p][0].y, acc[p][1].x, acc[p][1].y);
-      *(float4*)(row + 4) = make_float4(acc[p][2].x, acc[p][2].y, acc[p][3].x, acc[p][3].y);
+      for (int p = 0; p < 8; ++p) {
+        // (m, n) at ((n / 32) D + m) 32 + n % 32
+        *(float4*)(dst + ((cx >> 3) * D + 8 * ty + p) * 32 + (cx & 7) * 4) =
+            make_float4(acc[p][0].x, acc[p][0].y, acc[p][1].x, acc[p][1].y);
+      }
     }
   }
 }
@@ -246,7 +249,8 @@ cudaError_t launch_gram(const CUtensorMap& vmap, const Dims& dm, const Ws& ws, i
       default: return cudaErrorInvalidValue;
     }
   } else {
-    JACAP_TRY(launch_pdl(dm.pdl != 0, gram_f32_kernel, grid, GF_THREADS, 0, st, dm, ws, cu, (const float*)v));
+    JACAP_TRY(cudaFuncSetAttribute(gram_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GF_SMEM));
+    JACAP_TRY(launch_pdl(dm.pdl != 0, gram_f32_kernel, grid, GF_THREADS, GF_SMEM, st, dm, ws, cu, (const float*)v));
   }
   return cudaGetLastError();
 }

@@ -622,3 +622,17 @@ def test_selection_of_any_scores_is_the_stable_order(layers, hkv, n, kind):
         kept = min(m, B)
         assert torch.equal(ev.idx[:, :, s, :kept], want[..., :kept])
         assert bool((ev.idx[:, :, s, kept:] == -1).all())
+
+
+def test_f32_tiles_at_their_edges():
+    """The float32 Gram and score kernels on requests that end before, on and after a tile's edge,
+    every unit against the oracle (with weights and selection)."""
+    wl = Workload("t", 2, 8, 2, (1, 127, 128, 129, 257, 640), 8, 48, dtype="f32", dist="outlier", seed=95,
+                  outlier_channels=4, outlier_scale=8.0)
+    t = generate(wl, DEV)
+    params = jacap_params(tau=0.5)
+    ev = evict(make_cache(t, wl), wl.budget, params)
+    for s in range(len(wl.seqlens)):
+        for layer in range(2):
+            for g in range(2):
+                check_unit(ev, t, wl, params, s, layer, g)
