@@ -21,10 +21,12 @@ namespace {
 constexpr size_t ALIGN = 1024;
 inline size_t align_up(size_t x) { return (x + ALIGN - 1) & ~(ALIGN - 1); }
 
+constexpr int GRAM_PARTS_MAX = 1024;  // more than a GPU has SMs
+
 struct Carve {
   size_t status, plan, chunks, counters, mu, lam, qdev, lk, cstats, ustats, w, gpart, pflag, gram, minv,
       minv_img, total;
-  size_t units, trace, trace_cta, base, runs, sched;
+  size_t units, trace, trace_cta, base, runs, sched, seqs;
 };
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -108,6 +110,7 @@ Carve carve(const Dims& dm) {
   const size_t units = planes * dm.S;
   size_t o = 0;
   c.units = units;
+  c.seqs = dm.S;
   c.status = o; o = align_up(o + 64);
   c.plan = o; o = align_up(o + ((size_t)dm.S + 2) * 4);
   c.chunks = o; o = align_up(o + (size_t)dm.c_cap * 16);
@@ -128,7 +131,8 @@ Carve carve(const Dims& dm) {
   c.minv_img = o; o = align_up(o + units * 65536);
   c.base = o;  // the static scratch's limit applies to the sections up to here (jacap_static.cu)
   c.runs = o; o = align_up(o + 2 * (size_t)dm.c_cap * 16);
-  c.sched = o; o = align_up(o + 32 + 2 * ((size_t)dm.S + 2) * 4);  // run counters, then the run prefixes
+  // run counters, run prefixes, tile prefixes, the Gram's shares
+  c.sched = o; o = align_up(o + 32 + (2 * ((size_t)dm.S + 2) + dm.S + 1 + GRAM_PARTS_MAX + 1) * 4);
 #ifdef JACAP_TRACE
   c.trace = o; o = align_up(o + units * TR_SLOTS * 8);  // trace builds: the fused schedule's timeline,
   c.trace_cta = o; o = align_up(o + (size_t)TR_KERNELS * TR_CTAS * TR_CTA_SLOTS * 8);  // then the CTA accounting
@@ -149,6 +153,8 @@ Ws make_ws(void* base, const Carve& c) {
   ws.runs = (int4*)(b + c.runs);
   ws.sched = (int32_t*)(b + c.sched);
   ws.rplan = ws.sched + 8;
+  ws.tpre = ws.rplan + 2 * ((size_t)c.seqs + 2);
+  ws.starts = ws.tpre + c.seqs + 1;
   ws.gcount = (int32_t*)(b + c.counters);
   ws.fdone = ws.gcount + c.units;  // right after gcount: the plan kernel zeroes 2 x units words
   ws.mu = (float*)(b + c.mu);
@@ -436,6 +442,7 @@ jacap_status score_pass(const jacap_layout* layout, const jacap_params* params, 
   const int64_t items = pass_items(layout, dm);
   if (items >= ((int64_t)1 << 31)) return JACAP_ERR_UNSUPPORTED;
   pick_runs(dm, items, sms);
+  dm.gram_parts = std::min(persistent_grid(items, sms, 1), GRAM_PARTS_MAX);
   const int dt = bf ? 1 : 0;
   const int32_t* cu = layout->cu_seqlens;
   // hook(i): the boundary before kernel i (optional timing event; with
@@ -493,7 +500,8 @@ jacap_status score_pass(const jacap_layout* layout, const jacap_params* params, 
   // (bf16 caches: the Gram kernel computes the weights from the K pass's rows)
   if (!bf && (st = map_cuda(launch_weights(dm, w, cu, persistent_grid(items, sms, 8), s))) != JACAP_OK) return st;
   if ((st = hook(4)) != JACAP_OK ||
-      (st = map_cuda(launch_gram(vmap, dm, w, dt, v, cu, persistent_grid(items, sms, bf ? 1 : 3), s))) != JACAP_OK)
+      (st = map_cuda(launch_gram(vmap, dm, w, dt, v, cu, bf ? dm.gram_parts : persistent_grid(items, sms, 3), s))) !=
+          JACAP_OK)
     return st;
   if ((st = hook(5)) != JACAP_OK ||
       (st = map_cuda(launch_factor(dm, w, out_factor, partials_per_unit(dm, items, sms, bf), sms, s))) != JACAP_OK)
@@ -581,7 +589,7 @@ jacap_status jacap_append(const jacap_layout* layout, const void* k_new, const v
   }
   for (int s = 0; s < layout->num_seqs; ++s)
     if (lengths[s] < 0 || lengths[s] >= layout->max_seqlen) return JACAP_ERR_INVALID_ARG;
-  if ((int64_t)layout->num_layers * layout->num_kv_heads * 256 >= ((int64_t)1 << 31)) return JACAP_ERR_INVALID_ARG;
+  if ((int64_t)layout->num_layers * layout->num_q_heads * 256 >= ((int64_t)1 << 31)) return JACAP_ERR_INVALID_ARG;
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   Dims dm;

@@ -50,6 +50,7 @@ struct Dims {
   int run_items;      // fused: consecutive items a role's CTA takes at a time (one partial Gram per run)
   int run_chunks[2];  // separate kernels: chunks per run (at most) of the first big_planes planes, and of the
   int big_planes;     // planes after them, see RunStream
+  int gram_parts;     // CTAs of the bf16 Gram (ws.starts)
 };
 
 // Rows per split part of the full-covariance query image of one KV head's
@@ -68,6 +69,8 @@ struct Ws {
   int32_t* rplan;     // two lists of runs, list m at m (S + 2): [0] = runs per plane, [1 .. S+1] = run prefix
   int4* chunks;       // [c_cap] chunk r of every plane: {t0, t1, request, r}
   int4* runs;         // [2][c_cap] run r of every plane, for each list: {t0, t1, request, first chunk}
+  int32_t* tpre;      // [S+1] tiles of a plane before each request, and in all
+  int32_t* starts;    // [gram_parts + 1] the Gram's CTA b takes items starts[b] .. starts[b + 1] - 1
   int32_t* sched;     // [8] next run of each streaming kernel beyond the first one of each CTA (SCHED_*)
   int32_t* gcount;    // [units] fused schedule: Gram progress of a unit (each item adds 1 for its weights
                       // and 1 for its partial Gram; complete at 2 x the unit's chunk count)
@@ -137,8 +140,11 @@ struct ItemStream {
   // part + parts, ..., so the CTAs of a role sweep the units in order together
   // and each unit's items finish close in time.
   int64_t run_end, skip, runlen;
+  // With `starts` (not strided) CTA `part` takes items starts[part] .. starts[part +
+  // 1] - 1: shares of equal numbers of tiles, where equal numbers of items would
+  // not be (the last chunk of each request is short).
   __device__ __forceinline__ ItemStream(const Dims& dm, const Ws& ws, int64_t part, int64_t parts,
-                                        bool strided = false)
+                                        bool strided = false, const int32_t* starts = nullptr)
       : tab(ws.chunks) {
 #ifdef JACAP_CHECKED
     ntot = dm.Ntot;
@@ -156,8 +162,8 @@ struct ItemStream {
       runlen = R;
       end = total;
     } else {
-      i = part * total / parts;
-      end = (part + 1) * total / parts;
+      i = starts != nullptr ? (int64_t)starts[part] : part * total / parts;
+      end = starts != nullptr ? (int64_t)starts[part + 1] : (part + 1) * total / parts;
       run_end = end;
       skip = 0;
       runlen = 0;

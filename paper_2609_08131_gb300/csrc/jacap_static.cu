@@ -23,7 +23,7 @@ namespace {
 
 // The scratch, one copy per device context (the module is loaded per context).
 // JACAP_STATIC_SCRATCH_BYTES is the limit on a layout's workspace without its
-// run tables; those take at most 48 bytes per chunk and request on top, and a
+// run tables; those take at most 56 bytes per chunk and request (and 4 KB) on top, and a
 // layout within the limit has at most 1024 of each (64 KB of partial Gram per
 // chunk; a request adds a chunk).
 constexpr size_t SCRATCH_BYTES = (size_t)JACAP_STATIC_SCRATCH_BYTES + 65536;

@@ -80,14 +80,16 @@ __global__ void __launch_bounds__(D)
   if (c == 0) counts[b] = na + nb;
 }
 
-// One decode step of up to AP_MAX requests: a block per (request, layer, KV head)
-// copies the new K and V rows (16-byte pieces) and the tag into the request's next
-// free slot row and merges the queries of the head's group, one channel per
-// thread, with the arithmetic of stats_update_kernel for a batch of one. Bound: the
-// launch (4 requests x 28 layers x 4 KV heads: 0.9 MB moved). One launch with the
-// rows' numbers as arguments replaces two index tensors copied from the host (each
-// a synchronisation of the stream), three indexed copies and the update: 170 -> 22 us
-// of host time a step, and the steps no longer wait for the device.
+// One decode step of up to AP_MAX requests: a block per (request, layer, query
+// head) merges the head's query into the running statistics, one channel per thread,
+// with the arithmetic of stats_update_kernel for a batch of one; the first head of a
+// group's block also copies the new K and V rows (16-byte pieces) and the tag into
+// the request's next free slot row. Bound: the launch and two dependent reads (4
+// requests x 28 layers x 28 heads: 4 us; a block per KV head that took its seven
+// heads in turn: 16 us). One launch with the rows' numbers as arguments replaces two
+// index tensors copied from the host (each a synchronisation of the stream), three
+// indexed copies and the update: 170 -> 20 us of host time a step, and the steps no
+// longer wait for the device.
 constexpr int AP_MAX = 256;
 struct AppendRows {
   int32_t row[AP_MAX], id[AP_MAX];
@@ -98,38 +100,39 @@ __global__ void __launch_bounds__(D)
     append_kernel(Dims dm, AppendArgs a, const __grid_constant__ AppendRows rows, int s0) {
   pdl_wait();
   const int b = blockIdx.x, tid = threadIdx.x;
-  const int g = b % dm.Hkv, l = (b / dm.Hkv) % dm.L, sl = b / (dm.Hkv * dm.L), s = s0 + sl;
-  constexpr int CH = D * (int)sizeof(T) / 16;  // 16-byte pieces of a row
-  const int64_t row = (int64_t)s * a.slot_rows + rows.row[sl];
-  if (tid < 2 * CH) {
-    const bool isv = tid >= CH;
-    const int p = isv ? tid - CH : tid;
-    const int64_t* st = a.strides + (isv ? 3 : 0);
-    const T* src = (const T*)(isv ? a.v_new : a.k_new) + s * st[0] + l * st[1] + g * st[2];
-    T* dst = (T*)(isv ? a.v : a.k) + (int64_t)l * dm.kv_sl + (int64_t)g * dm.kv_sh + row * dm.kv_st;
-    ((uint4*)dst)[p] = ((const uint4*)src)[p];
-  } else if (tid == 2 * CH && a.pos != nullptr) {
-    a.pos[(int64_t)l * (dm.kv_sl / dm.kv_st) + (int64_t)g * (dm.kv_sh / dm.kv_st) + row] = rows.id[sl];
-  }
-  for (int h = 0; h < dm.G; ++h) {
-    const int hq = g * dm.G + h;
-    const int64_t sb = ((int64_t)s * dm.L + l) * dm.Hq + hq;
-    const float x = q_elem((const T*)a.q_new + s * dm.q_ss + l * dm.q_sl + hq * dm.q_sh + tid);
-    float* st = a.stats + sb * 2 * D;
-    int na = a.counts[sb];
-    if (na < 0) na = 0;
-    float mean = x, m2 = 0.f;
-    if (na > 0) {
-      const float n = (float)na + 1.f;
-      const float ma = st[tid], delta = x - ma;
-      mean = fmaf(delta, 1.f / n, ma);
-      m2 = st[D + tid] + delta * delta * ((float)na / n);
+  const int hq = b % dm.Hq, l = (b / dm.Hq) % dm.L, sl = b / (dm.Hq * dm.L), s = s0 + sl;
+  const int64_t sb = ((int64_t)s * dm.L + l) * dm.Hq + hq;
+  float* st = a.stats + sb * 2 * D;
+  const float x = q_elem((const T*)a.q_new + s * dm.q_ss + l * dm.q_sl + hq * dm.q_sh + tid);
+  const float ma = st[tid], sa = st[D + tid];
+  int na = a.counts[sb];
+  if (hq % dm.G == 0) {
+    constexpr int CH = D * (int)sizeof(T) / 16;  // 16-byte pieces of a row
+    const int g = hq / dm.G;
+    const int64_t row = (int64_t)s * a.slot_rows + rows.row[sl];
+    if (tid < 2 * CH) {
+      const bool isv = tid >= CH;
+      const int p = isv ? tid - CH : tid;
+      const int64_t* str = a.strides + (isv ? 3 : 0);
+      const T* src = (const T*)(isv ? a.v_new : a.k_new) + s * str[0] + l * str[1] + g * str[2];
+      T* dst = (T*)(isv ? a.v : a.k) + (int64_t)l * dm.kv_sl + (int64_t)g * dm.kv_sh + row * dm.kv_st;
+      ((uint4*)dst)[p] = ((const uint4*)src)[p];
+    } else if (tid == 2 * CH && a.pos != nullptr) {
+      a.pos[(int64_t)l * (dm.kv_sl / dm.kv_st) + (int64_t)g * (dm.kv_sh / dm.kv_st) + row] = rows.id[sl];
     }
-    __syncthreads();  // every thread has read counts before it changes
-    st[tid] = mean;
-    st[D + tid] = m2;
-    if (tid == 0) a.counts[sb] = na + 1;
   }
+  if (na < 0) na = 0;
+  float mean = x, m2 = 0.f;
+  if (na > 0) {
+    const float n = (float)na + 1.f;
+    const float delta = x - ma;
+    mean = fmaf(delta, 1.f / n, ma);
+    m2 = sa + delta * delta * ((float)na / n);
+  }
+  __syncthreads();  // every thread has read counts before it changes
+  st[tid] = mean;
+  st[D + tid] = m2;
+  if (tid == 0) a.counts[sb] = na + 1;
 }
 
 // The scoring pass's query statistics from running statistics: the same
@@ -234,7 +237,7 @@ cudaError_t launch_append(const Dims& dm, int dtype, const AppendArgs& a, const 
       rows.row[i] = i < n ? lengths[s0 + i] : 0;
       rows.id[i] = i < n ? ids[s0 + i] : 0;
     }
-    const int blocks = n * dm.L * dm.Hkv;
+    const int blocks = n * dm.L * dm.Hq;
     if (dtype == 1)
       JACAP_TRY(launch_pdl(dm.pdl != 0, append_kernel<__nv_bfloat16>, blocks, D, 0, st, dm, a, rows, s0));
     else

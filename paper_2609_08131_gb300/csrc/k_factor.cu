@@ -486,16 +486,34 @@ __global__ void __launch_bounds__(FR_THREADS) gram_reduce_kernel(Dims dm, Ws ws)
   float* gp = ws.gpart + ((int64_t)plane * dm.c_cap) * D * D + (nb * D + 32 * I) * 32 + 4 * tid;
   const int32_t* pf = ws.pflag + (int64_t)plane * dm.c_cap;
   float4 acc = *(const float4*)(gp + (int64_t)ch0 * D * D);
-  constexpr int N = 8;  // loads in flight
-  for (int c = ch0 + 1; c < ch1; c += N) {
-    float4 v[N];
+  __shared__ int s_list[FR_THREADS], s_cnt[FR_THREADS / 32];
+  const int lane = tid & 31, warp = tid >> 5;
+  for (int base = ch0 + 1; base < ch1; base += FR_THREADS) {
+    // the chunks that hold a partial
+    const bool has = base + tid < ch1 && pf[base + tid] != 0;
+    const uint32_t b = __ballot_sync(0xffffffffu, has);
+    __syncthreads();
+    if (lane == 0) s_cnt[warp] = __popc(b);
+    __syncthreads();
+    int at = 0, n = 0;
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (c + k < ch1 && pf[c + k] != 0) v[k] = *(const float4*)(gp + (int64_t)(c + k) * D * D);
+    for (int w = 0; w < FR_THREADS / 32; ++w) {
+      if (w < warp) at += s_cnt[w];
+      n += s_cnt[w];
     }
+    if (has) s_list[at + __popc(b & ((1u << lane) - 1u))] = base + tid;
+    __syncthreads();
+    constexpr int N = 16;  // loads in flight
+    for (int k0 = 0; k0 < n; k0 += N) {
+      float4 v[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) acc.x += v[k].x, acc.y += v[k].y, acc.z += v[k].z, acc.w += v[k].w;
+      for (int k = 0; k < N; ++k) {
+        v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k0 + k < n) v[k] = *(const float4*)(gp + (int64_t)s_list[k0 + k] * D * D);
+      }
+#pragma unroll
+      for (int k = 0; k < N; ++k) acc.x += v[k].x, acc.y += v[k].y, acc.z += v[k].z, acc.w += v[k].w;
+    }
   }
   *(float4*)(gp + (int64_t)ch0 * D * D) = acc;
 }

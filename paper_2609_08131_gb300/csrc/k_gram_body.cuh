@@ -188,7 +188,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
       uint32_t it = 0;
       bool ok = true;
       Item item;
-      for (ItemStream is(dm, ws, part, parts, FUSED); ok && is.next(item);) {
+      for (ItemStream is(dm, ws, part, parts, FUSED, FUSED ? nullptr : ws.starts); ok && is.next(item);) {
         const int l = item.plane / dm.Hkv, g = item.plane % dm.Hkv;
         if (FUSED) JACAP_TRACE_MIN(ws, (int64_t)item.plane * dm.S + item.seq, TR_GRAM0);
         for (int64_t t = item.t0; t < item.t1; t += TILE) {
@@ -233,7 +233,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
       uint32_t it = 0, nrun = 0;
       bool ok = true, cont = false, first = true;
       Item item;
-      for (ItemStream is(dm, ws, part, parts, FUSED); ok && is.next(item);) {
+      for (ItemStream is(dm, ws, part, parts, FUSED, FUSED ? nullptr : ws.starts); ok && is.next(item);) {
         // a run of consecutive chunks of a unit accumulates in the accumulator
         // pair; a new run starts on it once the previous run's epilogue has read it
         if (!cont) {
@@ -293,7 +293,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
     TRC_T(tr_all);
     uint32_t it = 0;
     Item item;
-    for (ItemStream is(dm, ws, part, parts, FUSED); is.next(item);) {
+    for (ItemStream is(dm, ws, part, parts, FUSED, FUSED ? nullptr : ws.starts); is.next(item);) {
       for (int64_t t = item.t0; t < item.t1; t += TILE, ++it) {
         if ((int)(it & 1) != grp) continue;
         const int vs = it % GR_VST;
@@ -383,7 +383,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
 #pragma unroll
     for (int e = 0; e < 2 * G; ++e) u[e] = 0.f;
     Item item;
-    for (ItemStream is(dm, ws, part, parts, FUSED); is.next(item);) {
+    for (ItemStream is(dm, ws, part, parts, FUSED, FUSED ? nullptr : ws.starts); is.next(item);) {
       if (!cont && !dm.linear) load_unit_stats<G>(dm, ws, item.plane, item.seq, u);
       cont = is.next_same_unit(item);
       const int64_t base = (int64_t)item.plane * dm.Ntot;
@@ -453,7 +453,7 @@ __device__ __forceinline__ void gram_bf16_body(const CUtensorMap* vmap_p, const 
     bool cont = false;
     int run_cidx = 0, run_items = 0;
     Item item;
-    for (ItemStream is(dm, ws, part, parts, FUSED); is.next(item);) {
+    for (ItemStream is(dm, ws, part, parts, FUSED, FUSED ? nullptr : ws.starts); is.next(item);) {
       // the partial of a run goes to its first chunk; pflag marks which
       // chunks hold one
       if (!cont) {
