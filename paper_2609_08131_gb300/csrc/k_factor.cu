@@ -25,14 +25,15 @@
 // one vector each into u (two barriers a step), and every tile below makes the
 // same rank-4 update.
 //
-// Bound: the chain of the 32 steps, 1360 cycles each alone on an SM (barriers 170,
+// Bound: the chain of the 32 steps, 1240 cycles each alone on an SM (barriers 170,
 // vectors left and turned into u 500, the pivot block's four reciprocals 170, the
-// update 520, of which the reads of u from shared memory are the larger part) and
-// 840 (700) per unit with two (three) CTAs on an SM. Measured against blocked
-// 32 x 32 eliminations of one warp each, with the blocks in shared memory: 256
-// units 0.055 -> 0.045 ms, 448 units 0.082 -> 0.061, 1024 units 0.173 -> 0.135;
-// output directions, 128 units, 0.124 -> 0.082 ms. 8 x 8 tiles whose owners formed
-// u themselves took 0.061 and 0.192 ms (two lanes a warp formed eight vectors each).
+// update 400) and 760 (650, 610) per unit with two (three, four) CTAs on an SM;
+// with many units also the 192 KB that each writes. Measured against blocked 32 x 32
+// eliminations of one warp each, with the blocks in shared memory: 256 units 0.055 ->
+// 0.042 ms, 448 units 0.082 -> 0.060, 1024 units 0.173 -> 0.120; output directions,
+// 128 units, 0.124 -> 0.080 ms. 8 x 8 tiles whose owners formed u themselves took
+// 0.061 and 0.192 ms (two lanes a warp formed eight vectors each); tiles paired by
+// columns, whose rows' values all had to be doubled, 1360 cycles a step.
 //
 // With output directions u = W v (Sec. 3.1) the capacity matrix I + sum w u u^T
 // lives in the output space; with a 128 x 128 factor F of W^T W (F^T F = W^T W)
@@ -59,24 +60,29 @@ namespace jacap {
 constexpr int FT_TILES = 272;     // tiles (ty, cx), cx <= 2 ty + 1
 constexpr int FT_THREADS = 288;
 
-// A step's vectors: raw by index, u by component (ut) and negated by row (ur,
-// with 16 bytes between the tile rows, so that a warp's rows fall in different
-// banks).
+// A step's vectors: raw by index (16 bytes between the tile rows, so that the rows
+// that a warp stores fall in different banks), u by component.
 struct FtSmem {
-  float4 raw[D];
+  float4 raw[D + D / 8];
   float4 linv[4];
   float ut[4][D];
-  float4 ur[D + D / 8];
   int list[FT_THREADS];
   int cnt[FT_THREADS / 32];
   int skip;
 };
 
-using Tile = float2[8][2];  // 8 rows of two column pairs
+// 4 pairs of rows, 4 columns: the packed multiply-adds of a rank-1 update then take
+// the rows' vector in pairs as it is loaded, and only the columns' 4 values doubled.
+using Tile = float2[4][4];
 
-__device__ __forceinline__ float4 tile_row(const Tile& T, int i) { return make_float4(T[i][0].x, T[i][0].y, T[i][1].x, T[i][1].y); }
 __device__ __forceinline__ float& tile_at(Tile& T, int i, int c) {  // i, c known after unrolling
-  return (c & 1) ? T[i][c >> 1].y : T[i][c >> 1].x;
+  return (i & 1) ? T[i >> 1][c].y : T[i >> 1][c].x;
+}
+__device__ __forceinline__ float4 tile_row(Tile& T, int i) {
+  return make_float4(tile_at(T, i, 0), tile_at(T, i, 1), tile_at(T, i, 2), tile_at(T, i, 3));
+}
+__device__ __forceinline__ void tile_set_row(Tile& T, int i, const float4 v) {
+  tile_at(T, i, 0) = v.x, tile_at(T, i, 1) = v.y, tile_at(T, i, 2) = v.z, tile_at(T, i, 3) = v.w;
 }
 
 // 1 / sqrt(x): the hardware's approximation refined by one Newton-Raphson step;
@@ -127,8 +133,8 @@ template <int O>
 __device__ __forceinline__ void leave_rows(Tile& T, FtSmem& sm, int ty) {
 #pragma unroll
   for (int i = O; i < O + 4; ++i) {
-    sm.raw[8 * ty + i] = tile_row(T, i);
-    T[i][0] = T[i][1] = make_float2(0.f, 0.f);
+    sm.raw[9 * ty + i] = tile_row(T, i);
+    tile_set_row(T, i, make_float4(0.f, 0.f, 0.f, 0.f));
   }
 }
 
@@ -148,26 +154,30 @@ __device__ __forceinline__ void leave_vectors(Tile& T, FtSmem& sm, int p, int ty
   } else if (ty == p && cx < b) {
 #pragma unroll
     for (int v = 0; v < 4; ++v)
-      sm.raw[4 * cx + v] = make_float4(tile_at(T, 4 * H, v), tile_at(T, 4 * H + 1, v), tile_at(T, 4 * H + 2, v),
+      sm.raw[4 * cx + (cx >> 1) + v] = make_float4(tile_at(T, 4 * H, v), tile_at(T, 4 * H + 1, v), tile_at(T, 4 * H + 2, v),
                                        tile_at(T, 4 * H + 3, v));
   }
 }
 
-// Rows O .. O + 3 of the tile: Z_rc -= u_r . u_c. The loads of the rows' vectors
-// are in flight together.
+// Rows O .. 7 of the tile: Z_rc -= u_r . u_c.
 template <int O>
-__device__ __forceinline__ void update_rows(Tile& T, const FtSmem& sm, const float2 (&uc)[4][2], int ty) {
-  float4 a[4];
+__device__ __forceinline__ void update_rows(Tile& T, const FtSmem& sm, int ty, int cx) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) a[i] = sm.ur[9 * ty + O + i];
+  for (int j = 0; j < 4; ++j) {
+    const float4 c = *(const float4*)&sm.ut[j][4 * cx];
+    const float2 n[4] = {make_float2(-c.x, -c.x), make_float2(-c.y, -c.y), make_float2(-c.z, -c.z),
+                         make_float2(-c.w, -c.w)};
+    float4 r[2];
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
+    for (int h = O / 4; h < 2; ++h) r[h] = *(const float4*)&sm.ut[j][8 * ty + 4 * h];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float x = j == 0 ? a[i].x : (j == 1 ? a[i].y : (j == 2 ? a[i].z : a[i].w));
+    for (int h = O / 4; h < 2; ++h)
 #pragma unroll
-      for (int c = 0; c < 2; ++c) T[O + i][c] = __ffma2_rn(make_float2(x, x), uc[j][c], T[O + i][c]);
-    }
+      for (int e = 0; e < 4; ++e) {
+        T[2 * h][e] = __ffma2_rn(make_float2(r[h].x, r[h].y), n[e], T[2 * h][e]);
+        T[2 * h + 1][e] = __ffma2_rn(make_float2(r[h].z, r[h].w), n[e], T[2 * h + 1][e]);
+      }
+  }
 }
 
 template <int H>
@@ -176,7 +186,7 @@ __device__ __forceinline__ void eliminate_step(Tile& T, FtSmem& sm, int p, int t
   named_barrier_sync(1, FT_THREADS);
   if (tid < D) {
     const float4 m0 = sm.linv[0], m1 = sm.linv[1], m2 = sm.linv[2], m3 = sm.linv[3];
-    float4 x = sm.raw[tid];
+    float4 x = sm.raw[tid + (tid >> 3)];
     const int e = tid - 4 * b;  // in the block: a unit vector
     if (e >= 0 && e < 4) x = make_float4(e == 0 ? 1.f : 0.f, e == 1 ? 1.f : 0.f, e == 2 ? 1.f : 0.f, e == 3 ? 1.f : 0.f);
     const float u0 = m0.x * x.x;
@@ -187,23 +197,15 @@ __device__ __forceinline__ void eliminate_step(Tile& T, FtSmem& sm, int p, int t
     sm.ut[1][tid] = u1;
     sm.ut[2][tid] = u2;
     sm.ut[3][tid] = u3;
-    sm.ur[tid + (tid >> 3)] = make_float4(-u0, -u1, -u2, -u3);
   }
   named_barrier_sync(1, FT_THREADS);
   if (ty >= p) {
-    float2 uc[4][2];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float4 a = *(const float4*)&sm.ut[j][4 * cx];
-      uc[j][0] = make_float2(a.x, a.y), uc[j][1] = make_float2(a.z, a.w);
-    }
     if (ty > p) {
-      update_rows<0>(T, sm, uc, ty);
-      update_rows<4>(T, sm, uc, ty);
-    } else {  // the block's rows are final; below it in the tile: rows 4 .. 7 (H == 0)
+      update_rows<0>(T, sm, ty, cx);
+    } else {  // below the block in the tile: rows 4 .. 7 (H == 0); the block's rows are final
+      if (H == 0) update_rows<4>(T, sm, ty, cx);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) T[4 * H + j][0] = uc[j][0], T[4 * H + j][1] = uc[j][1];
-      if (H == 0) update_rows<4>(T, sm, uc, ty);
+      for (int j = 0; j < 4; ++j) tile_set_row(T, 4 * H + j, *(const float4*)&sm.ut[j][4 * cx]);
     }
     if (H == 0) leave_vectors<1>(T, sm, p, ty, cx, bad);
     else if (p < 15) leave_vectors<0>(T, sm, p + 1, ty, cx, bad);
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
   // global memory (layout: (m, n) at ((n / 32) D + m) 32 + n % 32)
   Tile T;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) T[i][0] = T[i][1] = make_float2(0.f, 0.f);
+  for (int i = 0; i < 8; ++i) tile_set_row(T, i, make_float4(0.f, 0.f, 0.f, 0.f));
   {
     const float* gp = ws.gpart + ((int64_t)plane * dm.c_cap) * D * D + ((cx >> 3) * D + 8 * ty) * 32 + (cx & 7) * 4;
     const int32_t* pf = ws.pflag + (int64_t)plane * dm.c_cap;
@@ -338,8 +340,8 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
           for (int i = 0; i < 8; ++i) v[i] = *(const float4*)(src + i * 32);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            T[i][0].x += v[i].x, T[i][0].y += v[i].y;
-            T[i][1].x += v[i].z, T[i][1].y += v[i].w;
+            tile_at(T, i, 0) += v[i].x, tile_at(T, i, 1) += v[i].y;
+            tile_at(T, i, 2) += v[i].z, tile_at(T, i, 3) += v[i].w;
           }
         }
       __syncthreads();  // the list is read before the next round writes it
@@ -392,7 +394,7 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const float4 v = *(const float4*)(R0 + (8 * ty + i) * FT_LD + 4 * cx);
-        T[i][0] = make_float2(v.x, v.y), T[i][1] = make_float2(v.z, v.w);
+        tile_set_row(T, i, v);
       }
     }
     __syncthreads();
@@ -528,9 +530,18 @@ cudaError_t launch_factor(const Dims& dm, const Ws& ws, const float* out_factor,
     JACAP_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FT_PROJ_SMEM));
     JACAP_TRY(launch_pdl(dm.pdl != 0, kern, units, FT_THREADS, FT_PROJ_SMEM, st, dm, ws, out_factor, reduced));
   } else {
-    // three CTAs per SM (72 registers a thread) finish 17 % more units in the
-    // same time than two (96), but each later: worth it beyond one wave of two
-    auto kern = units > 2 * sms ? factor_kernel<false, 3> : factor_kernel<false, 2>;
+    // CTAs per SM (2, 3 or 4; with 96, 72 or 56 registers a thread): more of them
+    // finish more units in the same time but each later, and all units of a round
+    // end together, so the choice is the least rounds x time of a round in us (256
+    // units: 38 with two; 448: 55 with three, 65 with two; 1024: 115 with four, 128
+    // with three, 150 with two)
+    constexpr int ROUND_US[3] = {38, 50, 58};
+    int best = 0;
+    for (int i = 0; i < 3; ++i) {
+      auto cost = [&](int k) { return (int64_t)((units + (k + 2) * sms - 1) / ((k + 2) * sms)) * ROUND_US[k]; };
+      if (cost(i) < cost(best)) best = i;
+    }
+    auto kern = best == 0 ? factor_kernel<false, 2> : (best == 1 ? factor_kernel<false, 3> : factor_kernel<false, 4>);
     JACAP_TRY(launch_pdl(dm.pdl != 0, kern, units, FT_THREADS, 0, st, dm, ws, out_factor, reduced));
   }
   return cudaGetLastError();
