@@ -286,6 +286,32 @@ __device__ __forceinline__ void load_floats(float* v, const float* src) {
   for (; e < N; ++e) v[e] = src[e];
 }
 
+// The logits/kappa rows (2 G floats) of a tile's tokens 32 quarter + lane from the
+// lanes of a warp to lkp, the plane's rows (tokens t .., those before t1). They are
+// contiguous there: through shared memory (`rows`, the tile's), so that each store
+// instruction writes whole lines (a lane's own row written by itself costs 2 G / V
+// instructions of 32 partial sectors). All lanes.
+template <int G>
+__device__ __forceinline__ void store_rows(float* lkp, float* rows, const float (&row)[2 * G], int64_t t, int64_t t1,
+                                           int quarter, int lane) {
+  constexpr int V = LkAlign<G>::ROW;
+  float* wrows = rows + quarter * 32 * 2 * G;
+  store_floats<2 * G, V>(wrows + lane * 2 * G, row);
+  __syncwarp();
+  const int64_t left = t1 - t - 32 * quarter;
+  const int nf = (int)(left < 0 ? 0 : (left < 32 ? left : 32)) * 2 * G;
+  float* dst = lkp + (t + 32 * quarter) * (2 * G);
+#pragma unroll
+  for (int e = 0; e < 2 * G / V; ++e) {
+    const int f = (lane + 32 * e) * V;
+    if (f < nf) {
+      if constexpr (V == 4) *(float4*)(dst + f) = *(const float4*)(wrows + f);
+      else *(float2*)(dst + f) = *(const float2*)(wrows + f);
+    }
+  }
+  __syncwarp();
+}
+
 // Programmatic dependent launch. A kernel launched with the programmatic
 // stream-serialization attribute is set up while the previous kernel of the
 // stream still runs and is scheduled as its CTAs exit (no kernel here triggers

@@ -29,6 +29,12 @@
 // sum the delta columns per head, add the three logit parts, keep the online
 // (max, sum exp) and write the token's logits/kappa row in one piece.
 //
+// Bound: the MMAs (16 of N = rp + nb per tile, ~0.56 us at G w = 128) beside HBM.
+// A run starts behind the single image, so its mu' is read before the image's
+// buffer is free and split from registers; rows leave in whole lines. 16 x 8 x 16384
+// tokens (G = 4, w = 32): 0.121 -> 0.104 ms against mu' rows read value by value
+// (~8 us per run).
+//
 // Other shapes and float32 caches: a SIMT kernel (one thread per token, the
 // tile's keys and one head's centred queries staged in shared memory).
 #include "jacap_dev.cuh"
@@ -56,37 +62,48 @@ struct KxCfg {
   static constexpr uint32_t IDESC = idesc_bf16_f32(128, N, 0, 0);
   static_assert(RP > 0 && N <= 256 && N % 16 == 0 && 2 * ACC <= KX_TMEM_COLS, "tensor-core shape");
   static_assert(SEC % 1024 == 0, "sections start on a swizzle-pattern boundary");
-  static constexpr size_t SMEM = 1024 + (size_t)KX_STAGES * KX_TILE_BYTES + IMG_BYTES + 4 * 2 * G * 4 + 256;
+  static constexpr size_t SMEM = 1024 + (size_t)KX_STAGES * KX_TILE_BYTES + IMG_BYTES + TILE * 2 * G * 4 + 4 * 2 * G * 4 + 256;
 };
 
-// Rows rp .. rp + nb - 1 of section 0 of both atoms: row rp + part G + h holds
-// part (0 hi, 1 mid, 2 lo) of mu'_h with hi + mid + lo = mu'_h to about 24
-// bits; rows past 3 G are zero. One warp.
-template <int G, int W>
-__device__ __forceinline__ void write_mu_rows(uint8_t* img, const float* mu, int lane) {
-  using C = KxCfg<G, W>;
-  for (int e = lane; e < C::NB * 16; e += 32) {
-    const int n = e >> 4, cc = e & 15;  // row, 8-channel chunk
-    uint32_t wv[4] = {0u, 0u, 0u, 0u};
-    if (n < 3 * G) {
-      const int part = n / G, h = n % G;
+// mu' of the group in registers (8 channels of a head per lane and turn), and
+// from there rows rp .. rp + 3 G - 1 of section 0 of both atoms: row rp + part G + h
+// holds part (0 hi, 1 mid, 2 lo) of mu'_h with hi + mid + lo = mu'_h to about 24
+// bits. One warp; the loads come before the wait for the image's buffer.
+template <int G>
+struct MuRows {
+  static constexpr int N = (G * 16 + 31) / 32;
+  float4 v[N][2];
+  __device__ __forceinline__ void load(const float* mu, int lane) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float x[2];
-#pragma unroll
-        for (int z = 0; z < 2; ++z) {
-          const float v = mu[h * D + cc * 8 + 2 * q + z];
-          const float hi = __bfloat162float(__float2bfloat16_rn(v));
-          const float r1 = v - hi;
-          const float mid = __bfloat162float(__float2bfloat16_rn(r1));
-          x[z] = part == 0 ? hi : (part == 1 ? mid : r1 - mid);
-        }
-        wv[q] = pack_bf16x2(x[0], x[1]);
+    for (int i = 0; i < N; ++i)
+      if (lane + 32 * i < G * 16) {
+        v[i][0] = *(const float4*)(mu + (lane + 32 * i) * 8);
+        v[i][1] = *(const float4*)(mu + (lane + 32 * i) * 8 + 4);
       }
-    }
-    *(uint4*)(img + (cc >> 3) * C::ATOM + sw128_off(C::RP + n, cc & 7)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
   }
-}
+  template <int W>
+  __device__ __forceinline__ void write(uint8_t* img, int lane) const {
+    using C = KxCfg<G, W>;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int e = lane + 32 * i, h = e >> 4, cc = e & 15;
+      if (e >= G * 16) continue;
+      const float x[8] = {v[i][0].x, v[i][0].y, v[i][0].z, v[i][0].w, v[i][1].x, v[i][1].y, v[i][1].z, v[i][1].w};
+      uint32_t w[3][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        w[0][j] = pack_bf16x2(x[2 * j], x[2 * j + 1]);
+        const float r0 = x[2 * j] - bf16lo(w[0][j]), r1 = x[2 * j + 1] - bf16hi(w[0][j]);
+        w[1][j] = pack_bf16x2(r0, r1);
+        w[2][j] = pack_bf16x2(r0 - bf16lo(w[1][j]), r1 - bf16hi(w[1][j]));
+      }
+#pragma unroll
+      for (int part = 0; part < 3; ++part)
+        *(uint4*)(img + (cc >> 3) * C::ATOM + sw128_off(C::RP + part * G + h, cc & 7)) =
+            make_uint4(w[part][0], w[part][1], w[part][2], w[part][3]);
+    }
+  }
+};
 
 template <int G, int W>
 __global__ void __launch_bounds__(KX_THREADS, 1)
@@ -97,7 +114,8 @@ __global__ void __launch_bounds__(KX_THREADS, 1)
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* tiles = smem;
   uint8_t* img = tiles + KX_STAGES * KX_TILE_BYTES;     // one image, refilled per run
-  float* red = (float*)(img + C::IMG_BYTES);             // [4 readout warps][2G]
+  float* rows = (float*)(img + C::IMG_BYTES);            // [TILE][2G] the tile's rows on their way out
+  float* red = rows + TILE * 2 * G;                      // [4 readout warps][2G]
   uint64_t* full = (uint64_t*)(red + 4 * 2 * G);
   uint64_t* empty = full + KX_STAGES;
   uint64_t* accfull = empty + KX_STAGES;  // [2]
@@ -173,8 +191,10 @@ __global__ void __launch_bounds__(KX_THREADS, 1)
       const bool same = cont;
       cont = is.next_same_unit(item);
       if (same) continue;
-      if (n >= 1 && !mbar_wait(smem_u32(imgfree), (n - 1) & 1, ws, abort)) break;
       const int l = item.plane / dm.Hkv, g = item.plane % dm.Hkv;
+      MuRows<G> mu;
+      mu.load(ws.mu + (((int64_t)item.seq * dm.L + l) * dm.Hq + (int64_t)g * G) * D, lane);
+      if (n >= 1 && !mbar_wait(smem_u32(imgfree), (n - 1) & 1, ws, abort)) break;
       if (lane == 0) {
         const uint8_t* src = ws.qimg + (((int64_t)item.seq * dm.L + l) * dm.Hkv + g) * (int64_t)C::QIMG_BYTES;
         mbar_arrive_expect_tx(smem_u32(imgfull), 4 * C::RP * 128);
@@ -185,12 +205,12 @@ __global__ void __launch_bounds__(KX_THREADS, 1)
           bulk_g2s(smem_u32(img + a * C::ATOM + C::SEC), sa + C::RP * 128, C::RP * 128, smem_u32(imgfull));
         }
       }
-      const int64_t qb = (((int64_t)item.seq * dm.L + l) * dm.Hq + (int64_t)g * G) * D;
-      write_mu_rows<G, W>(img, ws.mu + qb, lane);
-      if (n == 0)  // the zero rows of section 1 (never rewritten)
-        for (int e = lane; e < 2 * C::NB * 8; e += 32) {
-          const int a = e / (C::NB * 8), r = (e / 8) % C::NB, cc = e % 8;
-          *(uint4*)(img + a * C::ATOM + C::SEC + sw128_off(C::RP + r, cc)) = make_uint4(0u, 0u, 0u, 0u);
+      mu.template write<W>(img, lane);
+      if (n == 0)  // the zero rows of both sections (never rewritten)
+        for (int e = lane; e < 2 * 2 * C::NB * 8; e += 32) {
+          const int at = e / (2 * C::NB * 8), sec = (e / (C::NB * 8)) % 2, r = (e / 8) % C::NB, cc = e % 8;
+          if (sec == 1 || r >= 3 * G)
+            *(uint4*)(img + at * C::ATOM + sec * C::SEC + sw128_off(C::RP + r, cc)) = make_uint4(0u, 0u, 0u, 0u);
         }
       fence_proxy_async_smem();
       __syncwarp();
@@ -201,7 +221,7 @@ __global__ void __launch_bounds__(KX_THREADS, 1)
     if (lane == 0 && n > 0) mbar_wait(smem_u32(imgfull), (n - 1) & 1, ws, nullptr);
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer ----------
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t it = 0, n = 0;  // n: runs started
       bool ok = true, cont = false;
       Item item;
@@ -302,9 +322,8 @@ __global__ void __launch_bounds__(KX_THREADS, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&accempty[slot]));
-        const int64_t tok = t + y;
-        if (tok < item.t1) {
-          float row[2 * G];
+        float row[2 * G];
+        if (t + y < item.t1) {
 #pragma unroll
           for (int h = 0; h < G; ++h) {
             const float lg = dv[h] + dv[G + h] + dv[2 * G + h];
@@ -318,9 +337,8 @@ __global__ void __launch_bounds__(KX_THREADS, 1)
             row[G + h] = kap[h] * invw;
             bad |= !isfinite(row[G + h]);
           }
-          float* dst = lkp + tok * (2 * G);
-          store_floats<2 * G, LkAlign<G>::ROW>(dst, row);
         }
+        store_rows<G>(lkp, rows, row, t, item.t1, quarter, lane);
       }
       // ---- softmax statistics of a run, at its last chunk; the run's other
       // chunks get empty statistics (m = -inf, s = 0), which merge as nothing

@@ -427,25 +427,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
             run_m[h] = mn;
           }
         }
-        // the warp's rows are contiguous in global memory: through shared memory,
-        // so that each store instruction writes whole lines (a lane's own row
-        // written by itself costs 2 G / V instructions of 32 partial sectors)
-        constexpr int V = LkAlign<G>::ROW;
-        float* wrows = rows + quarter * 32 * 2 * G;
-        store_floats<2 * G, V>(wrows + lane * 2 * G, row);
-        __syncwarp();
-        const int64_t left = item.t1 - t - 32 * quarter;
-        const int nf = (int)(left < 0 ? 0 : (left < 32 ? left : 32)) * 2 * G;
-        float* dst = lkp + (t + 32 * quarter) * (2 * G);
-#pragma unroll
-        for (int e = 0; e < 2 * G / V; ++e) {
-          const int f = (lane + 32 * e) * V;
-          if (f < nf) {
-            if constexpr (V == 4) *(float4*)(dst + f) = *(const float4*)(wrows + f);
-            else *(float2*)(dst + f) = *(const float2*)(wrows + f);
-          }
-        }
-        __syncwarp();
+        store_rows<G>(lkp, rows, row, t, item.t1, quarter, lane);
         TRC_ADD(13, tr_b);
       }
       // ---- softmax statistics of a run, at its last chunk; the run's other
