@@ -226,11 +226,12 @@ jacap_status jacap_score_out(const jacap_layout* layout, const jacap_params* par
 /*
  * jacap_score for callers that cannot allocate device memory (the paper has no
  * counterpart; this is a deployment convenience). The workspace is a fixed
- * library-owned array of JACAP_STATIC_SCRATCH_BYTES in static device memory,
- * one per device; no call allocates. The work and results are those of
+ * library-owned array of JACAP_STATIC_SCRATCH_BYTES (and 64 KB for the run
+ * tables) in static device memory, one per device; no call allocates. The work and results are those of
  * jacap_score with a caller workspace.
- *  - Layouts whose jacap_workspace_size() exceeds JACAP_STATIC_SCRATCH_BYTES
- *    are refused with JACAP_ERR_WORKSPACE before any CUDA call; an invalid
+ *  - Layouts whose workspace without the run tables (which take at most 56 bytes
+ *    per chunk and request, and 4 KB) exceeds JACAP_STATIC_SCRATCH_BYTES are
+ *    refused with JACAP_ERR_WORKSPACE before any CUDA call; an invalid
  *    or unsupported layout gives the status jacap_score would.
  *  - Set-up: the first call on a device (that device current) looks up the
  *    scratch address with cudaGetSymbolAddress, which loads the module's
@@ -238,8 +239,8 @@ jacap_status jacap_score_out(const jacap_layout* layout, const jacap_params* par
  *    call that finds another context current (after cudaDeviceReset, or a
  *    primary context released and retained again) looks it up afresh. Make
  *    the first call on each device before capturing a stream into a graph.
- *  - Footprint: every device context that loads libjacap's module holds the
- *    JACAP_STATIC_SCRATCH_BYTES array resident until the context ends, whether
+ *  - Footprint: every device context that loads libjacap's module holds that
+ *    array resident until the context ends, whether
  *    or not it ever calls this function (with CUDA_MODULE_LOADING=EAGER from
  *    the library's first use; with lazy loading once the module is loaded).
  *  - scratch_out (may be NULL) receives the scratch's device address; it is

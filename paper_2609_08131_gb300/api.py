@@ -282,12 +282,13 @@ TRACE_CTA_SLOTS = {
                    3: "MMA: wait for a free accumulator", 4: "MMA: wait for a V tile", 5: "MMA: loop", 6: "tiles",
                    7: "epilogue warp: wait for an accumulator", 8: "epilogue warp: read, reduce and meet its partner",
                    9: "epilogue warp: weight and store", 10: "epilogue warp: loop"}),
+    # the factor role of the fused schedule; the factor kernel of the separate kernels keeps no account
     3: ("factor", {0: "partial Grams summed into A", 1: "elimination of diagonal block 0",
                    2: "elimination of diagonal block 1", 3: "elimination of diagonal block 2",
                    4: "elimination of diagonal block 3", 5: "elimination warp: wait for the other warps",
                    6: "panels and look-ahead updates", 7: "last inverse phase", 8: "outputs", 9: "units",
                    10: "whole unit"}),
-    4: ("selection", {0: "scores loaded", 1: "radix passes", 2: "emission", 3: "rows gathered", 4: "units",
+    4: ("selection", {0: "scores loaded", 1: "boundary key found", 2: "emission", 3: "rows gathered", 4: "units",
                       5: "whole unit"}),
 }
 

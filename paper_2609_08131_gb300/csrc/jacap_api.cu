@@ -59,10 +59,10 @@ jacap_status check_layout(const jacap_layout* L) {
 
 // Tokens per work item: the largest of 16384..128 that still yields 4096
 // items (independent of the device so the workspace size is a pure function
-// of the layout). Each CTA takes a contiguous range of items, so the counts
-// per CTA differ by one item at most: with ~27 items per CTA on 152 SMs the
-// last item costs under 4 % of a pass. Items of one unit that follow each
-// other in a CTA's range share one partial Gram and one factor image.
+// of the layout): ~27 per CTA on 152 SMs. The K pass and the scores take runs of
+// items as they become free (RunStream); the Gram and the full-covariance K pass
+// give each CTA a contiguous range (the Gram's of equal numbers of tiles). Items
+// of one unit that follow each other there share one partial Gram or image.
 #ifndef JACAP_TARGET_ITEMS
 #define JACAP_TARGET_ITEMS 4096
 #endif

@@ -1,14 +1,15 @@
 // k_gram.cu - Jacobian weights and the weighted Gram pass over V.
 //
-// Weight pass (one streaming pass over the K pass's logits/kappa rows), per
-// work item (a chunk of one unit's tokens):
+// Weight pass (float32 caches; one streaming pass over the K pass's logits/kappa
+// rows; with bf16 caches the Gram kernel forms the same weights itself), per work
+// item (a chunk of one unit's tokens):
 //   1. combines the K pass's per-chunk (max, sum exp) into the pool-softmax
 //      normaliser (M_h, Z_h) of each query head h of the group (Sec. 3.4,
 //      display after Algorithm 1);
 //   2. forms w_i = (1/d) sum_h [alpha_bar (1 - alpha_bar)]^2 kappa_h,i with
 //      alpha_bar = exp(l_h,i - M_h) / Z_h (Eq. 8; GQA heads summed) and stores
 //      w for the score pass and as a bf16 pair hi + lo for the Gram pass.
-// Gram pass: accumulates the chunk's partial Gram  sum_i w_i v_i v_i^T  (Eq. 9).
+// Gram pass: accumulates a partial Gram per run of chunks,  sum_i w_i v_i v_i^T  (Eq. 9).
 //
 // bf16 caches use the 5th-generation tensor cores. B = V straight from the
 // TMA-staged tile (bf16 is exact); the scaled operand w_i v_i = hi + lo is

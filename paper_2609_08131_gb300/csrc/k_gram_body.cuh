@@ -40,7 +40,7 @@ __device__ __forceinline__ void load_unit_stats(const Dims& dm, const Ws& ws, in
 // tensor memory: D (128 x 128, fp32) += A (128 channels x 16 tokens, TMEM)
 // * B (16 tokens x 128 channels, the TMA-staged V tile, MN-major). The TMA
 // warp stages each V tile together with the tile's logits/kappa rows from the
-// K pass (2G floats per token). The weight warp turns them into the Eq. 8
+// K pass (2G floats per token). The weight warps turn them into the Eq. 8
 // weights (the same arithmetic as weight_kernel, with the unit's softmax
 // statistics merged once per run), writes w for the score pass and leaves w
 // as a bf16 pair hi + lo in the stage for the scaling warps. The scaling warps

@@ -37,7 +37,6 @@
 // The copies' bytes alone take 0.040, 0.079, 0.044, 0.020 and 0.040 ms of the first
 // five at the copy rate.
 //
-//
 // compact_kernel: 16-byte vector copies of the kept K and V rows into the
 // dense [L][Hkv][S][B][d] output; rows of -1 (or of a position outside the
 // request) are zero-filled, so no index value can make it read out of bounds.
