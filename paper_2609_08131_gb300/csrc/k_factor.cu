@@ -31,16 +31,18 @@
 // with many units also the 192 KB that each writes. Measured against blocked 32 x 32
 // eliminations of one warp each, with the blocks in shared memory: 256 units 0.055 ->
 // 0.042 ms, 448 units 0.082 -> 0.060, 1024 units 0.173 -> 0.120; output directions,
-// 128 units, 0.124 -> 0.080 ms. 8 x 8 tiles whose owners formed u themselves took
+// 128 units, 0.124 -> 0.070 ms. 8 x 8 tiles whose owners formed u themselves took
 // 0.061 and 0.192 ms (two lanes a warp formed eight vectors each); tiles paired by
 // columns, whose rows' values all had to be doubled, 1360 cycles a step.
 //
 // With output directions u = W v (Sec. 3.1) the capacity matrix I + sum w u u^T
 // lives in the output space; with a 128 x 128 factor F of W^T W (F^T F = W^T W)
 // it reduces exactly to M = I + F G F^T, and u^T A^{-1} u = ||L_M^{-1} F v||^2.
-// That variant (PROJ) forms F G F^T with two float32 products of the same 8 x 8
-// register tiles (operands in shared memory), factors M as above and writes
-// T = L_M^{-1} F, a third product, in place of L^{-1}.
+// That variant (PROJ) forms F G with 8 x 8 register tiles (operands in shared
+// memory) and the tiles that the elimination holds of F (F G)^T straight in their
+// owners' registers, factors M as above and writes T = L_M^{-1} F, a third product
+// (to the diagonal only), in place of L^{-1}. Full 128 x 128 x 128 for the last two,
+// M by way of shared memory: 0.080 ms for 128 units instead of 0.070.
 //
 // L^{-1} is written twice: as float32 (used by the float32 score pass and
 // exposed for tests) and as a bf16 hi/lo pair laid out exactly as the
@@ -227,15 +229,15 @@ constexpr int FT_LD = D + 4;
 constexpr size_t FT_PROJ_SMEM = (size_t)2 * D * FT_LD * sizeof(float);
 
 // acc = P Q (row-major, stride FT_LD), 8 x 8 outputs per thread of a 16 x 16 grid:
-// rows 8 ty .., columns 8 tx ..
+// rows 8 ty .., columns 8 tx .., from the first `mend` (a multiple of 4) columns of P
 using Acc = float2[8][4];
-__device__ __forceinline__ void tile_product(Acc& acc, const float* P, const float* Q, int ty, int tx) {
+__device__ __forceinline__ void tile_product(Acc& acc, const float* P, const float* Q, int ty, int tx, int mend = D) {
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[i][c] = make_float2(0.f, 0.f);
 #pragma unroll 1
-  for (int m = 0; m < D; m += 4) {
+  for (int m = 0; m < mend; m += 4) {
     float2 q[4][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -258,14 +260,31 @@ __device__ __forceinline__ void tile_product(Acc& acc, const float* P, const flo
   }
 }
 
-__device__ __forceinline__ void store_acc(const Acc& T, float* dst, int ld, int ty, int tx) {
+// T = the tile of rows 8 ty .., columns 4 cx .. of P Q, the same sums in the same order.
+__device__ __forceinline__ void own_tile_product(Tile& T, const float* P, const float* Q, int ty, int cx) {
+  float2 acc[8][2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    float* r = dst + (int64_t)(8 * ty + i) * ld + 8 * tx;
-    *(float4*)r = make_float4(T[i][0].x, T[i][0].y, T[i][1].x, T[i][1].y);
-    *(float4*)(r + 4) = make_float4(T[i][2].x, T[i][2].y, T[i][3].x, T[i][3].y);
+  for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int m = 0; m < D; m += 4) {
+    float4 q[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = *(const float4*)(Q + (m + j) * FT_LD + 4 * cx);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float4 x = *(const float4*)(P + (8 * ty + i) * FT_LD + m);
+      const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        acc[i][0] = __ffma2_rn(make_float2(xs[j], xs[j]), make_float2(q[j].x, q[j].y), acc[i][0]);
+        acc[i][1] = __ffma2_rn(make_float2(xs[j], xs[j]), make_float2(q[j].z, q[j].w), acc[i][1]);
+      }
+    }
   }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) tile_set_row(T, i, make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y));
 }
+
 __device__ __forceinline__ void store_acc_t(const Acc& T, float* dst, int ld, int ty, int tx) {
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
@@ -364,7 +383,7 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
   float *R0 = fmat, *R1 = fmat + D * FT_LD;
   const int py = tid >> 4, px = tid & 15;  // the products' grid (threads 0-255)
   if constexpr (PROJ) {
-    // M = F G F^T: (F G)^T to R0, then M = F (F G)^T (M is symmetric), to R0
+    // M = F G F^T: (F G)^T to R0, then the tiles of M = F (F G)^T (M is symmetric)
     const float* F = out_factor + (int64_t)plane * D * D;
     if (own) {
 #pragma unroll
@@ -386,17 +405,7 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
     __syncthreads();
     if (tid < 256) store_acc_t(acc, R0, FT_LD, py, px);
     __syncthreads();
-    if (tid < 256) tile_product(acc, R1, R0, py, px);
-    __syncthreads();
-    if (tid < 256) store_acc(acc, R0, FT_LD, py, px);
-    __syncthreads();
-    if (own) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 v = *(const float4*)(R0 + (8 * ty + i) * FT_LD + 4 * cx);
-        tile_set_row(T, i, v);
-      }
-    }
+    if (own) own_tile_product(T, R1, R0, ty, cx);
     __syncthreads();
   }
   eliminate(T, sm, ty, cx, tid, bad);
@@ -420,11 +429,15 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
     }
     __syncthreads();
     if (tid < 256) {
+      // L_M^{-1}'s rows end at the diagonal: the 16 rows of a warp need as many
+      // columns as its last row has; warps w and w + 4, which share a sub-partition,
+      // take the row blocks w and 7 - w, i.e. 144 columns between them
       Acc acc;
-      tile_product(acc, R0, R1, py, px);
+      const int pr = py < 8 ? py : 23 - py;
+      tile_product(acc, R0, R1, pr, px, 16 * ((pr >> 1) + 1));
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const uint32_t n = 8 * py + i;
+        const uint32_t n = 8 * pr + i;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const float4 x = make_float4(acc[i][2 * h].x, acc[i][2 * h].y, acc[i][2 * h + 1].x, acc[i][2 * h + 1].y);

@@ -579,6 +579,28 @@ def test_factor_inverts_the_capacity_matrix(layers, hkv, lens, tau):
     assert bool((err <= 4 * 128 * 2.0 ** -24 * cond).all()), (err / cond).max()
 
 
+@pytest.mark.parametrize("layers, hkv, lens, tau", [(1, 2, (20000,), 10.0), (1, 1, (1, 0, 130), 0.2), (20, 8, (300,), 1.0)])
+def test_factor_with_output_directions_of_a_full_factor(layers, hkv, lens, tau):
+    """T = L_M^{-1} F as the factor writes it, F a full matrix: T^T T = F^T M^{-1} F, M = I + F G F^T,
+    within first-order bounds: forming M errs by 2 n 2^-24 |F|^2 |G| and M^{-1} is at most 1, the
+    factor and the product T by 2 n 2^-24 cond(M), both taken between F^T and F (Frobenius norms)."""
+    wl = Workload("t", layers, 4 * hkv, hkv, lens, 16, 16, seed=92)
+    t = generate(wl, DEV)
+    g = torch.Generator(device=DEV).manual_seed(5)
+    F = torch.randn((layers, hkv, 128, 128), generator=g, device=DEV) / 128 ** 0.5
+    ev = Evictor(make_cache(t, wl), wl.budget, jacap_params(tau=tau), out_factor=F)
+    ev.run()
+    ev.check()
+    x = ev.intermediates()
+    G, T, Fd = x["gram"].double(), x["chol_inv"].double(), F.double()[:, :, None]
+    G = G.tril() + G.tril(-1).mT
+    M = torch.eye(128, dtype=torch.float64, device=DEV) + Fd @ G @ Fd.mT
+    err = (T.mT @ T - Fd.mT @ torch.linalg.solve(M, Fd.expand_as(M))).abs().amax((-2, -1))
+    nf, ng = Fd.square().sum((-2, -1)), G.square().sum((-2, -1)).sqrt()
+    bound = 2 * 128 * 2.0 ** -24 * (nf * ng + torch.linalg.cond(M)) * nf
+    assert bool((err <= bound).all()), (err / bound).max()
+
+
 SELECT_UNITS = ((1, 1), (20, 8), (40, 8))  # layers, KV heads: few units, more than SMs, more than twice
 
 
