@@ -194,7 +194,9 @@ __global__ void __launch_bounds__(D, 10) window_stats_kernel(Dims dm, Ws ws, con
 #pragma unroll
   for (int i = 0; i < WS_HOLD; ++i)
     if (rg + i * RG < dm.window) held[i] = piece(rg + i * RG);
-  if (status_failed(ws)) return;  // (read with the rows)
+  // the word is read with the rows; the threads decide together, as blocks of this
+  // launch may set it (a window that is not finite) and barriers follow
+  if (__syncthreads_or(status_failed(ws) ? 1 : 0)) return;
   // acc[e] += f(channel e's value) over this thread's rows, in row order
   auto over_rows = [&](float* acc, auto f) {
     float x[V];

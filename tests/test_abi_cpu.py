@@ -191,3 +191,30 @@ def test_tracing_and_checked_variants_compile(tmp_path):
                os.path.join(_lib.CSRC, src), "-o", str(tmp_path / (src + ".o"))]
         r = subprocess.run(cmd, capture_output=True, text=True)
         assert r.returncode == 0, r.stderr[-2000:]
+
+
+def kernel_bodies(src):
+    """(name, body) of every __global__ function of a source file."""
+    text = open(os.path.join(_lib.CSRC, src)).read()
+    for m in re.finditer(r"__global__[^{;]*?(\w+)\s*\(", re.sub(r"__launch_bounds__\([^)]*\)\s*", "", text)):
+        name = m.group(1)
+        at = text.index("{", text.index(name + "("))
+        depth, end = 0, at
+        while True:
+            depth += {"{": 1, "}": -1}.get(text[end], 0)
+            end += 1
+            if depth == 0:
+                break
+        yield name, text[at:end]
+
+
+@pytest.mark.parametrize("src", ["k_stream.cu"])
+def test_blocks_with_barriers_decide_together_whether_to_skip(src):
+    """Blocks of one launch may set the status word while others read it, so a thread that leaves on
+    its own reading of it may miss the barriers that the rest of its block waits at."""
+    seen = 0
+    for name, body in kernel_bodies(src):
+        seen += 1
+        own = re.search(r"if \(status_failed\(ws\)\) return;", body)
+        assert own is None or "__syncthreads" not in body[own.end():], name
+    assert seen > 0

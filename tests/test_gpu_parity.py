@@ -279,6 +279,26 @@ def test_nonfinite_input_is_reported_on_the_device():
     assert ev.device_status() == 5  # JACAP_ERR_NONFINITE
 
 
+@pytest.mark.parametrize("dtype", ("bf16", "f32"))
+def test_windows_that_are_not_finite_among_many_are_reported(dtype):
+    """The statistics of 4096 heads, some of whose windows hold a NaN: their blocks set the status word
+    while others read it, and each block skips or finishes as a whole. The next pass, over finite
+    windows, starts clean."""
+    wl = Workload("t", 32, 32, 8, (300, 200, 129, 77), 8, 32, dtype=dtype, seed=29)
+    t = generate(wl, DEV)
+    ref = evict(make_cache(t, wl), wl.budget)
+    q = t.q_win.clone()
+    t.q_win[:, ::3, ::5, 3, 17] = float("nan")
+    ev = Evictor(make_cache(t, wl), wl.budget)
+    for _ in range(5):
+        ev.run()
+        assert ev.device_status() == 5  # JACAP_ERR_NONFINITE
+    t.q_win.copy_(q)
+    ev.run()
+    ev.check()
+    assert torch.equal(ev.scores, ref.scores) and torch.equal(ev.idx, ref.idx)
+
+
 def test_config1_every_unit():
     wl = config(1)
     t = generate(wl, DEV)
