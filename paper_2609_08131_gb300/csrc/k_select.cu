@@ -3,18 +3,19 @@
 //
 // select_kernel: one CTA per unit. Scores are non-negative float32, so their bit
 // patterns order like unsigned integers. The kept set of a unit of more than B
-// tokens is {key > T} and the keys == T at positions <= I, for the B-th token
-// (T, I) in the order of Algorithm 1 (score descending, then position):
-//  1. histogram of the keys' distance from a reference R just above the first
-//     slab's maximum, in 2048 bins of 2^16 (1/128 octave each: 16 octaves, in
-//     which the lanes of a warp rarely meet in one bin); keys further down cannot
-//     count unless the bins hold fewer than B keys;
+// tokens is {key > T} and the first keys == T by position, for the key T of the
+// B-th token in the order of Algorithm 1 (score descending, then position):
+//  1. histogram of the keys in SE_FINE bins of 2^16 (1/128 octave each: 15.75
+//     octaves, in which the lanes of a warp rarely meet in one bin) that end just
+//     above the maximum (of the first slab and a sample of the others);
 //  2. the bin that holds the B-th key, by a scan over all warps;
-//  3. that bin's keys (a handful) go to a list, and each one's rank in it names
-//     (T, I).
-// If the bins hold fewer than B keys, or the bin more than SE_CAND (many ties, as
-// with a window of one query), a radix selection over key digits and then, for
-// ties, position digits finds (T, I) instead.
+//  3. that bin's keys (a handful) go to a list, and each one's rank in it names T
+//     and the number of keys == T that are kept.
+// If the B-th key lies above or below the fine bins, a histogram of 2048 bins over
+// the keys there names its bin. While a bin holds more than SE_CAND keys (many ties,
+// as with a window of one query), a histogram over its next 11 bits names a smaller
+// one. Each of these reads the keys once more, from registers where one slab holds
+// them.
 // Emission: the keys are held in registers in slabs of NT KPT (KPT per lane, all
 // loads in flight together; the smallest that holds the longest request; a longer
 // one is read again by each step, from L2); warp w owns 32 KPT consecutive
@@ -59,18 +60,17 @@ namespace jacap {
 
 
 constexpr int SE_BINS = 2048;
-constexpr int SE_SHIFT = 16;    // a bin spans 2^16 keys
+constexpr int SE_FINE = 2016;   // bins of 2^16 keys, below bin 0 (every key above them)
 constexpr int SE_CAND = 256;    // keys of the B-th key's bin that are ranked directly (a rank reads them all: ~3 us)
 constexpr int SE_IDX = 2048;    // kept positions also held in shared memory
 
 struct SeSmem {
   uint32_t hist[SE_BINS];
-  uint32_t ckey[SE_CAND];
-  int32_t cidx[SE_CAND];
+  __align__(16) uint32_t ckey[SE_CAND];
+  __align__(16) int32_t cidx[SE_CAND];
   int32_t idx[SE_IDX];
   uint32_t tot[2][32];  // counts per warp
   uint32_t max, digit, need, count, T;
-  int32_t I;
   int skip;
 };
 
@@ -120,18 +120,17 @@ __device__ __forceinline__ void gather_unit(const Dims& dm, int plane, int64_t s
 }
 
 // The digit d (0 .. SE_BINS - 1) with (sum of hist over digits before d) < need <=
-// (that sum + hist[d]), digits counted from the top (DESC) or from 0, into
-// sm.digit; need less that sum into sm.need and hist[d] into sm.count. Every
-// thread of the CTA; the histogram is complete and holds at least `need`.
-template <int NT, bool DESC>
+// (that sum + hist[d]) into sm.digit; need less that sum into sm.need and hist[d]
+// into sm.count; SE_BINS if the histogram holds fewer than `need`. Every thread of
+// the CTA; the histogram is complete.
+template <int NT>
 __device__ __forceinline__ void find_digit(SeSmem& sm, uint32_t need, int tid) {
   constexpr int PER = SE_BINS / NT, NW = NT / 32;
   const int lane = tid & 31, warp = tid >> 5;
   uint32_t c[PER], sum = 0;
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
-    const int r = tid * PER + k;  // rank of the digit in the order of the sums
-    c[k] = sm.hist[DESC ? SE_BINS - 1 - r : r];
+    c[k] = sm.hist[tid * PER + k];
     sum += c[k];
   }
   uint32_t inc = sum;
@@ -146,96 +145,15 @@ __device__ __forceinline__ void find_digit(SeSmem& sm, uint32_t need, int tid) {
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
     if (before < need && before + c[k] >= need) {  // one thread, one k
-      const int r = tid * PER + k;
-      sm.digit = (uint32_t)(DESC ? SE_BINS - 1 - r : r);
+      sm.digit = (uint32_t)(tid * PER + k);
       sm.need = need - before;
       sm.count = c[k];
     }
     before += c[k];
   }
-  __syncthreads();
-}
-
-// Histogram of digit(key, position) over the unit's keys from global memory (-1:
-// not counted). A warp's most frequent case, ties, makes one addition: the digit of
-// its first counted lane is added for all lanes that share it.
-template <int NT, typename F>
-__device__ __forceinline__ void digit_histogram(SeSmem& sm, const uint32_t* key, int n, int tid, F digit) {
-  __syncthreads();
-  for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
-  __syncthreads();
-  for (int i0 = 0; i0 < n; i0 += NT) {
-    const int i = i0 + tid;
-    const int d = i < n ? digit(__ldg(key + i), (uint32_t)i) : -1;
-    const uint32_t some = __ballot_sync(0xffffffffu, d >= 0);
-    if (some == 0) continue;
-    const int first = __ffs(some) - 1, d0 = __shfl_sync(0xffffffffu, d, first);
-    const uint32_t same = __ballot_sync(0xffffffffu, d == d0);
-    if ((tid & 31) == first) atomicAdd(&sm.hist[d0], (uint32_t)__popc(same));
-    else if (d >= 0 && d != d0) atomicAdd(&sm.hist[d], 1u);
-  }
-  __syncthreads();
-}
-
-// (T, I) of the B-th token by digits, most significant first: of the distance below
-// R within its bin (known; the need-th key of it), or (bin < 0) of the whole keys;
-// then, if only some of the keys == T are kept, of their positions. (Every thread
-// of the CTA.)
-template <int NT>
-__device__ __noinline__ void radix_boundary(SeSmem& sm, const uint32_t* key, int n, uint32_t R, int bin,
-                                            uint32_t need, int tid) {
-  uint32_t T;
-  if (bin >= 0) {
-    const uint32_t hi = (uint32_t)bin << SE_SHIFT;  // distance >> 16 of the bin's keys, all of them <= R
-    digit_histogram<NT>(sm, key, n, tid, [&](uint32_t x, uint32_t) {
-      const uint32_t e = R - x;
-      return (e & ~0xffffu) == hi ? (int)((e & 0xffffu) >> 5) : -1;
-    });
-    find_digit<NT, false>(sm, need, tid);
-    need = sm.need;
-    const uint32_t mid = hi | (sm.digit << 5);
-    digit_histogram<NT>(sm, key, n, tid, [&](uint32_t x, uint32_t) {
-      const uint32_t e = R - x;
-      return (e & ~31u) == mid ? (int)(e & 31u) : -1;
-    });
-    find_digit<NT, false>(sm, need, tid);
-    need = sm.need;
-    T = R - (mid | sm.digit);
-  } else {
-    uint32_t prefix = 0, mask = 0;
-#pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-      const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-      const uint32_t dmask = pass == 2 ? 1023u : 2047u;
-      digit_histogram<NT>(sm, key, n, tid,
-                          [&](uint32_t x, uint32_t) { return (x & mask) == prefix ? (int)((x >> shift) & dmask) : -1; });
-      find_digit<NT, true>(sm, need, tid);
-      prefix |= sm.digit << shift;
-      mask |= dmask << shift;
-      need = sm.need;
-    }
-    T = prefix;
-  }
-  uint32_t pos = (uint32_t)n;  // all keys == T
-  if (sm.count > need) {       // the first `need` of them by position
-    uint32_t pmask = 0;
-    pos = 0;
-    // digits of 11 bits, from the highest one that a position has
-#pragma unroll 1
-    for (int shift = n > (1 << 22) ? 22 : (n > 2048 ? 11 : 0); shift >= 0; shift -= 11) {
-      digit_histogram<NT>(sm, key, n, tid, [&](uint32_t x, uint32_t i) {
-        return x == T && (i & pmask) == pos ? (int)((i >> shift) & 2047u) : -1;
-      });
-      find_digit<NT, false>(sm, need, tid);
-      pos |= sm.digit << shift;
-      pmask |= 2047u << shift;
-      need = sm.need;
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    sm.T = T;
-    sm.I = (int32_t)pos;
+  if (tid == NT - 1 && before < need) {
+    sm.digit = SE_BINS;
+    sm.need = need - before;
   }
   __syncthreads();
 }
@@ -260,7 +178,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     // (not a bit that another CTA of this launch may have set)
     sm.skip = (*((volatile uint32_t*)ws.status) & ~(uint32_t)ST_SELECT) != 0u ? 1 : 0;
     sm.max = 0;
-    sm.count = 0;
   }
   for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
   __syncthreads();
@@ -291,34 +208,77 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
   uint32_t m = 0;
 #pragma unroll
   for (int j = 0; j < KPT; ++j) m = max(m, kr[j]);
+  if (nslab > 1) {  // of the other slabs, every 16th line
+#pragma unroll 8
+    for (int i = SLAB + warp * 512 + lane; i < n; i += NW * 512) m = max(m, __ldg(key + i));
+  }
   m = __reduce_max_sync(0xffffffffu, m);
   if (lane == 0) atomicMax(&sm.max, m);
   __syncthreads();
   TRC_ADD(0, tr_u);
   TRC_T(tr_r);
-  // the reference is an octave above the first slab's maximum if there are others
+  // The fine bins end above the maximum, or an octave above it if it is that of a
+  // part of the keys; their ends are multiples of 2^21 keys.
   const uint32_t up = nslab > 1 ? 1u << 23 : 0u;
-  const uint32_t R = sm.max > 0xffffffffu - up ? 0xffffffffu : sm.max + up;
-  // bin of a key: 0 from the reference up, SE_BINS or more if too far below it
-  auto bin_of = [&](uint32_t x) { return x >= R ? 0u : (R - x) >> SE_SHIFT; };
+  const int top = (int)((min(sm.max, 0xffffffffu - up) + up) >> 16) | 31;
 #pragma unroll 1
   for (int sl = 0; sl < nslab; ++sl) {
     if (sl > 0) load_slab<KPT, NT>(key, n, sl, warp, lane, kr);
     const int base = sl * SLAB + warp * (32 * KPT) + lane;
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
-      const uint32_t d = bin_of(kr[j]);
-      if (base + 32 * j < n && d < SE_BINS) atomicAdd(&sm.hist[d], 1u);
+      const int d = max(top - (int)(kr[j] >> 16), -1) + 1;
+      if (base + 32 * j < n && d <= SE_FINE) atomicAdd(&sm.hist[d], 1u);
     }
   }
   __syncthreads();
-  find_digit<NT, false>(sm, (uint32_t)B, tid);
-  uint32_t T;
-  int32_t I;
-  // (sm.count is still 0 where the bins hold fewer than B keys)
-  if (sm.count != 0 && sm.count <= SE_CAND) {
-    const uint32_t d = sm.digit, need = sm.need;
-    const int cand = (int)sm.count;
+  find_digit<NT>(sm, (uint32_t)B, tid);
+  // hist[digit(key)] over the keys (SE_BINS: not counted)
+  auto histogram = [&](auto digit) {
+    __syncthreads();  // everyone has read digit, need and count
+    for (int b = tid; b < SE_BINS; b += NT) sm.hist[b] = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int sl = 0; sl < nslab; ++sl) {
+      if (nslab > 1) load_slab<KPT, NT>(key, n, sl, warp, lane, kr);
+      const int base = sl * SLAB + warp * (32 * KPT) + lane;
+#pragma unroll
+      for (int j = 0; j < KPT; ++j) {
+        const uint32_t d = digit(kr[j]);
+        if (base + 32 * j < n && d < SE_BINS) atomicAdd(&sm.hist[d], 1u);
+      }
+    }
+    __syncthreads();
+  };
+  // The sm.need-th of the sm.count keys with (key >> bits) == pre is the B-th.
+  uint32_t pre = (uint32_t)(top + 1 - (int)sm.digit);
+  int bits = 16;
+  if (sm.digit == 0 || sm.digit == SE_BINS) {
+    // above or below the fine bins: the keys there by their first 11 bits; 0, which
+    // many scores may be, has a bin of its own
+    const bool over = sm.digit == 0;
+    const uint32_t high = over ? 2047u : 2046u, left = over ? (uint32_t)B : sm.need;
+    histogram([&](uint32_t x) {
+      const int f = top - (int)(x >> 16);
+      return (over ? f < 0 : f >= SE_FINE) ? (x == 0u ? 2047u : high - (x >> 21)) : (uint32_t)SE_BINS;
+    });
+    find_digit<NT>(sm, left, tid);
+    bits = sm.digit == 2047u ? 0 : 21;
+    pre = sm.digit == 2047u ? 0u : high - sm.digit;
+  }
+#pragma unroll 1
+  while (sm.count > SE_CAND && bits > 0) {  // too many to rank: the next digit of those keys
+    const int w = min(bits, 11);
+    const uint32_t dmask = (1u << w) - 1u, left = sm.need;
+    histogram([&](uint32_t x) { return x >> bits == pre ? ~(x >> (bits - w)) & dmask : (uint32_t)SE_BINS; });
+    find_digit<NT>(sm, left, tid);
+    pre = (pre << w) | (~sm.digit & dmask);
+    bits -= w;
+  }
+  const int cand = (int)sm.count;
+  // The B-th key T; the first sm.need of the keys == T are kept.
+  uint32_t T = pre;  // (cand > SE_CAND: the whole key)
+  if (cand <= SE_CAND) {
     __syncthreads();  // everyone has read the bin's count
     if (tid == 0) sm.count = 0;
     __syncthreads();
@@ -328,7 +288,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
       const int base = sl * SLAB + warp * (32 * KPT) + lane;
 #pragma unroll
       for (int j = 0; j < KPT; ++j) {
-        if (base + 32 * j < n && bin_of(kr[j]) == d) {
+        if (base + 32 * j < n && kr[j] >> bits == pre) {
           const uint32_t at = atomicAdd(&sm.count, 1u);
           sm.ckey[at] = kr[j];
           sm.cidx[at] = base + 32 * j;
@@ -336,46 +296,54 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
       }
     }
     __syncthreads();
+    if (tid < 4 && cand + tid < SE_CAND) {  // ranked four at a time: the last ones count for nobody
+      sm.ckey[cand + tid] = 0u;
+      sm.cidx[cand + tid] = INT32_MAX;
+    }
+    const uint32_t need = sm.need;
+    __syncthreads();
     for (int c = tid; c < cand; c += NT) {  // the token of rank need - 1 in the bin
       const uint32_t x = sm.ckey[c];
       const int32_t i = sm.cidx[c];
-      uint32_t rank = 0;
-      for (int e = 0; e < cand; ++e) {
-        const uint32_t y = sm.ckey[e];
-        rank += y > x || (y == x && sm.cidx[e] < i) ? 1u : 0u;
+      uint32_t more = 0, same = 0;  // keys above this one, equal ones before it
+      for (int e = 0; e < cand; e += 4) {
+        const uint4 y = *(const uint4*)&sm.ckey[e];
+        const int4 p = *(const int4*)&sm.cidx[e];
+        more += (y.x > x) + (y.y > x) + (y.z > x) + (y.w > x);
+        same += (y.x == x && p.x < i) + (y.y == x && p.y < i) + (y.z == x && p.z < i) + (y.w == x && p.w < i);
       }
-      if (rank == need - 1) {
+      if (more + same == need - 1) {
         sm.T = x;
-        sm.I = i;
+        sm.need = same + 1;
       }
     }
     __syncthreads();
-  } else {
-    // in the bin, unless none was found or (several slabs) bin 0 reaches beyond R
-    const bool in_bin = sm.count != 0 && (nslab == 1 || sm.digit != 0);
-    const int bin = in_bin ? (int)sm.digit : -1;
-    const uint32_t need = in_bin ? sm.need : (uint32_t)B;
-    __syncthreads();  // (read before the next histogram's digit replaces them)
-    radix_boundary<NT>(sm, key, n, R, bin, need, tid);
+    T = sm.T;
   }
-  T = sm.T;
-  I = sm.I;
   TRC_ADD(1, tr_r);
   TRC_T(tr_e);
   // ---- emission, slab by slab ----
-  uint32_t run = 0;  // kept before this slab
+  const uint32_t nties = sm.need;
+  uint32_t run = 0, eq_run = 0;  // keys > T and == T before this slab
 #pragma unroll 1
   for (int sl = 0; sl < nslab; ++sl) {
     if (nslab > 1) load_slab<KPT, NT>(key, n, sl, warp, lane, kr);
     const int first = sl * SLAB + warp * (32 * KPT);
-    uint32_t mine = 0;  // the kept tokens of slot `lane`
+    // the tokens > T and == T of slot `lane` (keys past the request's end are 0 in kr:
+    // not above T, and the last of any ties)
+    uint32_t mine = 0, eq = 0;
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
-      const int i = first + 32 * j + lane;
-      const uint32_t b = __ballot_sync(0xffffffffu, i < n && (kr[j] > T || (kr[j] == T && i <= I)));
-      if (lane == j) mine = b;
+      const uint32_t b = __ballot_sync(0xffffffffu, kr[j] > T);
+      const uint32_t e = __ballot_sync(0xffffffffu, kr[j] == T);
+      if (lane == j) {
+        mine = b;
+        eq = e;
+      }
     }
-    const uint32_t c = __popc(mine);
+    // prefixes over lanes, then warps: keys > T in the low half, ties in the high one
+    // (a slab has at most 32768 keys)
+    const uint32_t c = __popc(mine) | (uint32_t)__popc(eq) << 16;
     uint32_t inc = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -386,8 +354,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     if (lane == 31) tot[warp] = inc;
     __syncthreads();
     const uint32_t w = lane < NW ? tot[lane] : 0u;
-    uint32_t at = run + __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + inc - c;
-    run += __reduce_add_sync(0xffffffffu, w);
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + inc - c;
+    const uint32_t all = __reduce_add_sync(0xffffffffu, w);
+    const uint32_t eb = eq_run + (before >> 16);  // ties before the lane's
+    uint32_t at = run + (before & 0xffffu) + min(eb, nties);
+    run += all & 0xffffu;
+    eq_run += all >> 16;
+    for (uint32_t take = eb < nties ? min(nties - eb, (uint32_t)__popc(eq)) : 0u; take != 0; --take) {
+      mine |= eq & (0u - eq);
+      eq &= eq - 1;
+    }
     while (mine != 0) {
       const int i = first + 32 * lane + __ffs(mine) - 1;
       mine &= mine - 1;

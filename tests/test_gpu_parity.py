@@ -678,3 +678,90 @@ def test_f32_tiles_at_their_edges():
         for layer in range(2):
             for g in range(2):
                 check_unit(ev, t, wl, params, s, layer, g)
+
+
+def _select(x, B):
+    """jacap_select_compact of one request's scores x [L, Hkv, n]; K holds each token's position."""
+    L, hkv, n = x.shape
+    k = torch.zeros((L, hkv, n, 128), dtype=torch.float32, device=DEV)
+    k[..., 0] = torch.arange(n, device=DEV)
+    q = torch.zeros((1, L, hkv, 1, 128), dtype=torch.float32, device=DEV)
+    ev = Evictor(Cache(q, k, k, torch.tensor([0, n], dtype=torch.int32, device=DEV), [n], hkv), B)
+    ev.ws[:64].zero_()
+    ev.scores.copy_(x)
+    return ev
+
+
+@pytest.mark.parametrize("layers, hkv", SELECT_UNITS)
+@pytest.mark.parametrize("n", (2052, 4097, 20000, 40000))
+@pytest.mark.parametrize("kind", ("far_below", "above_the_first_slab", "far_above", "half_ties", "subnormal", "equal_tail"))
+def test_selection_outside_the_fine_bins_is_the_stable_order(layers, hkv, n, kind):
+    """Boundaries that the selection's first histogram does not resolve: octaves far below the
+    maximum, later slabs that exceed the first one's maximum (by an octave and by many), ties of which
+    some are kept that straddle lanes, warps and slabs, subnormal scores and a tail of equal ones; at
+    budgets whose bin holds a handful of keys and thousands. Bit patterns, so exactly the stable sort."""
+    if layers * hkv > 8 and n > 20000:
+        hkv, layers = 8, 20
+    g = torch.Generator(device=DEV).manual_seed(n + layers)
+    x = torch.rand((layers, hkv, n), generator=g, device=DEV)
+    at = torch.arange(n, device=DEV)
+    if kind == "far_below":
+        x = torch.where(at % 97 == 0, x * 2.0 ** 40, x + 1e-3)
+    elif kind == "above_the_first_slab":
+        x = (x + 1e-2) * torch.where(at >= n - n // 4, 2.0 ** 6, 1.0)
+    elif kind == "far_above":
+        x = (x + 1e-2) * torch.exp2(at / n * 60 - 30)
+    elif kind == "half_ties":
+        x = torch.where(x < 0.6, torch.full_like(x, 0.3), x)
+    elif kind == "subnormal":
+        x = x * 2.0 ** -130
+    else:
+        x = torch.where(at < n // 3, x, torch.full_like(x, 2.0 ** -20))
+    order = torch.sort(x, dim=-1, descending=True, stable=True).indices
+    for B in (1, n // 97 + 200, n // 3, n - n // 5):
+        ev = _select(x, B)
+        ev.select_compact()
+        ev.check()
+        want = torch.sort(order[..., :B], dim=-1).values.int()
+        assert torch.equal(ev.idx[:, :, 0], want)
+        assert torch.equal(ev.k_out[:, :, 0, :, 0], want.float())
+
+
+@pytest.mark.parametrize("kind", ("equal", "far_below", "far_above"))
+def test_selection_takes_about_as_long_whatever_the_scores(kind):
+    """256 units of 131072 scores, all equal (a window of one query), with the boundary 20 octaves below
+    the maximum or growing along the request, against scores of a few octaves: a further digit is one
+    more read of the keys beside at least four, so at most 1.6 times as long with the ranking saved or
+    not (a read that waits for each key took 4 to 6 times as long)."""
+    n, B = 131072, 8192
+    g = torch.Generator(device=DEV).manual_seed(3)
+    x = torch.rand((32, 8, n), generator=g, device=DEV)
+
+    def us(scores):
+        ev = _select(scores[:, :, :1024], 16)  # (a small cache; jacap_select reads no K or V)
+        wide = torch.empty((32, 8, 1, B), dtype=torch.int32, device=DEV)
+        lay = ev.lay
+        cu = torch.tensor([0, n], dtype=torch.int32, device=DEV)
+        lay.cu_seqlens, lay.max_seqlen, lay.total_tokens = cu.data_ptr(), n, n
+        from paper_2609_08131_gb300 import jacap_select, jacap_workspace_size
+        from paper_2609_08131_gb300.api import _ptr, _stream
+
+        ws = torch.zeros(jacap_workspace_size(lay, B), dtype=torch.uint8, device=DEV)
+        times = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            assert jacap_select(lay, _ptr(scores), B, _ptr(wide), _ptr(ev.kept), _ptr(ws), ws.numel(), _stream()) == 0
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times)[3]
+
+    plain = us(torch.exp(x * 4 - 9))
+    if kind == "equal":
+        y = torch.full_like(x, 0.25)
+    elif kind == "far_below":
+        y = torch.where(torch.arange(n, device=DEV) % 97 == 0, x * 2.0 ** 20, x + 1e-3)
+    else:
+        y = x * torch.linspace(0, 30, n, device=DEV).exp2()
+    assert us(y.contiguous()) < 1.6 * plain
