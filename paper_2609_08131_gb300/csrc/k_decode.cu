@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(CI_THREADS)
     compact_inplace_kernel(Dims dm, Ws ws, const int32_t* __restrict__ cu, T* k, T* v, int32_t* pos,
                            const int32_t* __restrict__ idx, int budget) {
   pdl_wait();
-  if (status_failed(ws)) return;
+  // together, as a block of this launch may set the word (a unit's positions)
+  if (__syncthreads_or(status_failed(ws) ? 1 : 0)) return;
   const int u = blockIdx.x;
   const int s = u % dm.S, plane = u / dm.S;
   const int tid = threadIdx.x;
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(CI_THREADS)
                       const int32_t* __restrict__ idx, int budget) {
   pdl_wait();
   __shared__ int s_f;
-  if (status_failed(ws)) return;
+  if (__syncthreads_or(status_failed(ws) ? 1 : 0)) return;  // together, as above
   const int u = blockIdx.x;
   const int s = u % dm.S, plane = u / dm.S;
   const int tid = threadIdx.x;

@@ -208,7 +208,7 @@ def kernel_bodies(src):
         yield name, text[at:end]
 
 
-@pytest.mark.parametrize("src", ["k_stream.cu"])
+@pytest.mark.parametrize("src", [s for s in _lib.SOURCES if s.startswith("k_")])
 def test_blocks_with_barriers_decide_together_whether_to_skip(src):
     """Blocks of one launch may set the status word while others read it, so a thread that leaves on
     its own reading of it may miss the barriers that the rest of its block waits at."""

@@ -214,6 +214,37 @@ def test_compaction_refuses_positions_that_do_not_ascend():
         assert torch.equal(ev.k, before)
 
 
+@pytest.mark.parametrize("ordered", (0, 1))
+def test_a_refused_unit_leaves_every_other_one_whole(ordered):
+    """Positions that repeat in some of 1280 units, whose blocks set the status word while others start:
+    each other unit is compacted completely or not touched at all, never in part."""
+    from paper_2609_08131_gb300 import JACAP_ERR_INVALID_ARG, jacap_compact_inplace, jacap_device_status
+    from paper_2609_08131_gb300.api import _ptr, _stream
+
+    L, Hkv, B, T = 160, 8, 96, 160
+    ev = DecodeEvictor(1, L, Hkv, Hkv, B, T, dtype=torch.float32, device=DEV)
+    g = torch.Generator(device=DEV).manual_seed(4)
+    rows = torch.arange(B + T, device=DEV, dtype=torch.float32)[:, None].expand(-1, 128)
+    for _ in range(4):
+        ev.k.copy_(rows)
+        ev.v.copy_(-rows)
+        idx = torch.rand((L, Hkv, 1, B + T), generator=g, device=DEV).argsort(-1)[..., :B].sort(-1).values.int()
+        bad = torch.zeros((L, Hkv), dtype=torch.bool, device=DEV)
+        bad.view(-1)[300::77] = True
+        idx[..., 5] = torch.where(bad[..., None], idx[..., 4], idx[..., 5])
+        ev.idx.copy_(idx)
+        ev.ws.zero_()
+        assert jacap_compact_inplace(ev.slot, _ptr(ev._k), _ptr(ev._v), _ptr(ev._pos), _ptr(ev.idx), B, ordered,
+                                     _ptr(ev.ws), ev.ws.numel(), _stream()) == 0
+        assert jacap_device_status(_ptr(ev.ws), _stream()) == JACAP_ERR_INVALID_ARG
+        k, before = ev._k[:, :, 0, :B], rows[:B].expand(L, Hkv, B, 128)
+        whole = (k == before).all((-2, -1))
+        kept = torch.sort(k[..., 0], dim=-1).values
+        moved = (k == k[..., :1]).all((-2, -1)) & (kept == idx[:, :, 0].float()).all(-1)
+        assert bool((whole | moved).all()) and bool(whole[bad].all())
+        assert torch.equal(ev._v[:, :, 0, :B], -k)
+
+
 def test_host_evictor_matches_the_oracle():
     # a cache in pinned host memory, evicted through jacap_evict_host in layer
     # groups of 2 through two device buffers (the groups' copies overlap the
