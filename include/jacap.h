@@ -245,7 +245,8 @@ jacap_status jacap_score_out(const jacap_layout* layout, const jacap_params* par
  *    the library's first use; with lazy loading once the module is loaded).
  *  - scratch_out (may be NULL) receives the scratch's device address; it is
  *    laid out as a workspace (see jacap_workspace_offsets) and can be passed
- *    as `ws` to jacap_select and jacap_device_status. Its status word is reset
+ *    as `ws`, of JACAP_STATIC_SCRATCH_BYTES, to the selection and compaction
+ *    calls, and to jacap_device_status. Its status word is reset
  *    by every call; nothing else needs to start at zero.
  *  - Every call on a device shares that one scratch: calls (and any use of the
  *    returned address) that overlap in time race and corrupt each other's

@@ -144,6 +144,16 @@ Carve carve(const Dims& dm) {
   return c;
 }
 
+// Whether the selection and the compactions take a workspace of this size: that of
+// jacap_workspace_size, or the static scratch for a layout that jacap_score_static
+// accepts (it limits the workspace without the run tables, which they do not read).
+bool selection_ws_fits(const Carve& c, size_t ws_bytes) {
+#ifndef JACAP_TRACE  // (there the selection writes its account behind the run tables)
+  if (ws_bytes >= JACAP_STATIC_SCRATCH_BYTES && c.base <= JACAP_STATIC_SCRATCH_BYTES) return true;
+#endif
+  return ws_bytes >= c.total;
+}
+
 Ws make_ws(void* base, const Carve& c) {
   uint8_t* b = (uint8_t*)base;
   Ws ws;
@@ -615,7 +625,7 @@ jacap_status jacap_compact_inplace(const jacap_layout* layout, void* k, void* v,
   Dims dm;
   make_dims(layout, nullptr, dm);
   const Carve c = carve(dm);
-  if (((uintptr_t)ws & 255u) != 0 || ws_bytes < c.total) return JACAP_ERR_WORKSPACE;
+  if (((uintptr_t)ws & 255u) != 0 || !selection_ws_fits(c, ws_bytes)) return JACAP_ERR_WORKSPACE;
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   return map_cuda(launch_compact_inplace(dm, make_ws(ws, c), layout->dtype == JACAP_BF16 ? 1 : 0,
@@ -638,7 +648,7 @@ jacap_status jacap_select_compact_inplace(const jacap_layout* layout, const floa
   Dims dm;
   make_dims(layout, nullptr, dm);
   const Carve c = carve(dm);
-  if (((uintptr_t)ws & 255u) != 0 || ws_bytes < c.total) return JACAP_ERR_WORKSPACE;
+  if (((uintptr_t)ws & 255u) != 0 || !selection_ws_fits(c, ws_bytes)) return JACAP_ERR_WORKSPACE;
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   const Ws w = make_ws(ws, c);
@@ -666,7 +676,7 @@ jacap_status jacap_select(const jacap_layout* layout, const float* scores, int32
   Dims dm;
   make_dims(layout, nullptr, dm);
   const Carve c = carve(dm);
-  if (((uintptr_t)ws & 255u) != 0 || ws_bytes < c.total) return JACAP_ERR_WORKSPACE;
+  if (((uintptr_t)ws & 255u) != 0 || !selection_ws_fits(c, ws_bytes)) return JACAP_ERR_WORKSPACE;
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   const Ws w = make_ws(ws, c);
@@ -689,7 +699,7 @@ jacap_status jacap_select_compact(const jacap_layout* layout, const float* score
   Dims dm;
   make_dims(layout, nullptr, dm);
   const Carve c = carve(dm);
-  if (((uintptr_t)ws & 255u) != 0 || ws_bytes < c.total) return JACAP_ERR_WORKSPACE;
+  if (((uintptr_t)ws & 255u) != 0 || !selection_ws_fits(c, ws_bytes)) return JACAP_ERR_WORKSPACE;
   int sms = 0;
   if ((st = check_device(&sms)) != JACAP_OK) return st;
   const Ws w = make_ws(ws, c);

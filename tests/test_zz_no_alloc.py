@@ -12,6 +12,7 @@ import pytest
 import torch
 
 from paper_2609_08131_gb300 import (
+    JACAP_ERR_CUDA,
     JACAP_ERR_INVALID_ARG,
     JACAP_ERR_WORKSPACE,
     JACAP_OK,
@@ -87,3 +88,31 @@ def test_oversized_and_invalid_layouts_are_refused_on_the_host():
     lay.window = 0
     st, scratch = jacap_score_static(lay, jacap_params(), null, null, null, null, null)
     assert (st, scratch) == (JACAP_ERR_INVALID_ARG, 0)
+
+
+@pytest.mark.parametrize("lens", [(42154,) * 3, (31487,) * 4, (7471,) * 16])
+def test_the_scratch_serves_the_selection_wherever_it_served_the_scores(lens):
+    """Layouts within the scratch's limit whose run tables lie beyond JACAP_STATIC_SCRATCH_BYTES: the
+    calls that take the scratch with that size refuse none of them. (On a machine without a GPU both
+    stop at the device check; nothing is enqueued, as the buffers here are misaligned for the scores.)"""
+    from paper_2609_08131_gb300 import jacap_compact_inplace, jacap_layout, jacap_select_compact, jacap_select_compact_inplace
+
+    S, n, N = len(lens), max(lens), sum(lens)
+    lay = jacap_layout()
+    lay.num_seqs, lay.cu_seqlens, lay.max_seqlen, lay.total_tokens = S, 0x1000, n, N
+    lay.num_layers, lay.num_q_heads, lay.num_kv_heads, lay.head_dim, lay.window, lay.dtype = 1, 1, 1, 128, 16, 1
+    lay.kv_stride_layer, lay.kv_stride_head, lay.kv_stride_token = N * 128, N * 128, 128
+    lay.q_stride_seq, lay.q_stride_layer, lay.q_stride_head, lay.q_stride_pos = 16 * 128, 16 * 128, 16 * 128, 128
+    assert jacap_workspace_size(lay, 8) > JACAP_STATIC_SCRATCH_BYTES
+    p, odd, null = ctypes.c_void_p(0x1000), ctypes.c_void_p(0x1008), ctypes.c_void_p(0)
+    # refused for the buffers, that is not for the size
+    assert jacap_score_static(lay, jacap_params(), odd, p, p, p, null)[0] in (JACAP_ERR_INVALID_ARG, JACAP_ERR_CUDA)
+    if torch.cuda.is_available():
+        return  # (the calls below would be enqueued)
+    nb = JACAP_STATIC_SCRATCH_BYTES
+    for st in (jacap_select(lay, p, 8, p, p, p, nb, null),
+               jacap_select_compact(lay, p, 8, p, p, p, p, p, p, p, nb, null),
+               jacap_compact_inplace(lay, p, p, null, p, 8, 0, p, nb, null),
+               jacap_select_compact_inplace(lay, p, 8, p, p, p, p, null, 0, p, nb, null)):
+        assert st != JACAP_ERR_WORKSPACE
+    assert jacap_select(lay, p, 8, p, p, p, nb - 1, null) == JACAP_ERR_WORKSPACE
