@@ -14,11 +14,23 @@
 // into tensor memory as two A operands (lane = token, two channels per column),
 // and B = lambda. mu' and lambda are split exactly into three bf16 parts (hi +
 // mid + lo carries ~24 significant bits) for the G heads, so the products are
-// those of float32 operands. The MMAs' fp32 sums truncate: kappa's channels go
-// into KG groups of columns (four of 32 channels, two of 64 for G > 5) that the
-// readout adds, which keeps the scores as close to float64 as the float32
-// multiply-adds did (rel. 6.6e-7 either way at G = 4, n = 32768; one group for
-// all channels: 7.7e-7).
+// those of float32 operands (k^2 while its lo part is not subnormal: |k| > 2^-58).
+//
+// The MMAs' fp32 sums truncate, which would leave kappa's sums of positive terms too
+// small by half a unit in the last place per addition. So kappa's K-steps go into KG
+// groups of columns (four of 2 steps; three of 3, 3 and 2 for G > 5, where a group
+// takes twice the columns) that the readout adds, and the sum is recentred: of m
+// additions of about equal terms the j-th truncates at a sum of j / m of the group's,
+// losing 2^-24 / (2 ln 2) of it on average over a mantissa, together (m + 1) 2^-23 /
+// (8 ln 2) of the group's sum, which the readout adds to the small parts before its
+// last addition rounds. Error of sum_h kappa against 64 bits, rms (n = 8192, windows of
+// 32): 4.8e-8, 4.5e-8, 4.6e-8, 5.0e-8, 5.1e-8 for G = 1, 4, 5, 7, 8, and 4.8e-8, 4.5e-8,
+// 4.6e-8, 4.9e-8, 5.0e-8 with float32 multiply-adds; not recentred (two groups for G >
+// 5) 8.0e-8, 7.7e-8, 7.8e-8, 1.27e-7, 1.27e-7. With four key channels 8 times the others
+// 5.2e-8, 4.8e-8, 4.9e-8, 5.3e-8, 5.5e-8 (multiply-adds 5.2e-8, 4.6e-8, 4.7e-8, 5.0e-8,
+// 5.1e-8). Recentring costs no time, the third group 1 % of the K pass at G = 7 and 8.
+// The softmax sums take expf: with __expf they were 3.4e-8 too small and the weights
+// 9e-8 too large (n >= 32768), with it 0.3e-8 to 0.8e-8 and 1.5e-8 to 2.8e-8.
 //
 // Why this way: issued under elect.sync, an M = 128, N = 16 MMA costs 9 cycles
 // with A in tensor memory and 39 with A in shared memory (45 either way under a
@@ -53,7 +65,17 @@ static_assert(KB_ACC_COLS + 2 * KB_A_COLS <= KB_TMEM_COLS, "tensor memory budget
 template <int G>
 struct KbCfg {
   static constexpr int NB = (3 * G <= 16) ? 16 : 32;  // MMA N = rows of an image
-  static constexpr int KG = NB == 16 ? 4 : 2;          // kappa's channel groups, each with columns of its own
+  static constexpr int KG = NB == 16 ? 4 : 3;          // kappa's channel groups, each with columns of its own
+  static constexpr int step0(int g) { return (g * (D / 16) + KG - 1) / KG; }  // K-steps (16 channels) before group g
+  // what truncation takes from kappa on average, relative (see the top)
+  static constexpr float recentre() {
+    float c = 0.f;
+    for (int g = 0; g < KG; ++g) {
+      const int m = step0(g + 1) - step0(g);
+      c += (float)m / (D / 16) * (float)(m + 1) * 0.18033688f;  // 1 / (8 ln 2)
+    }
+    return c * 1.1920929e-7f;  // 2^-23
+  }
   static constexpr int ACC = (1 + KG) * NB;            // columns of an accumulator slot: logits, then the groups
   static constexpr int NACC = KB_ACC_COLS / ACC;
   static constexpr int IMG_ATOM = NB * 128;            // bytes per 64-channel atom
@@ -245,16 +267,15 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
           const uint32_t a = tmem + KB_ACC_COLS + ab * KB_A_COLS;
           const uint64_t a0 = smem_desc_sw128(smem_u32(tiles + st * KB_TILE_BYTES), 16, 1024);
           const uint32_t dl = tmem + ac * C::ACC;
-          constexpr int KS = D / 16 / C::KG;  // K-steps (16 channels) per group
 #pragma unroll
           for (int g = 0; g < C::KG; ++g) {
 #pragma unroll
             for (int part = 0; part < 2; ++part)  // lo first: the sums stay small until the last steps
 #pragma unroll
-              for (int k = g * KS; k < (g + 1) * KS; ++k)
+              for (int k = C::step0(g); k < C::step0(g + 1); ++k)
                 umma_f16_ts(dl + (1 + g) * NB, a + (part == 0 ? 64 : 0) + 8 * k,
                             blam + (uint64_t)((((k >> 2) * C::IMG_ATOM) + (k & 3) * 32) >> 4), C::IDESC,
-                            part == 0 && k == g * KS ? 0u : 1u);
+                            part == 0 && k == C::step0(g) ? 0u : 1u);
           }
 #pragma unroll
           for (int k = 0; k < D / 16; ++k)
@@ -409,7 +430,7 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
             }
           }
 #pragma unroll
-          for (int h = 0; h < G; ++h) row[G + h] += low[h];
+          for (int h = 0; h < G; ++h) row[G + h] += fmaf(C::recentre(), row[G + h], low[h]);
         }
         tc_fence_before();
         __syncwarp();
@@ -419,11 +440,9 @@ __global__ void __launch_bounds__(KB_THREADS, 1)
           for (int h = 0; h < G; ++h) {
             const float lg = row[h];
             bad |= !isfinite(lg) || !isfinite(row[G + h]);
-            // branch-free online update: one of the two exponentials is exp(0);
-            // both arguments are <= 0, where the fast exponential's relative
-            // error (a few ulp) is far below what the statistics need
+            // branch-free online update: one of the two exponentials is exp(0)
             const float mn = fmaxf(run_m[h], lg);
-            run_s[h] = run_s[h] * __expf(run_m[h] - mn) + __expf(lg - mn);
+            run_s[h] = run_s[h] * expf(run_m[h] - mn) + expf(lg - mn);
             run_m[h] = mn;
           }
         }
