@@ -282,12 +282,14 @@ TRACE_CTA_SLOTS = {
                    3: "MMA: wait for a free accumulator", 4: "MMA: wait for a V tile", 5: "MMA: loop", 6: "tiles",
                    7: "epilogue warp: wait for an accumulator", 8: "epilogue warp: read, reduce and meet its partner",
                    9: "epilogue warp: weight and store", 10: "epilogue warp: loop"}),
-    # the factor role of the fused schedule; the factor kernel of the separate kernels keeps no account
+    # slots 1 to 7: the factor role of the fused schedule; 11 to 14: the factor kernel of the separate ones
     3: ("factor", {0: "partial Grams summed into A", 1: "elimination of diagonal block 0",
                    2: "elimination of diagonal block 1", 3: "elimination of diagonal block 2",
                    4: "elimination of diagonal block 3", 5: "elimination warp: wait for the other warps",
                    6: "panels and look-ahead updates", 7: "last inverse phase", 8: "outputs", 9: "units",
-                   10: "whole unit"}),
+                   10: "whole unit", 11: "elimination steps: wait for all vectors",
+                   12: "elimination steps: vectors turned into u", 13: "elimination steps: update and vectors left",
+                   14: "products before the elimination (output directions)"}),
     4: ("selection", {0: "scores loaded", 1: "boundary key found", 2: "emission", 3: "rows gathered", 4: "units",
                       5: "whole unit"}),
 }

@@ -392,8 +392,17 @@ __device__ __forceinline__ void trace_max(const Ws& ws, int64_t u, int slot) {
 #define JACAP_TRACE_MIN(ws, u, slot) trace_min(ws, u, slot)
 #define JACAP_TRACE_MAX(ws, u, slot) trace_max(ws, u, slot)
 // time accounting: TRC_T(v) starts a stopwatch, TRC_ADD(acc, v) adds its
-// elapsed ns to acc, TRC_PUT(ws, k, slot, acc) adds acc to the CTA's slot
+// elapsed ns to acc, TRC_PUT(ws, k, slot, acc) adds acc to the CTA's slot;
+// TRC_PARAM and TRC_PASS hand the accounts to a function. TRC_AFTER(v, x) reads the
+// clock once the 32-bit value x is there (a plain reading may be taken before a
+// barrier, or before arithmetic, that precedes it); TRC_SPAN(acc, a, b) adds b - a.
 #define TRC_DECL(n) unsigned long long trc[n] = {}
+#define TRC_PARAM , unsigned long long (&trc)[TR_CTA_SLOTS]
+#define TRC_PASS , trc
+#define TRC_AFTER(v, x)      \
+  unsigned long long v = 0;  \
+  if ((x) != 0x7fedcba9) v = globaltimer()
+#define TRC_SPAN(i, a, b) (trc[i] += (b) - (a))
 #define TRC_T(v) const unsigned long long v = globaltimer()
 #define TRC_ADD(i, v) (trc[i] += globaltimer() - (v))
 #define TRC_INC(i) (++trc[i])
@@ -408,6 +417,10 @@ __device__ __forceinline__ void trace_max(const Ws& ws, int64_t u, int slot) {
 #define JACAP_TRACE_MIN(ws, u, slot) ((void)0)
 #define JACAP_TRACE_MAX(ws, u, slot) ((void)0)
 #define TRC_DECL(n) ((void)0)
+#define TRC_PARAM
+#define TRC_PASS
+#define TRC_AFTER(v, x) ((void)0)
+#define TRC_SPAN(i, a, b) ((void)0)
 #define TRC_T(v) ((void)0)
 #define TRC_ADD(i, v) ((void)0)
 #define TRC_INC(i) ((void)0)

@@ -61,6 +61,7 @@ namespace jacap {
 
 constexpr int FT_TILES = 272;     // tiles (ty, cx), cx <= 2 ty + 1
 constexpr int FT_THREADS = 288;
+constexpr int FT_TRACED = 240;    // (time accounting) the owner of the last tile row's first tile: in every step
 
 // A step's vectors: raw by index (16 bytes between the tile rows, so that the rows
 // that a warp stores fall in different banks), u by component.
@@ -183,9 +184,12 @@ __device__ __forceinline__ void update_rows(Tile& T, const FtSmem& sm, int ty, i
 }
 
 template <int H>
-__device__ __forceinline__ void eliminate_step(Tile& T, FtSmem& sm, int p, int ty, int cx, int tid, bool& bad) {
+__device__ __forceinline__ void eliminate_step(Tile& T, FtSmem& sm, int p, int ty, int cx, int tid,
+                                               bool& bad TRC_PARAM) {
   const int b = 2 * p + H;
+  TRC_AFTER(tr_w, __float_as_int(tile_at(T, 7, 3)));
   named_barrier_sync(1, FT_THREADS);
+  TRC_AFTER(tr_v, *(volatile int*)&sm.linv[3].w);
   if (tid < D) {
     const float4 m0 = sm.linv[0], m1 = sm.linv[1], m2 = sm.linv[2], m3 = sm.linv[3];
     float4 x = sm.raw[tid + (tid >> 3)];
@@ -201,6 +205,7 @@ __device__ __forceinline__ void eliminate_step(Tile& T, FtSmem& sm, int p, int t
     sm.ut[3][tid] = u3;
   }
   named_barrier_sync(1, FT_THREADS);
+  TRC_AFTER(tr_u, *(volatile int*)&sm.ut[3][D - 1]);
   if (ty >= p) {
     if (ty > p) {
       update_rows<0>(T, sm, ty, cx);
@@ -212,15 +217,22 @@ __device__ __forceinline__ void eliminate_step(Tile& T, FtSmem& sm, int p, int t
     if (H == 0) leave_vectors<1>(T, sm, p, ty, cx, bad);
     else if (p < 15) leave_vectors<0>(T, sm, p + 1, ty, cx, bad);
   }
+  TRC_AFTER(tr_e, __float_as_int(tile_at(T, 7, 3)));
+  if (tid == FT_TRACED) {
+    TRC_SPAN(11, tr_w, tr_v);
+    TRC_SPAN(12, tr_v, tr_u);
+    TRC_SPAN(13, tr_u, tr_e);
+  }
 }
 
 // T (the tiles of A - I) -> L^{-1}'s, by FT_THREADS threads (the last ones without a tile: ty = -1).
-__device__ __forceinline__ void eliminate(Tile& T, FtSmem& sm, int ty, int cx, int tid, bool& bad) {
+__device__ __forceinline__ void eliminate(Tile& T, FtSmem& sm, int ty, int cx, int tid,
+                                          bool& bad TRC_PARAM) {
   if (ty >= 0) leave_vectors<0>(T, sm, 0, ty, cx, bad);
 #pragma unroll 1
   for (int p = 0; p < 16; ++p) {
-    eliminate_step<0>(T, sm, p, ty, cx, tid, bad);
-    eliminate_step<1>(T, sm, p, ty, cx, tid, bad);
+    eliminate_step<0>(T, sm, p, ty, cx, tid, bad TRC_PASS);
+    eliminate_step<1>(T, sm, p, ty, cx, tid, bad TRC_PASS);
   }
 }
 
@@ -327,6 +339,13 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
   __syncthreads();
   if (sm.skip) return;
   bool bad = false;
+  // time accounting (trace builds): 0 the partials summed, 8 the outputs, 9 units, 10 the
+  // whole unit, 14 the products before the elimination (thread 0); of the elimination, by
+  // FT_TRACED, 11 from its arrival at a step's first barrier until all vectors are left,
+  // 12 from there to the second (the vectors turned into u), 13 the rest of the step
+  // (update, vectors left)
+  TRC_DECL(TR_CTA_SLOTS);
+  TRC_T(tr_unit);
 
   // G's tiles: the sum of the unit's partials, in chunk order, straight from
   // global memory (layout: (m, n) at ((n / 32) D + m) 32 + n % 32)
@@ -387,9 +406,15 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
       }
     }
   }
+  TRC_AFTER(tr_g, __float_as_int(tile_at(T, 0, 0)));
+  if (tid == 0) {
+    TRC_SPAN(0, tr_unit, tr_g);
+    TRC_INC(9);
+  }
   float *R0 = fmat, *R1 = fmat + D * FT_LD;
   const int py = tid >> 4, px = tid & 15;  // the products' grid (threads 0-255)
   if constexpr (PROJ) {
+    TRC_T(tr_p);
     // M = F G F^T: (F G)^T to R0, then the tiles of M = F (F G)^T (M is symmetric)
     const float* F = out_factor + (int64_t)plane * D * D;
     if (own) {
@@ -414,8 +439,10 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
     __syncthreads();
     if (own) own_tile_product(T, R1, R0, ty, cx);
     __syncthreads();
+    if (tid == 0) TRC_ADD(14, tr_p);
   }
-  eliminate(T, sm, ty, cx, tid, bad);
+  eliminate(T, sm, ty, cx, tid, bad TRC_PASS);
+  TRC_T(tr_o);
   if (own && cx >= 2 * ty) {  // zeros above the diagonal
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -485,6 +512,11 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
       }
     }
   }
+  if (tid == 0) {
+    TRC_ADD(8, tr_o);
+    TRC_ADD(10, tr_unit);
+  }
+  if (tid == 0 || tid == FT_TRACED) TRC_PUT(ws, TR_K_FACTOR, TR_CTA_SLOTS);
   if (bad) flag(ws, ST_NONFINITE);
 }
 

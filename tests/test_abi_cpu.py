@@ -218,3 +218,32 @@ def test_blocks_with_barriers_decide_together_whether_to_skip(src):
         own = re.search(r"if \(status_failed\(ws\)\) return;", body)
         assert own is None or "__syncthreads" not in body[own.end():], name
     assert seen > 0
+
+
+@pytest.mark.parametrize("kernel, sources", [
+    (2, ["k_kpass.cu"]), (0, ["k_gram_body.cuh"]), (1, ["k_score_body.cuh"]), (4, ["k_select.cu"]),
+    (3, ["k_factor.cu", "k_factor_body.cuh"]),  # the separate kernel, the fused schedule's role
+])
+def test_every_kernel_keeps_the_account_that_the_report_reads(kernel, sources):
+    """A JACAP_TRACE build: each of a kernel's sources hands its slots over, and together they fill
+    exactly those that the report names."""
+    from paper_2609_08131_gb300.api import TRACE_CTA_SLOTS
+
+    put = {0: "TR_K_GRAM", 1: "TR_K_SCORE", 2: "TR_K_KPASS", 3: "TR_K_FACTOR", 4: "TR_K_SELECT"}[kernel]
+    filled = set()
+    for src in sources:
+        text = open(os.path.join(_lib.CSRC, src)).read()
+        assert f"TRC_PUT(ws, {put}," in text, src
+        for a, plus in re.findall(r"TRC_(?:ADD|INC|SPAN)\((\d+)( \+ K)?", text):
+            filled |= set(range(int(a), int(a) + (4 if plus else 1)))
+    assert filled == set(TRACE_CTA_SLOTS[kernel][1])
+
+
+@pytest.mark.parametrize("src", ["k_factor.cu", "k_fused.cu"])
+def test_traced_factor_compiles(tmp_path, src):
+    import subprocess
+
+    cmd = [_lib.nvcc(), *_lib.ARCH, *_lib.CFLAGS, "-DJACAP_TRACE", "-c", os.path.join(_lib.CSRC, src), "-o",
+           str(tmp_path / "o.o")]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
