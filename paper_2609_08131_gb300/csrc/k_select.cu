@@ -281,6 +281,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
   if (cand <= SE_CAND) {
     __syncthreads();  // everyone has read the bin's count
     if (tid == 0) sm.count = 0;
+    if (tid < 4 && cand + tid < SE_CAND) {  // ranked four at a time: the last ones count for nobody
+      sm.ckey[cand + tid] = 0u;
+      sm.cidx[cand + tid] = INT32_MAX;
+    }
     __syncthreads();
 #pragma unroll 1
     for (int sl = 0; sl < nslab; ++sl) {
@@ -294,11 +298,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
           sm.cidx[at] = base + 32 * j;
         }
       }
-    }
-    __syncthreads();
-    if (tid < 4 && cand + tid < SE_CAND) {  // ranked four at a time: the last ones count for nobody
-      sm.ckey[cand + tid] = 0u;
-      sm.cidx[cand + tid] = INT32_MAX;
     }
     const uint32_t need = sm.need;
     __syncthreads();
