@@ -783,3 +783,28 @@ def test_kappa_rounds_like_float32_multiply_adds(G):
     err = x["weights"].double() / ref - 1
     assert abs(float(err.mean())) <= 0.25 * 2.0 ** -24
     assert float(err.square().mean().sqrt()) <= 2.0 ** -24
+
+
+@pytest.mark.parametrize("dtype", ("bf16", "f32"))
+@pytest.mark.parametrize("layers, hkv, lens", [
+    (1, 1, (40000,)),               # one unit of 313 chunks: the reducing launch lists its partials twice
+    (2, 1, (70000,)),
+    (1, 1, (40000,) + (20,) * 60),  # the same in a pack whose mean has few partials: the factor lists them itself
+])
+def test_every_partial_gram_of_a_long_unit_is_summed(dtype, layers, hkv, lens):
+    """G as the factor leaves it against sum_i w_i v_i v_i^T in 64 bits, with the pass's own weights, in
+    units of more chunks than the lists of partials hold at once (256 and 288). w v is split within
+    2^-17; sums over n tokens and their partials are float32, of random signs off the diagonal and each
+    truncation at most 2^-23: 2^-15 of the sum of the terms' magnitudes covers them. One chunk of 313
+    left out, or taken twice, is 3e-3 of it."""
+    wl = Workload("t", layers, 4 * hkv, hkv, lens, 16, 16, dtype=dtype, dist="latent" if dtype == "bf16" else "outlier",
+                  seed=93)
+    t = generate(wl, DEV)
+    ev = evict(make_cache(t, wl), wl.budget)
+    x = ev.intermediates()
+    at = 0
+    for s, n in enumerate(lens):
+        v, w = t.v[:, :, at:at + n].double(), x["weights"][:, :, at:at + n, None].double()
+        at += n
+        ref, size = v.mT @ (w * v), v.abs().mT @ (w * v.abs())
+        assert bool(((x["gram"][:, :, s].double() - ref).abs() <= 2.0 ** -15 * size).all()), s
