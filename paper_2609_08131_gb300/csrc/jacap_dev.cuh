@@ -235,12 +235,10 @@ constexpr int G_MAX = 8;
 
 // The logits/kappa rows hold 2G floats per token: l_h at [0, G), kappa_h at
 // [G, 2G). A row starts on a multiple of 2G floats from a 1 KB-aligned base, so
-// it is 16-byte aligned for even G and 8-byte aligned for odd G; the kappa
-// half (G floats further) keeps 16 bytes only when G % 4 == 0.
+// it is 16-byte aligned for even G and 8-byte aligned for odd G.
 template <int G>
 struct LkAlign {
-  static constexpr int ROW = G % 2 == 0 ? 4 : 2;                      // floats
-  static constexpr int KAPPA = G % 4 == 0 ? 4 : (G % 2 == 0 ? 2 : 1);  // floats
+  static constexpr int ROW = G % 2 == 0 ? 4 : 2;  // floats
 };
 
 // dst[0 .. N) = v with the widest stores an alignment of A floats (1, 2 or 4)
@@ -809,28 +807,12 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t& r0, uint3
                : "memory");
 }
 
-// Store to tensor memory, shape 16 lanes x 128 bits: thread t writes r0 to
-// (lane t/4, column t%4) and r1 to (lane 8 + t/4, column t%4), relative to taddr.
-__device__ __forceinline__ void tmem_st_16x128b(uint32_t taddr, uint32_t r0, uint32_t r1) {
-  asm volatile("tcgen05.st.sync.aligned.16x128b.x1.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(r0), "r"(r1)
-               : "memory");
-}
-
-// Eight repetitions of the 16x128b store along columns: registers 2j, 2j+1
-// go to columns 4j .. 4j + 3 (32 columns in all).
+// Store to tensor memory, shape 16 lanes x 128 bits, eight repetitions along
+// columns: thread t writes registers 2j and 2j + 1 to (lane t/4, column 4j + t%4)
+// and (lane 8 + t/4, column 4j + t%4), relative to taddr (32 columns in all).
 __device__ __forceinline__ void tmem_st_16x128b_x8(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], "
-      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-      "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-      : "memory");
-}
-
-// Store 16 consecutive 32-bit columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
       "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
       "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
@@ -980,19 +962,9 @@ __device__ __forceinline__ uint4 lds_u128(uint32_t addr) {
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
   return v;
 }
-__device__ __forceinline__ float4 lds_f128(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-  return v;
-}
 __device__ __forceinline__ uint2 lds_u64(uint32_t addr) {
   uint2 v;
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
   return v;
 }
 

@@ -152,7 +152,8 @@ cudaError_t launch_score(const CUtensorMap& vmap, const Dims& dm, const Ws& ws, 
                          const int32_t* cu, float* scores, int grid, cudaStream_t st) {
   if (dtype == 1) {
     const size_t smem = dm.dense_minv ? score_bf16_smem_bytes<true>() : score_bf16_smem_bytes<false>();
-    static_assert(score_bf16_smem_bytes<true>() <= 232448 && score_bf16_smem_bytes<false>() <= 232448, "smem");
+    static_assert(score_bf16_smem_bytes<true>() + 512 <= 232448 && score_bf16_smem_bytes<false>() + 512 <= 232448,
+                  "shared memory");  // 512: the static variables
     auto kern = dm.dense_minv ? score_bf16_kernel<true> : score_bf16_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
