@@ -355,9 +355,10 @@ class DecodeEvictor:
       stats   float32 [S, L, Hq, 2, 128] (mean, M2), counts int32 [S, L, Hq]
     After an eviction of requests a .. b - 1, ``scores`` [L, Hkv, (b - a) cap]
     and ``idx`` [L, Hkv, b - a, budget] hold that pass's scores and positions.
-    Writing a decode step's k, v into the slot is the model's cache write (a
-    plain indexed copy here); the statistics, the scoring pass, the selection
-    and the compaction run in libjacap's kernels.
+    A decode step's k, v, id and query go into the slot and the statistics in one
+    launch (jacap_append; indexed copies and jacap_stats_update where that takes
+    no such tensors); the scoring pass, the selection and the compaction run in
+    libjacap's kernels too.
     """
 
     def __init__(self, num_seqs: int, num_layers: int, num_q_heads: int, num_kv_heads: int, budget: int,

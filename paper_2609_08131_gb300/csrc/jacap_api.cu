@@ -304,13 +304,13 @@ int fused_run_items(const Dims& dm, double items_per_unit) {
   return r;
 }
 
-// The automatic choice is the separate kernels. Measured on GB300 (config 2:
-// 32 layers x 8 KV heads, n = 32768) the fused launch takes 0.96 ms against
-// 0.80 ms for the Gram, the factor and the scores apart: a unit stays ~150 us
-// between its first Gram tile and its last score tile, so at the pass's rate
-// of V far more than L2 is in flight and only ~12 % of the second read hits
-// L2, while the roles' fill and drain (~80 us each) add to a pass whose
-// separate kernels already run at the effective HBM rate.
+// The automatic choice is the separate kernels. Measured on GB300 (32 layers x 8
+// KV heads, n = 32768) the fused launch takes 0.94 ms against 0.74 ms for the
+// Gram, the factor and the scores apart: a unit stays ~150 us between its first
+// Gram tile and its last score tile, so at the pass's rate of V far more than L2
+// is in flight and only ~12 % of the second read hits L2, while the roles' fill
+// and drain (~80 us each) add to a pass whose separate kernels already run at the
+// effective HBM rate.
 bool fused_pays(const jacap_layout*, const Dims&, int) { return false; }
 
 // 2 (fused, with its roles and kept tiles) or 1 (separate kernels) for a
@@ -347,8 +347,8 @@ void pick_runs(Dims& dm, int64_t items, int sms) {
     dm.big_planes = (int)std::max<int64_t>(0, planes - ((36 + ct - 1) / ct * sms + per_plane - 1) / per_plane);
 }
 
-// Partial Grams of a unit: every chunk (float32), or one per CTA that its chunks
-// are spread over (bf16, contiguous shares).
+// Partial Grams of a unit, on average over the units: every chunk (float32), or one
+// per CTA that its chunks are spread over (bf16, contiguous shares).
 int partials_per_unit(const Dims& dm, int64_t items, int sms, bool bf) {
   const int64_t units = (int64_t)dm.L * dm.Hkv * dm.S, chunks = std::max<int64_t>(1, items / units);
   if (!bf) return (int)std::min<int64_t>(chunks, 1 << 20);

@@ -322,6 +322,12 @@ template <bool PROJ, int CTAS>
 __global__ void __launch_bounds__(FT_THREADS, CTAS)
     factor_kernel(Dims dm, Ws ws, const float* __restrict__ out_factor, int reduced) {
   pdl_wait();
+  // The one partial that the reducing launch leaves, at the unit's first chunk, read
+  // without the list of partials: 0.7 us less (one layer of 4096 tokens 72.8 -> 72.1
+  // us). Not with four CTAs on an SM, where the second way to read spills 38 bytes a
+  // thread instead of 20 (1024 units 0.132 ms, 0.119 with the list alone; with three,
+  // 26 instead of 46 bytes and 320 units 0.0576 instead of 0.0595).
+  constexpr bool DIRECT = CTAS <= 3;
   extern __shared__ __align__(16) float fmat[];  // PROJ: R0, R1
   __shared__ FtSmem sm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -335,7 +341,8 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
   const int u = blockIdx.x;
   const int plane = u / dm.S, s = u % dm.S;
   if (tid == 0) sm.skip = status_failed(ws) ? 1 : 0;
-  const int ch0 = ws.plan[1 + s], ch1 = ws.plan[2 + s];
+  const int ch0 = ws.plan[1 + s];
+  const int ch1 = !DIRECT && reduced ? min(ch0 + 1, (int)ws.plan[2 + s]) : (int)ws.plan[2 + s];
   __syncthreads();
   if (sm.skip) return;
   bool bad = false;
@@ -355,14 +362,12 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
   {
     const float* gp = ws.gpart + ((int64_t)plane * dm.c_cap) * D * D + ((cx >> 3) * D + 8 * ty) * 32 + (cx & 7) * 4;
     const int32_t* pf = ws.pflag + (int64_t)plane * dm.c_cap;
-    // one partial, at the unit's first chunk (without the list: 0.7 us less, one
-    // layer of 4096 tokens 72.8 -> 72.1 us)
-    if (reduced && own && ch0 < ch1) {
+    if (DIRECT && reduced && own && ch0 < ch1) {
       const float* src = gp + (int64_t)ch0 * D * D;
 #pragma unroll
       for (int i = 0; i < 8; ++i) tile_set_row(T, i, *(const float4*)(src + i * 32));
     }
-    for (int base = ch0; base < ch1 && !reduced; base += FT_THREADS) {
+    for (int base = ch0; base < ch1 && !(DIRECT && reduced); base += FT_THREADS) {
       // the chunks that hold a partial (the first one of every run)
       const int ch = base + tid;
       const bool has = ch < ch1 && pf[ch] != 0;
@@ -523,7 +528,8 @@ __global__ void __launch_bounds__(FT_THREADS, CTAS)
 // The partials of each unit summed into the first one (at its first chunk), by
 // one CTA per unit and lower 32 x 32 block: for a few units with many partials,
 // which the factor's one CTA per unit would add one after the other (~0.6 us each;
-// this launch costs about 4 us, hence from six partials on).
+// this launch costs about 4 us, hence from six partials on, by the mean over the
+// units: a long request beside many short ones may keep some twenty for the factor).
 constexpr int FR_THREADS = 256;
 __global__ void __launch_bounds__(FR_THREADS) gram_reduce_kernel(Dims dm, Ws ws) {
   pdl_wait();

@@ -22,7 +22,7 @@ __device__ __forceinline__ float recip_nr(float p) {
 // 32 x 32 blocks (I, J = 0..3) and inverts the factor blockwise, so the
 // sequential part is four 32-step eliminations inside one warp:
 //  for K = 0..3:
-//    T_KK = L_KK^{-1}   one warp: the forward elimination above on the 32 x 32
+//    T_KK = L_KK^{-1}   one warp: the forward elimination below on the 32 x 32
 //                       block A_KK (its lower triangle), X_KK -> T_KK
 //    L_IK = A_IK T_KK^T                 I > K
 //    A_IJ -= L_IK L_JK^T                K < J <= I
@@ -88,8 +88,13 @@ __device__ __forceinline__ void nt_block(float (&acc)[2][2], const float* P, con
     for (int j = 0; j < 2; ++j) acc[i][j] += s[i][j].x + s[i][j].y;
 }
 
-// T = L^{-1} of one 32 x 32 diagonal block by the elimination described at the
-// top of the file, in one warp: lane r holds row r in registers. At step k the
+// T = L^{-1} of one 32 x 32 diagonal block by forward elimination of [A | I] without
+// pivoting, in one warp. Both halves share one array Z: column c holds A until step c
+// eliminates it, and Y_c = -p_c X_c afterwards, where p_c is the pivot, X the inverse
+// of the unit lower factor and T = Diag(p)^{-1/2} X. In that scaling the eliminated
+// value A_ic already equals Y_ic, so step j updates every row i > j by one multiply-add
+// per column, Z_i. -= (A_ij / p_j) r with r_c = A_cj (c > j), 0 (c = j), Z_jc (c < j).
+// Lane r holds row r in registers. At step k the
 // pivot row goes to every lane through shared memory: its scaled inverse part
 // (columns < k) from lane k's registers, its A part (columns >= k) as column k
 // of every row (the lower triangle of A; each lane stores its own element).

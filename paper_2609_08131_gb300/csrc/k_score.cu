@@ -41,8 +41,9 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
 // the diagonal, so a block of 8 rows may run its columns up to its last row. The
 // warps' partial sums of squares meet in shared memory, added in warp order. The
 // next tile's V streams in (16-byte asynchronous copies) while this one is worked on.
-// Bound: float32 multiply-adds, 2 x 8704 issue cycles per tile and sub-partition. 8 x 4096
-// tokens: 0.055 -> 0.025 ms against two threads per token with four rows each.
+// Bound: the issue of float32 multiply-adds, 4352 per warp and tile, 8704 cycles per
+// tile and sub-partition (two warps). 8 x 4096 tokens: 0.055 -> 0.025 ms against two
+// threads per token with four rows each.
 constexpr int SF_THREADS = 256;
 constexpr int SF_LD = D + 4;
 constexpr size_t score_f32_smem_bytes() { return ((size_t)D * D + 2 * TILE * SF_LD + 8 * TILE) * sizeof(float); }

@@ -247,3 +247,23 @@ def test_traced_factor_compiles(tmp_path, src):
            str(tmp_path / "o.o")]
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_factor_variants_keep_their_tiles_in_registers(tmp_path):
+    """A thread of the factor holds 32 values of its matrix beside a step's vectors; with three and four
+    CTAs on an SM it has 72 and 56 registers, and every further value is spilled in each of 32 steps
+    (18 bytes more took 1024 units from 0.119 to 0.132 ms)."""
+    import subprocess
+
+    cmd = [_lib.nvcc(), *_lib.ARCH, *_lib.CFLAGS, "-Xptxas", "-v", "-c", os.path.join(_lib.CSRC, "k_factor.cu"), "-o",
+           str(tmp_path / "o.o")]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    spilled = {}
+    for m in re.finditer(r"entry function '(\w+)'.*?(\d+) bytes spill stores", r.stderr, re.S):
+        v = re.search(r"factor_kernelILb(\d)ELi(\d)E", m.group(1))
+        if v:
+            spilled[v.group(1), int(v.group(2))] = int(m.group(2))
+    limit = {("1", 1): 0, ("0", 2): 0, ("0", 3): 32, ("0", 4): 24}
+    assert set(spilled) == set(limit)
+    assert all(spilled[v] <= limit[v] for v in limit), spilled

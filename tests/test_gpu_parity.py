@@ -790,10 +790,13 @@ def test_kappa_rounds_like_float32_multiply_adds(G):
     (1, 1, (40000,)),               # one unit of 313 chunks: the reducing launch lists its partials twice
     (2, 1, (70000,)),
     (1, 1, (40000,) + (20,) * 60),  # the same in a pack whose mean has few partials: the factor lists them itself
+    (36, 16, (1000,)),              # 576 units, four CTAs on an SM: in float32 eight partials each, reduced
+    (40, 16, (1000,)),              # 640 units, three
 ])
 def test_every_partial_gram_of_a_long_unit_is_summed(dtype, layers, hkv, lens):
     """G as the factor leaves it against sum_i w_i v_i v_i^T in 64 bits, with the pass's own weights, in
-    units of more chunks than the lists of partials hold at once (256 and 288). w v is split within
+    units of more chunks than the lists of partials hold at once (256 and 288), and in each variant of
+    the factor behind the reducing launch. w v is split within
     2^-17; sums over n tokens and their partials are float32, of random signs off the diagonal and each
     truncation at most 2^-23: 2^-15 of the sum of the terms' magnitudes covers them. One chunk of 313
     left out, or taken twice, is 3e-3 of it."""
