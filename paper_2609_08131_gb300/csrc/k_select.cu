@@ -32,9 +32,9 @@
 // batch each time when the number of requests divided the grid.
 // Measured against three radix passes over all keys in such a grid, selection and
 // row copies: 1024 units of 731-3072 tokens (256 kept) 0.152 -> 0.055 ms, 1024 units
-// of 2K-64K tokens (512) 0.290 -> 0.158, 320 units of 9001 (900) 0.102 -> 0.080, 256
-// units of 32768 (512) 0.057 -> 0.044, of 131072 (1024) 0.154 -> 0.124, 8 units of
-// 4099 (512) 0.018 -> 0.012; 448 slots of 2052 tokens with holes filled 0.045 -> 0.020.
+// of 2K-64K tokens (512) 0.290 -> 0.155, 320 units of 9001 (900) 0.102 -> 0.079, 256
+// units of 32768 (512) 0.057 -> 0.043, of 131072 (1024) 0.154 -> 0.119, 8 units of
+// 4099 (512) 0.018 -> 0.011; 448 slots of 2052 tokens with holes filled 0.045 -> 0.020.
 // The copies' bytes alone take 0.040, 0.079, 0.044, 0.020 and 0.040 ms of the first
 // five at the copy rate.
 //
@@ -457,9 +457,9 @@ cudaError_t launch_select(const Dims& dm, const Ws& ws, const int32_t* cu, const
                                         pos, grid, parts, st)))
   // More units than SMs: CTAs of 256 threads (four per SM) while they hold the
   // longest request in one slab, of 512 (two per SM) beyond that (256 units of 32768
-  // tokens: 44 us, 51 with 1024 threads; of 131072: 124 and 132). Otherwise CTAs of
+  // tokens: 42 us, 46 with 1024 threads; of 131072: 119 and 120). Otherwise CTAs of
   // 1024 threads, as many per unit as there are SMs for (112 units of 20011 tokens,
-  // 2048 kept: 55 us; 64 with two CTAs of 512 threads each).
+  // 2048 kept: 51 us; 60 with two CTAs of 512 threads each).
   int dev = 0, sms = 0;
   JACAP_TRY(cudaGetDevice(&dev));
   JACAP_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
